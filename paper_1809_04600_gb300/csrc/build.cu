@@ -378,6 +378,28 @@ static inline unsigned grid_for(int64_t n, int threads = 256) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, threads), 152 * 32));
 }
 
+// bits a spin string can have set, per word
+template <int W>
+struct OrbMask {
+    uint64_t w[W];
+    explicit OrbMask(int n_orb) {
+        for (int k = 0; k < W; k++) {
+            const int bits = std::min(64, std::max(0, n_orb - 64 * k));
+            w[k] = bits == 64 ? ~0ull : (1ull << bits) - 1;
+        }
+    }
+};
+
+// bits in which the composite keys (major << 32 | minor) of the given ranges can differ
+static uint64_t composite_mask(int64_t n_major, int64_t n_minor) {
+    auto bits = [](int64_t count) {
+        uint64_t m = 0;
+        while ((int64_t)m < count - 1) m = 2 * m + 1;
+        return m;
+    };
+    return (bits(n_major) << 32) | bits(n_minor);
+}
+
 template <int W>
 static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf<int32_t> &sidx, int64_t &U) {
     const int64_t n = c->n_det;
@@ -386,7 +408,7 @@ static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf
     c->sort_vals.alloc((size_t)n);
     k_extract_strings<W><<<grid_for(n), 256, 0, st>>>(c->dets.p, n, spin, c->sort_keys.p, c->sort_vals.p);
     KERNEL_CHECK();
-    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st);
+    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st, OrbMask<W>(c->n_orb).w);
     c->i64a.alloc((size_t)n + 1);
     c->i64b.alloc((size_t)n + 1);
     c->i64c.alloc((size_t)scan_tmp_len(n + 1));
@@ -403,13 +425,14 @@ static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf
 }
 
 template <int W>
-static void group_by(shci_ctx *c, const int32_t *major, const int32_t *minor, int64_t n_groups, int other_spin,
-                     DevBuf<int64_t> &off, DevBuf<int32_t> &mdet, DevBuf<uint64_t> &mstr) {
+static void group_by(shci_ctx *c, const int32_t *major, const int32_t *minor, int64_t n_groups, int64_t n_minor,
+                     int other_spin, DevBuf<int64_t> &off, DevBuf<int32_t> &mdet, DevBuf<uint64_t> &mstr) {
     const int64_t n = c->n_det;
     cudaStream_t st = c->st;
     k_composite<<<grid_for(n), 256, 0, st>>>(major, minor, n, c->sort_keys.p, c->sort_vals.p);
     KERNEL_CHECK();
-    radix_sort<1>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st);
+    const uint64_t vary = composite_mask(n_groups, n_minor);
+    radix_sort<1>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st, &vary);
     off.alloc((size_t)n_groups + 1);
     mdet.alloc((size_t)n);
     mstr.alloc((size_t)n * W);
@@ -431,7 +454,8 @@ static void group_by_index(shci_ctx *c, const int32_t *major, int64_t n_groups, 
     cudaStream_t st = c->st;
     k_composite<<<grid_for(n), 256, 0, st>>>(major, nullptr, n, c->sort_keys.p, c->sort_vals.p);
     KERNEL_CHECK();
-    radix_sort<1>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st);
+    const uint64_t vary = composite_mask(n_groups, n);
+    radix_sort<1>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st, &vary);
     off.alloc((size_t)n_groups + 1);
     mdet.alloc((size_t)n);
     mstr.alloc((size_t)n * W);
@@ -464,7 +488,7 @@ static int64_t string_singles(shci_ctx *c, const uint64_t *ustr, int64_t U, int 
     c->sort_vals.alloc((size_t)std::max<int64_t>(nk, c->n_det));
     k_minus_one_keys<W><<<grid_for(U), 256, 0, st>>>(ustr, U, ne, c->sort_keys.p, c->sort_vals.p);
     KERNEL_CHECK();
-    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, nk, c->sw, st);
+    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, nk, c->sw, st, OrbMask<W>(c->n_orb).w);
     DevBuf<int64_t> seg_start;
     DevBuf<int32_t> seg_len;
     seg_start.alloc((size_t)nk);
@@ -588,8 +612,8 @@ static void lists_w(shci_ctx *c) {
 
     unique_strings<W>(c, 0, c->astr, c->ia, c->Ua);
     unique_strings<W>(c, 1, c->bstr, c->ib, c->Ub);
-    group_by<W>(c, c->ia.p, c->ib.p, c->Ua, 1, c->ga_off, c->ga_det, c->ga_str);
-    group_by<W>(c, c->ib.p, c->ia.p, c->Ub, 0, c->gb_off, c->gb_det, c->gb_str);
+    group_by<W>(c, c->ia.p, c->ib.p, c->Ua, c->Ub, 1, c->ga_off, c->ga_det, c->ga_str);
+    group_by<W>(c, c->ib.p, c->ia.p, c->Ub, c->Ua, 0, c->gb_off, c->gb_det, c->gb_str);
     CUDA_TRY(cudaMemcpyAsync(&flags, c->counter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
     if (flags & 8) throw ShciError{SHCI_ERR_INVALID, "duplicate determinants in V"};

@@ -69,7 +69,9 @@ __global__ void k_scan_blocksums(T *block_sums, int64_t nb) {
     if (threadIdx.x == 0) block_sums[nb] = carry;
 }
 
-template <typename T>
+// OWN_PREFIX: block_sums holds plain sums and each block adds up those before
+// its own (few blocks); otherwise they are already scanned.
+template <typename T, bool OWN_PREFIX>
 __global__ void k_scan_apply(const T *__restrict__ in, int64_t n, const T *__restrict__ block_sums,
                              T *__restrict__ out) {
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
@@ -80,15 +82,28 @@ __global__ void k_scan_apply(const T *__restrict__ in, int64_t n, const T *__res
         v[k] = base + k < n ? in[base + k] : T(0);
         s += v[k];
     }
+    T before;
+    if (OWN_PREFIX) {
+        T part = 0;
+        for (unsigned b = threadIdx.x; b < blockIdx.x; b += SCAN_THREADS) part += block_sums[b];
+        block_excl_scan<T>(part, &before);
+    } else {
+        before = block_sums[blockIdx.x];
+    }
     T tot;
-    T ex = block_excl_scan<T>(s, &tot) + block_sums[blockIdx.x];
+    T ex = block_excl_scan<T>(s, &tot) + before;
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         if (base + k < n) out[base + k] = ex;
         ex += v[k];
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) out[n] = block_sums[gridDim.x];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) out[n] = before + tot;
 }
+
+// Up to this many blocks every block sums the totals before it itself (at most
+// two loads per thread) instead of a launch of its own doing so: the short
+// scans of the helper lists are bound by their launches.
+constexpr int64_t SCAN_OWN_PREFIX = 2 * SCAN_THREADS;
 
 // out[0..n] = exclusive scan of in[0..n), out[n] = total.  `tmp` needs
 // ceil(n / SCAN_TILE) + 1 elements.  in and out may alias.
@@ -99,24 +114,43 @@ inline void exclusive_scan(const T *in, T *out, int64_t n, T *tmp, cudaStream_t 
         return;
     }
     int64_t nb = ceil_div(n, SCAN_TILE);
-    k_scan_reduce<T><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(in, n, tmp);
-    k_scan_blocksums<T><<<1, 1024, 0, st>>>(tmp, nb);
-    k_scan_apply<T><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(in, n, tmp, out);
+    if (nb > 1) {
+        k_scan_reduce<T><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(in, n, tmp);
+        g_kernel_launches += 1;
+    }
+    if (nb <= SCAN_OWN_PREFIX) {
+        k_scan_apply<T, true><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(in, n, tmp, out);
+    } else {
+        k_scan_blocksums<T><<<1, 1024, 0, st>>>(tmp, nb);
+        k_scan_apply<T, false><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(in, n, tmp, out);
+        g_kernel_launches += 1;
+    }
     KERNEL_CHECK();
-    g_kernel_launches += 3;
+    g_kernel_launches += 1;
 }
 
 inline int64_t scan_tmp_len(int64_t n) { return ceil_div(n, SCAN_TILE) + 1; }
 
 // ---------------------------------------------------------------- radix sort
 
-constexpr int RS_THREADS = 256;
+constexpr int RS_THREADS = 256;                    // one thread per digit value in the tile-wide steps
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ROUNDS = 8;                       // 32-element rounds per warp
-constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;    // 2048 elements per tile
 
+// 32-element rounds per warp: a tile's keys and payloads are reordered in
+// shared memory before they are written, so that a digit's elements leave as
+// one run; the tile is the largest that keeps the block below 48 KB (five
+// blocks per SM for one-word keys).
 template <int KW>
-__global__ void k_key_or_and(const uint64_t *__restrict__ keys, int64_t n, unsigned long long *orand) {
+struct RsTile {
+    static constexpr int ROUNDS = KW == 1 ? 12 : (KW == 2 ? 7 : 4);
+    static constexpr int N = RS_THREADS * ROUNDS;
+};
+
+// OR and AND of every key word: one atomic per block and word (an atomic per
+// thread took 275 us of a 1e6-key sort's 390, all of it serialised on one L2 line).
+template <int KW>
+__global__ void __launch_bounds__(RS_THREADS) k_key_or_and(const uint64_t *__restrict__ keys, int64_t n,
+                                                          unsigned long long *orand) {
     unsigned long long o[KW], a[KW];
 #pragma unroll
     for (int w = 0; w < KW; w++) { o[w] = 0; a[w] = ~0ull; }
@@ -124,76 +158,125 @@ __global__ void k_key_or_and(const uint64_t *__restrict__ keys, int64_t n, unsig
 #pragma unroll
         for (int w = 0; w < KW; w++) { uint64_t k = keys[i * KW + w]; o[w] |= k; a[w] &= k; }
     }
+    __shared__ unsigned long long so[RS_WARPS][KW], sa[RS_WARPS][KW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int w = 0; w < KW; w++) {
-        atomicOr(&orand[w], o[w]);
-        atomicAnd(&orand[KW + w], a[w]);
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+            o[w] |= __shfl_xor_sync(0xffffffffu, o[w], d);
+            a[w] &= __shfl_xor_sync(0xffffffffu, a[w], d);
+        }
+        if (lane == 0) { so[wid][w] = o[w]; sa[wid][w] = a[w]; }
+    }
+    __syncthreads();
+    if (threadIdx.x < KW) {
+        const int w = threadIdx.x;
+        for (int x = 1; x < RS_WARPS; x++) { so[0][w] |= so[x][w]; sa[0][w] &= sa[x][w]; }
+        atomicOr(&orand[w], so[0][w]);
+        atomicAnd(&orand[KW + w], sa[0][w]);
     }
 }
 
 template <int KW>
-__global__ void k_rs_hist(const uint64_t *__restrict__ keys, int64_t n, int word, int shift,
-                          uint32_t *__restrict__ hist, int64_t n_tiles) {
+__global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint64_t *__restrict__ keys, int64_t n, int word,
+                                                       int shift, uint32_t *__restrict__ hist, int64_t n_tiles) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int k = threadIdx.x; k < RS_TILE; k += RS_THREADS) {
-        int64_t i = base + k;
+    const int64_t base = (int64_t)blockIdx.x * RsTile<KW>::N;
+#pragma unroll
+    for (int r = 0; r < RsTile<KW>::ROUNDS; r++) {
+        const int64_t i = base + r * RS_THREADS + threadIdx.x;
         if (i < n) atomicAdd(&h[(keys[i * KW + word] >> shift) & 255u], 1u);
     }
     __syncthreads();
     hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
 }
 
+// One digit's stable scatter of a tile: ranks by warp-wide matching, the tile
+// reordered by digit in shared memory, then written in that order (a warp
+// writes runs of one digit's consecutive slots).  Bound by HBM: read and write
+// of the elements.  vin == nullptr: an element's payload is its position;
+// vout == nullptr: keys alone.
 template <int KW>
-__global__ void k_rs_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-                             uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n,
-                             int word, int shift, const uint32_t *__restrict__ offs, int64_t n_tiles) {
+__global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t *__restrict__ kin,
+                                                          const uint32_t *__restrict__ vin,
+                                                          uint64_t *__restrict__ kout, uint32_t *__restrict__ vout,
+                                                          int64_t n, int word, int shift,
+                                                          const uint32_t *__restrict__ offs, int64_t n_tiles) {
+    constexpr int ROUNDS = RsTile<KW>::ROUNDS, TILE = RsTile<KW>::N;
     __shared__ uint32_t wcnt[RS_WARPS][256];
+    __shared__ uint32_t gbase[256];                 // a digit's first global slot minus its first slot in the tile
+    __shared__ uint64_t skey[TILE * KW];
+    __shared__ uint32_t sval[TILE];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int d = lane; d < 256; d += 32) wcnt[w][d] = 0;
     __syncwarp();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE + (int64_t)w * (32 * RS_ROUNDS);
-    uint32_t rank[RS_ROUNDS];
-    int dig[RS_ROUNDS];
-    const unsigned lt = (1u << lane) - 1u;
+    const int64_t tile0 = (int64_t)blockIdx.x * TILE;
+    const int64_t base = tile0 + (int64_t)w * (32 * ROUNDS);
+    uint64_t key[ROUNDS][KW];
+    uint32_t val[ROUNDS], rank[ROUNDS];
 #pragma unroll
-    for (int r = 0; r < RS_ROUNDS; r++) {
-        int64_t i = base + r * 32 + lane;
-        bool valid = i < n;
-        int d = valid ? (int)((kin[i * KW + word] >> shift) & 255u) : 256 + lane;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        uint32_t before = valid ? wcnt[w][d] : 0u;
+    for (int r = 0; r < ROUNDS; r++) {
+        const int64_t i = base + r * 32 + lane;
+#pragma unroll
+        for (int q = 0; q < KW; q++) key[r][q] = i < n ? kin[i * KW + q] : 0ull;
+        val[r] = (i < n && vin) ? vin[i] : (uint32_t)i;
+    }
+    const unsigned lt = (1u << lane) - 1u;
+    auto digit = [&](const uint64_t *k) {
+        uint64_t x = k[0];
+#pragma unroll
+        for (int q = 1; q < KW; q++) x = word == q ? k[q] : x;
+        return (int)((x >> shift) & 255u);
+    };
+#pragma unroll
+    for (int r = 0; r < ROUNDS; r++) {
+        const bool valid = base + r * 32 + lane < n;
+        const int d = valid ? digit(key[r]) : 256 + lane;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = valid ? wcnt[w][d] : 0u;
         __syncwarp();
         if (valid && (peers & lt) == 0) wcnt[w][d] = before + __popc(peers);
         __syncwarp();
         rank[r] = before + __popc(peers & lt);
-        dig[r] = d;
     }
     __syncthreads();
-    // exclusive scan across warps of each digit's count
+    // per digit: exclusive prefix over the warps; then over the digits
     {
-        int d = threadIdx.x;   // RS_THREADS == 256 digits
+        const int d = threadIdx.x;
         uint32_t run = 0;
 #pragma unroll
         for (int x = 0; x < RS_WARPS; x++) {
-            uint32_t t = wcnt[x][d];
+            const uint32_t t = wcnt[x][d];
             wcnt[x][d] = run;
             run += t;
         }
+        uint32_t total;
+        const uint32_t start = block_excl_scan<uint32_t>(run, &total);
+        gbase[d] = offs[(int64_t)d * n_tiles + blockIdx.x] - start;
+#pragma unroll
+        for (int x = 0; x < RS_WARPS; x++) wcnt[x][d] += start;
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < RS_ROUNDS; r++) {
-        int64_t i = base + r * 32 + lane;
-        if (i < n) {
-            int d = dig[r];
-            int64_t pos = (int64_t)offs[(int64_t)d * n_tiles + blockIdx.x] + wcnt[w][d] + rank[r];
+    for (int r = 0; r < ROUNDS; r++) {
+        if (base + r * 32 + lane < n) {
+            const uint32_t pos = wcnt[w][digit(key[r])] + rank[r];
 #pragma unroll
-            for (int q = 0; q < KW; q++) kout[pos * KW + q] = kin[i * KW + q];
-            vout[pos] = vin[i];
+            for (int q = 0; q < KW; q++) skey[pos * KW + q] = key[r][q];
+            if (vout) sval[pos] = val[r];
         }
+    }
+    __syncthreads();
+    const int cnt = (int)min((int64_t)TILE, n - tile0);
+    for (int e = threadIdx.x; e < cnt; e += RS_THREADS) {
+        const uint64_t *k = skey + (int64_t)e * KW;
+        const uint32_t pos = gbase[digit(k)] + (uint32_t)e;
+#pragma unroll
+        for (int q = 0; q < KW; q++) kout[(int64_t)pos * KW + q] = k[q];
+        if (vout) vout[pos] = sval[e];
     }
 }
 
@@ -206,51 +289,74 @@ struct SortWork {
     DevBuf<unsigned long long> orand;
 };
 
+__global__ static void k_rs_iota(uint32_t *__restrict__ v, int64_t n) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+        v[e] = (uint32_t)e;
+}
+
+// What the sort does with vals: carries them, sets them to each key's original
+// position (the first pass writes them, nothing is read), or has none (vals unused).
+enum { RS_VALS = 0, RS_POSITION = 1, RS_KEYS = 2 };
+
 // Stable sort of (keys[n][KW], vals[n]) in place (ping-pong through ws).
 // Word 0 is the least significant.  Digits that are equal for every key are
-// skipped (found by an OR/AND reduction), so short keys cost few passes.
+// skipped: those outside `may_vary` (per key word, where the caller knows the
+// bits its keys can differ in), or those found by an OR/AND reduction over the
+// keys and a read-back (may_vary == nullptr).
 template <int KW>
-inline void radix_sort(uint64_t *keys, uint32_t *vals, int64_t n, SortWork &ws, cudaStream_t st) {
-    if (n <= 1) return;
+inline void radix_sort(uint64_t *keys, uint32_t *vals, int64_t n, SortWork &ws, cudaStream_t st,
+                       const uint64_t *may_vary = nullptr, int payload = RS_VALS) {
+    if (n <= 1) {
+        if (payload == RS_POSITION && n == 1) CUDA_TRY(cudaMemsetAsync(vals, 0, sizeof(uint32_t), st));
+        return;
+    }
     if (n > 0xFFFFFFFFll) throw ShciError{SHCI_ERR_INVALID, "radix_sort: too many elements"};
-    int64_t n_tiles = ceil_div(n, RS_TILE);
+    int64_t n_tiles = ceil_div(n, RsTile<KW>::N);
     ws.keys_alt.alloc((size_t)n * KW);
-    ws.vals_alt.alloc((size_t)n);
+    if (payload != RS_KEYS) ws.vals_alt.alloc((size_t)n);
     ws.hist.alloc((size_t)(256 * n_tiles + 1));
     ws.scan_tmp.alloc((size_t)scan_tmp_len(256 * n_tiles));
-    ws.orand.alloc(2 * KW);
-    std::vector<unsigned long long> init(2 * KW);
-    for (int w = 0; w < KW; w++) { init[w] = 0ull; init[KW + w] = ~0ull; }
-    CUDA_TRY(cudaMemcpyAsync(ws.orand.p, init.data(), sizeof(unsigned long long) * 2 * KW,
-                             cudaMemcpyHostToDevice, st));
-    k_key_or_and<KW><<<(unsigned)std::min<int64_t>(ceil_div(n, 256), 1024), 256, 0, st>>>(keys, n, ws.orand.p);
-    KERNEL_CHECK();
-    g_kernel_launches += 1;
-    std::vector<unsigned long long> oa(2 * KW);
-    CUDA_TRY(cudaMemcpyAsync(oa.data(), ws.orand.p, sizeof(unsigned long long) * 2 * KW,
-                             cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
+    uint64_t varying[KW];
+    if (may_vary) {
+        for (int w = 0; w < KW; w++) varying[w] = may_vary[w];
+    } else {
+        ws.orand.alloc(2 * KW);
+        CUDA_TRY(cudaMemsetAsync(ws.orand.p, 0, sizeof(unsigned long long) * KW, st));
+        CUDA_TRY(cudaMemsetAsync(ws.orand.p + KW, 0xFF, sizeof(unsigned long long) * KW, st));
+        k_key_or_and<KW><<<(unsigned)std::min<int64_t>(ceil_div(n, RS_THREADS), 1024), RS_THREADS, 0, st>>>(keys, n,
+                                                                                                          ws.orand.p);
+        KERNEL_CHECK();
+        g_kernel_launches += 1;
+        unsigned long long oa[2 * KW];
+        CUDA_TRY(cudaMemcpyAsync(oa, ws.orand.p, sizeof(oa), cudaMemcpyDeviceToHost, st));
+        CUDA_TRY(cudaStreamSynchronize(st));
+        for (int w = 0; w < KW; w++) varying[w] = oa[w] ^ oa[KW + w];
+    }
     uint64_t *ka = keys, *kb = ws.keys_alt.p;
-    uint32_t *va = vals, *vb = ws.vals_alt.p;
-    int passes = 0;
+    uint32_t *va = payload == RS_KEYS ? nullptr : vals, *vb = payload == RS_KEYS ? nullptr : ws.vals_alt.p;
+    bool first = true;
     for (int w = 0; w < KW; w++) {
-        uint64_t varying = oa[w] ^ oa[KW + w];
         for (int shift = 0; shift < 64; shift += 8) {
-            if (((varying >> shift) & 255u) == 0) continue;
+            if (((varying[w] >> shift) & 255u) == 0) continue;
             k_rs_hist<KW><<<(unsigned)n_tiles, RS_THREADS, 0, st>>>(ka, n, w, shift, ws.hist.p, n_tiles);
             exclusive_scan<uint32_t>(ws.hist.p, ws.hist.p, 256 * n_tiles, ws.scan_tmp.p, st);
-            k_rs_scatter<KW><<<(unsigned)n_tiles, RS_THREADS, 0, st>>>(ka, va, kb, vb, n, w, shift, ws.hist.p,
-                                                                       n_tiles);
+            k_rs_scatter<KW><<<(unsigned)n_tiles, RS_THREADS, 0, st>>>(
+                ka, first && payload == RS_POSITION ? nullptr : va, kb, vb, n, w, shift, ws.hist.p, n_tiles);
             KERNEL_CHECK();
             g_kernel_launches += 2;
+            first = false;
             std::swap(ka, kb);
             std::swap(va, vb);
-            passes++;
         }
+    }
+    if (first && payload == RS_POSITION) {           // nothing to sort by
+        k_rs_iota<<<(unsigned)std::min<int64_t>(ceil_div(n, RS_THREADS), 1024), RS_THREADS, 0, st>>>(vals, n);
+        KERNEL_CHECK();
+        g_kernel_launches += 1;
     }
     if (ka != keys) {
         CUDA_TRY(cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n * KW, cudaMemcpyDeviceToDevice, st));
-        CUDA_TRY(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st));
+        if (va) CUDA_TRY(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st));
     }
 }
 
