@@ -257,36 +257,35 @@ __device__ __forceinline__ double hij_offdiag(const DevInts &I, const Str<W> &ai
     return flip_sign(v, neg);
 }
 
+// f(o) for every set bit o of s above orbital `from`, ascending
+template <int W, typename F>
+__device__ __forceinline__ void for_bits_above(const Str<W> &s, int from, F f) {
+#pragma unroll
+    for (int k = 0; k < W; k++) {
+        uint64_t m = s.w[k];
+        const int lo = from + 1 - 64 * k;                // first bit of word k that counts
+        if (lo >= 64) continue;
+        if (lo > 0) m &= ~0ull << lo;
+        while (m) {
+            f(64 * k + __ffsll((long long)m) - 1);
+            m &= m - 1;
+        }
+    }
+}
+
 // H_ii
 template <int W>
 __device__ __forceinline__ double hii(const DevInts &I, const Str<W> &a, const Str<W> &b) {
     const int n = I.n;
     double e = I.e_core;
-    int oa[SHCI_MAX_ORB], ob[SHCI_MAX_ORB];
-    int na = 0, nb = 0;
-#pragma unroll
-    for (int k = 0; k < W; k++) {
-        uint64_t m = a.w[k];
-        while (m) { oa[na++] = 64 * k + __ffsll((long long)m) - 1; m &= m - 1; }
-        m = b.w[k];
-        while (m) { ob[nb++] = 64 * k + __ffsll((long long)m) - 1; m &= m - 1; }
-    }
-    for (int x = 0; x < na; x++) {
-        int k = oa[x];
+    for_bits_above<W>(a, -1, [&](int k) {
         e += __ldg(&I.h[k * n + k]);
-        for (int y = x + 1; y < na; y++) {
-            int l = oa[y];
-            e += __ldg(&I.jdiag[k * n + l]) - __ldg(&I.kdiag[k * n + l]);
-        }
-        for (int y = 0; y < nb; y++) e += __ldg(&I.jdiag[k * n + ob[y]]);
-    }
-    for (int x = 0; x < nb; x++) {
-        int k = ob[x];
+        for_bits_above<W>(a, k, [&](int l) { e += __ldg(&I.jdiag[k * n + l]) - __ldg(&I.kdiag[k * n + l]); });
+        for_bits_above<W>(b, -1, [&](int l) { e += __ldg(&I.jdiag[k * n + l]); });
+    });
+    for_bits_above<W>(b, -1, [&](int k) {
         e += __ldg(&I.h[k * n + k]);
-        for (int y = x + 1; y < nb; y++) {
-            int l = ob[y];
-            e += __ldg(&I.jdiag[k * n + l]) - __ldg(&I.kdiag[k * n + l]);
-        }
-    }
+        for_bits_above<W>(b, k, [&](int l) { e += __ldg(&I.jdiag[k * n + l]) - __ldg(&I.kdiag[k * n + l]); });
+    });
     return e;
 }
