@@ -233,6 +233,15 @@ int shci_davidson_history(shci_ctx *ctx, int cap, double *theta, double *rnorm, 
 int shci_select(shci_ctx *ctx, int k_roots, const double *c, double eps1, int64_t cap, uint64_t *new_dets,
                 int64_t *n_new, int mem_space);
 
+/* shci_select for callers that do not know the count: once it is known,
+ * alloc(user, count) is called on the calling thread and returns where the
+ * count rows go (mem_space; NULL: the call ends with SHCI_ERR_OOM).  It is not
+ * called when the count is 0.  One screen instead of a query and a second
+ * full call.  alloc must not call back into ctx or throw. */
+typedef uint64_t *(*shci_alloc_rows)(void *user, int64_t rows);
+int shci_select_alloc(shci_ctx *ctx, int k_roots, const double *c, double eps1, shci_alloc_rows alloc, void *user,
+                      int64_t *n_new, int mem_space);
+
 /* Screened second-order Epstein-Nesbet energy (Sec. II.B, Eq. 7):
  *   dE2 = sum_{a not in V} (sum_i^{(eps2)} H_ai c_i)^2 / (E_V - H_aa),
  * the inner sum keeping the terms with |H_ai c_i| >= eps2 (FP64), found with

@@ -40,9 +40,13 @@ EXPORTED = [
     "shci_batch_create", "shci_batch_get_modes", "shci_batch_davidson", "shci_batch_get_stats",
     "shci_batch_set_wait_limit", "shci_batch_destroy",
     "shci_davidson",
-    "shci_davidson_history", "shci_select", "shci_pt2", "shci_alias_draw", "shci_pt2_samples",
+    "shci_davidson_history", "shci_select", "shci_select_alloc", "shci_pt2", "shci_alias_draw", "shci_pt2_samples",
     "shci_pt2_semistochastic", "shci_pt2_3step", "shci_get_stats", "shci_set_timing",
 ]
+
+
+# shci_alloc_rows: (user, rows) -> address of the rows, or NULL
+ALLOC_ROWS = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64)
 
 
 class ShciError(RuntimeError):
@@ -127,6 +131,7 @@ def load_library(path: str = LIB_PATH):
         "shci_davidson": (i32, [vp, i32, f64, i32, vp, vp, vp, i32, ctypes.POINTER(i32)]),
         "shci_davidson_history": (i32, [vp, i32, vp, vp, vp, ctypes.POINTER(i32)]),
         "shci_select": (i32, [vp, i32, vp, f64, i64, vp, ctypes.POINTER(i64), i32]),
+        "shci_select_alloc": (i32, [vp, i32, vp, f64, ALLOC_ROWS, vp, ctypes.POINTER(i64), i32]),
         "shci_pt2": (i32, [vp, vp, f64, f64, i32, ctypes.POINTER(f64), ctypes.POINTER(i64), i32]),
         "shci_alias_draw": (i32, [vp, vp, i64, ctypes.c_uint64, vp, i32]),
         "shci_pt2_samples": (i32, [vp, vp, f64, f64, f64, i64, i32, vp, vp, i32, i32, vp]),
@@ -309,20 +314,40 @@ def shci_davidson_history(ctx, k_roots):
 def shci_select(ctx, c, eps1, cap=None):
     """Heat-bath selection: the new determinants [count, 2W] (uint64 numpy for a
     host c, int64 torch tensor on c's device for a device c), ascending, no
-    repeats.  c: [k, n_det] (or [n_det]) coefficients of V."""
+    repeats.  c: [k, n_det] (or [n_det]) coefficients of V.  cap: rows to try
+    with first (default: as many as there are)."""
     lib = load_library()
     pc, mc, kc = _ptr(c, np.float64)
     k = 1 if len(c.shape) == 1 else int(c.shape[0])
-    n_det = int(c.shape[-1])
     W = shci_get_stats(ctx)["n_words"]
-    cap = max(1024, 2 * n_det) if cap is None else int(cap)
     n = ctypes.c_int64(0)
-    while True:
+    held = []
+
+    def rows(count):
         if mc == SHCI_MEM_DEVICE:
             import torch
-            out = torch.empty((max(cap, 1), 2 * W), dtype=torch.int64, device=c.device)
-        else:
-            out = np.empty((max(cap, 1), 2 * W), np.uint64)
+            return torch.empty((count, 2 * W), dtype=torch.int64, device=c.device)
+        return np.empty((count, 2 * W), np.uint64)
+
+    if cap is None:
+        # the library asks for the rows once it knows how many there are
+        def alloc(_, count):
+            try:
+                held.append(rows(count))
+                return _ptr(held[0], np.uint64)[0]
+            except Exception as e:      # handed on below: it must not cross the C call
+                held.append(e)
+                return None
+
+        fn = ALLOC_ROWS(alloc)
+        rc = lib.shci_select_alloc(ctx, k, pc, float(eps1), fn, None, ctypes.byref(n), mc)
+        if held and isinstance(held[-1], Exception):
+            raise held[-1]
+        _check(ctx, rc)
+        return held[0] if held else rows(0)
+    cap = int(cap)
+    while True:
+        out = rows(max(cap, 1))
         po, mo, ko = _ptr(out, np.uint64)
         _check(ctx, lib.shci_select(ctx, k, pc, float(eps1), cap, po, ctypes.byref(n), mc))
         if n.value <= cap:

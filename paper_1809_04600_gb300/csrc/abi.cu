@@ -228,7 +228,24 @@ int shci_davidson_history(shci_ctx *c, int cap, double *theta, double *rnorm, do
 int shci_select(shci_ctx *c, int k, const double *coef, double eps1, int64_t cap, uint64_t *out, int64_t *n_out,
                 int mem) {
     return guarded(c, [&] {
-        shci::select_dets(c, k, coef, eps1, cap, out, n_out, mem);
+        if (cap < 0) throw ShciError{SHCI_ERR_INVALID, "cap must be >= 0"};
+        shci::select_dets(c, k, coef, eps1, mem, n_out, [&](int64_t rows) {
+            if (cap > 0 && !out) throw ShciError{SHCI_ERR_INVALID, "null output pointer"};
+            return std::make_pair(out, std::min(cap, rows));
+        });
+        return SHCI_OK;
+    });
+}
+
+int shci_select_alloc(shci_ctx *c, int k, const double *coef, double eps1, shci_alloc_rows alloc, void *user,
+                      int64_t *n_out, int mem) {
+    return guarded(c, [&] {
+        if (!alloc) throw ShciError{SHCI_ERR_INVALID, "null allocator"};
+        shci::select_dets(c, k, coef, eps1, mem, n_out, [&](int64_t rows) {
+            uint64_t *out = alloc(user, rows);
+            if (!out) throw ShciError{SHCI_ERR_OOM, "the caller could not allocate the selected determinants"};
+            return std::make_pair(out, rows);
+        });
         return SHCI_OK;
     });
 }

@@ -18,7 +18,7 @@ namespace shci {
 
 __global__ void k_mean_field_tables(const double *__restrict__ eri, int n, double *__restrict__ jk1,
                                     double *__restrict__ j1, double *__restrict__ jdiag,
-                                    double *__restrict__ kdiag) {
+                                    double *__restrict__ jkdiag) {
     DevInts I{};
     I.eri = eri;
     I.n = n;
@@ -34,7 +34,7 @@ __global__ void k_mean_field_tables(const double *__restrict__ eri, int n, doubl
         jk1[t] = j - x;
         if (p == q) {
             jdiag[p * n + k] = eri_get(I, p, p, k, k);
-            kdiag[p * n + k] = eri_get(I, p, k, k, p);
+            jkdiag[p * n + k] = eri_get(I, p, p, k, k) - eri_get(I, p, k, k, p);
         }
     }
 }
@@ -62,12 +62,12 @@ void load_integrals(shci_ctx *c, int n_orb, double e_core, const double *h, cons
     c->jk1.alloc((size_t)n_orb * n_orb * n_orb);
     c->j1.alloc((size_t)n_orb * n_orb * n_orb);
     c->jdiag.alloc((size_t)n_orb * n_orb);
-    c->kdiag.alloc((size_t)n_orb * n_orb);
+    c->jkdiag.alloc((size_t)n_orb * n_orb);
     CUDA_TRY(cudaMemcpyAsync(c->h.p, hh.data(), sizeof(double) * hh.size(), cudaMemcpyHostToDevice, c->st));
     CUDA_TRY(cudaMemcpyAsync(c->eri.p, eri, sizeof(double) * neri, kind, c->st));
     int64_t total = (int64_t)n_orb * n_orb * n_orb;
     k_mean_field_tables<<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 4096), 256, 0, c->st>>>(
-        c->eri.p, n_orb, c->jk1.p, c->j1.p, c->jdiag.p, c->kdiag.p);
+        c->eri.p, n_orb, c->jk1.p, c->j1.p, c->jdiag.p, c->jkdiag.p);
     KERNEL_CHECK();
     LAUNCHED(1);
     CUDA_TRY(cudaStreamSynchronize(c->st));
@@ -84,7 +84,7 @@ DevInts dev_ints(const shci_ctx *c) {
     I.jk1 = c->jk1.p;
     I.j1 = c->j1.p;
     I.jdiag = c->jdiag.p;
-    I.kdiag = c->kdiag.p;
+    I.jkdiag = c->jkdiag.p;
     I.e_core = c->e_core;
     I.n = c->n_orb;
     return I;

@@ -155,7 +155,7 @@ struct DevInts {
     const double *jk1;      // [n*n][n]: (pq|kk) - (pk|kq)   (same-spin mean field)
     const double *j1;       // [n*n][n]: (pq|kk)             (opposite-spin mean field)
     const double *jdiag;    // [n][n]:   (kk|ll)
-    const double *kdiag;    // [n][n]:   (kl|lk)
+    const double *jkdiag;   // [n][n]:   (kk|ll) - (kl|lk)
     double e_core;
     int n;
 };
@@ -280,12 +280,12 @@ __device__ __forceinline__ double hii(const DevInts &I, const Str<W> &a, const S
     double e = I.e_core;
     for_bits_above<W>(a, -1, [&](int k) {
         e += __ldg(&I.h[k * n + k]);
-        for_bits_above<W>(a, k, [&](int l) { e += __ldg(&I.jdiag[k * n + l]) - __ldg(&I.kdiag[k * n + l]); });
+        for_bits_above<W>(a, k, [&](int l) { e += __ldg(&I.jkdiag[k * n + l]); });
         for_bits_above<W>(b, -1, [&](int l) { e += __ldg(&I.jdiag[k * n + l]); });
     });
     for_bits_above<W>(b, -1, [&](int k) {
         e += __ldg(&I.h[k * n + k]);
-        for_bits_above<W>(b, k, [&](int l) { e += __ldg(&I.jdiag[k * n + l]) - __ldg(&I.kdiag[k * n + l]); });
+        for_bits_above<W>(b, k, [&](int l) { e += __ldg(&I.jkdiag[k * n + l]); });
     });
     return e;
 }

@@ -1,5 +1,7 @@
 // The library context and the internal entry points shared by the .cu files.
 #pragma once
+#include <functional>
+
 #include "common.cuh"
 #include "prims.cuh"
 
@@ -42,7 +44,7 @@ struct shci_ctx {
     bool have_ints = false;
     int n_orb = 0;
     double e_core = 0.0;
-    DevBuf<double> h, eri, jk1, j1, jdiag, kdiag;
+    DevBuf<double> h, eri, jk1, j1, jdiag, jkdiag;
     // heat-bath lists for the selection (built on first use per set of integrals)
     bool hb_valid = false;
     HBList hb_same, hb_opp;
@@ -131,8 +133,9 @@ void sigma_stored_preload();
 void noalloc_prepare(int device);
 
 // select.cu: heat-bath selection of new determinants (Sec. II)
-void select_dets(shci_ctx *c, int k, const double *coef, double eps1, int64_t cap, uint64_t *out, int64_t *n_out,
-                 int mem);
+// place(rows): where the selected rows go and how many of them are wanted
+void select_dets(shci_ctx *c, int k, const double *coef, double eps1, int mem, int64_t *n_out,
+                 const std::function<std::pair<uint64_t *, int64_t>(int64_t)> &place);
 void pt2(shci_ctx *c, const double *coef, double e_var, double eps2, int nbatch, double *e2, int64_t *n_pert,
          int mem);
 void alias_draw(shci_ctx *c, const double *coef, int64_t n_draws, uint64_t seed, int64_t *out, int mem);

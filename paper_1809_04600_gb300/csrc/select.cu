@@ -28,9 +28,12 @@ constexpr int SEL_THREADS = 256;
 // {r, s} disjoint from {p, q}, magnitude |(pr|qs) - (ps|qr)|.  List 1
 // (opposite spin, p and r alpha, q and s beta): r != p, s != q, magnitude
 // |(pr|qs)|.  Entries with magnitude 0 never meet eps1 > 0 and are dropped.
+// v is the element up to the parity of the electrons below p, q, r and s in
+// the determinant: moving p -> r and then q -> s passes those strictly between
+// each pair, i.e. the parities below the four orbitals and the order relations
+// among them, which v's sign already holds.
 __device__ __forceinline__ bool hb_entry(const DevInts &I, int same, int64_t t, int &slot, int &r, int &s,
                                          double &v) {
-    // v is signed: the element without the excitation's phase
     const int n = I.n;
     s = (int)(t % n);
     r = (int)((t / n) % n);
@@ -39,10 +42,10 @@ __device__ __forceinline__ bool hb_entry(const DevInts &I, int same, int64_t t, 
     slot = p * n + q;
     if (same) {
         if (!(p < q && r < s) || r == p || r == q || s == p || s == q) return false;
-        v = eri_get(I, p, r, q, s) - eri_get(I, p, s, q, r);
+        v = flip_sign(eri_get(I, p, r, q, s) - eri_get(I, p, s, q, r), (p < r) + (p < s) + (r < q) + (q < s));
     } else {
         if (r == p || s == q) return false;
-        v = eri_get(I, p, r, q, s);
+        v = flip_sign(eri_get(I, p, r, q, s), (p < r) + (q < s));
     }
     return fabs(v) > 0.0;
 }
@@ -266,7 +269,97 @@ struct SelArgs {
     // w (n_d - 1) / p - w^2 / p^2; second term and |H_ai c_i| per candidate
     const double *f1, *f2;
     double *terms2, *mags;
+    // single moves from per-string tables (null: evaluated in full), and each
+    // determinant's string indices
+    const double *ma, *mb;
+    const int32_t *ia, *ib;
 };
+
+// Single moves p -> r of a determinant (A, B): the element is
+//   [h_pr + sum_{k in A} ((pr|kk) - (pk|kr))] + sum_{k in B} (pr|kk)
+// (k = p contributes an exact zero to the first sum), a term of the moving
+// string and one of the other.  Both are tabulated for every string of V and
+// every orbital pair, M[u][0][pr] and M[u][1][pr], so that a move costs one
+// FP64 addition instead of one per electron: those additions held the FP64
+// pipe (74 % busy in the count pass).
+template <int W>
+__global__ void k_move_tables(const uint64_t *__restrict__ str, int64_t U, DevInts I, double *__restrict__ M) {
+    const int n = I.n, np = n * (n + 1) / 2;
+    const int64_t total = U * np;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t u = t / np;
+        const int pr = (int)(t - u * np);
+        int p = (int)((sqrtf(8.0f * (float)pr + 1.0f) - 1.0f) * 0.5f);
+        while (p * (p + 1) / 2 > pr) p--;
+        while ((p + 1) * (p + 2) / 2 <= pr) p++;
+        const int r = pr - p * (p + 1) / 2;
+        const double *jk = I.jk1 + (int64_t)(p * n + r) * n, *j1 = I.j1 + (int64_t)(p * n + r) * n;
+        double same = __ldg(&I.h[p * n + r]), opp = 0.0;
+        for_bits_above<W>(load_str<W>(str, u), -1, [&](int k) {
+            same += __ldg(&jk[k]);
+            opp += __ldg(&j1[k]);
+        });
+        M[2 * u * np + pr] = same;
+        M[(2 * u + 1) * np + pr] = opp;
+    }
+}
+
+// The tables of both spins' strings, owned by one call.
+struct MoveTables {
+    DevBuf<double> a, b;
+};
+
+// Tabulate when that is less work than evaluating the moves of `rows`
+// determinants (table entries against moves, both a sum over the electrons;
+// a quarter, since the tables are written and read back) and takes at most a
+// sixteenth of the free memory; otherwise S keeps evaluating each move.
+template <int W>
+static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double rows, MoveTables &T) {
+    const int n = c->n_orb;
+    const int64_t np = (int64_t)n * (n + 1) / 2;
+    const double entries = (double)(c->Ua + c->Ub) * np;
+    const double moves = rows * ((double)S.na * (n - S.na) + (double)S.nb * (n - S.nb));
+    if (entries > 0.25 * moves) return;
+    size_t fr = 0, tot = 0;
+    CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+    if (entries * 16.0 > (double)fr / 16.0) return;
+    T.a.alloc((size_t)(2 * c->Ua * np));
+    T.b.alloc((size_t)(2 * c->Ub * np));
+    auto grid = [&](int64_t m) { return (unsigned)std::min<int64_t>(ceil_div(m, SEL_THREADS), (int64_t)c->n_sm * 32); };
+    k_move_tables<W><<<grid(c->Ua * np), SEL_THREADS, 0, c->st>>>(c->astr.p, c->Ua, I, T.a.p);
+    k_move_tables<W><<<grid(c->Ub * np), SEL_THREADS, 0, c->st>>>(c->bstr.p, c->Ub, I, T.b.p);
+    KERNEL_CHECK();
+    g_kernel_launches += 2;
+    S.ma = T.a.p;
+    S.mb = T.b.p;
+    S.ia = c->ia.p;
+    S.ib = c->ib.p;
+}
+
+// The test |v| cmax >= eps without FP64 arithmetic where the answer is not
+// close: against eps / cmax in FP32, widened by 2^-16 on both sides (three
+// FP32 roundings), comparing the high words of |v|; FP64 decides in between,
+// for infinities and NaN, and everywhere when the ratio leaves FP32's range.
+struct Cut {
+    double cmax, eps;
+    float reach;                            // list keys below this are out of reach (0: none is)
+    uint32_t no, yes;                       // high words: below `no` fails, above `yes` passes
+};
+
+__device__ __forceinline__ Cut make_cut(double eps, double cmax) {
+    Cut t{cmax, eps, 0.0f, 0u, 0x7FF00000u};
+    const float e = (float)eps, m = (float)cmax, x = e / m;
+    if (e > 1e-30f && e < 1e30f && m > 1e-30f && m < 1e30f && x > 1e-30f && x < 1e30f) {
+        t.reach = x * (1.0f - 0x1p-16f);
+        auto high = [](float f) {                         // high word of (double)f, f positive and normal
+            const uint32_t b = __float_as_uint(f);
+            return (((b >> 23) + 896u) << 20) | ((b >> 3) & 0xFFFFFu);
+        };
+        t.no = high(t.reach);
+        t.yes = high(x * (1.0f + 0x1p-16f));
+    }
+    return t;
+}
 
 static SelArgs sel_args(const shci_ctx *c, double eps) {
     SelArgs S{};
@@ -308,20 +401,67 @@ __device__ __forceinline__ bool has_bit(const Str<W> &s, int b) {
     return (s.w[b >> 6] >> (b & 63)) & 1ull;
 }
 
-// Above this bound no later entry of a list can meet the threshold: a key is
-// the magnitude rounded toward zero to FP32, so the magnitude is below
-// key (1 + 2^-23) for normal keys and below FLT_MIN otherwise.
-__device__ __forceinline__ double key_bound(float kf) {
-    return kf < FLT_MIN ? (double)FLT_MIN : (double)kf * (1.0 + 0x1p-22);
+// The exact comparison, out of line: as part of `passes` the compiler would
+// turn the branch into predicated FP64 instructions that every element issues.
+static __device__ __noinline__ bool passes_exactly(double v, double cmax, double eps) { return fabs(v) * cmax >= eps; }
+
+__device__ __forceinline__ bool passes(const Cut &t, double v) {
+    const uint32_t h = (uint32_t)__double2hiint(v) & 0x7FFFFFFFu;
+    if (h < t.no) return false;
+    if (h > t.yes && h < 0x7FF00000u) return true;
+    return passes_exactly(v, t.cmax, t.eps);
 }
 
-// Occupied and empty orbitals of both strings, ascending, listed by a warp.
-struct OrbLists {
+// A determinant as the bits of its key: spin orbital o (alpha), beta(n) + o.
+template <int W, int KW>
+__device__ __forceinline__ int beta_bit(int n) { return KW == 1 ? n : 64 * W; }
+
+template <int KW>
+__device__ __forceinline__ void set_bit(Key<KW> &k, int x) {
+    if constexpr (KW == 1) {
+        k.w[0] |= 1ull << x;
+    } else {
+#pragma unroll
+        for (int w = 0; w < KW; w++)
+            if (w == (x >> 6)) k.w[w] |= 1ull << (x & 63);
+    }
+}
+
+// bit x: the parity of the set bits below x within x's spin string (up to a
+// constant per string, which the two orbitals of every move cancel)
+template <int W, int KW>
+__device__ __forceinline__ Key<KW> parity_below(const Key<KW> &d) {
+    Key<KW> o;
+#pragma unroll
+    for (int w = 0; w < KW; w++) {
+        uint64_t y = d.w[w] << 1;
+#pragma unroll
+        for (int s = 1; s < 64; s <<= 1) y ^= y << s;
+        if (KW > 1 && (w % W) != 0 && (__popcll(d.w[w - 1]) & 1)) y = ~y;     // W <= 2: one lower word
+        o.w[w] = y;
+    }
+    return o;
+}
+
+// parity of the number of bits set in both
+template <int KW>
+__device__ __forceinline__ int common_parity(const Key<KW> &a, const Key<KW> &b) {
+    uint64_t x = 0;
+#pragma unroll
+    for (int w = 0; w < KW; w++) x ^= a.w[w] & b.w[w];
+    return __popcll(x) & 1;
+}
+
+// Occupied and empty orbitals of both strings, ascending, and the double
+// excitation lists in reach, of a warp's determinant.
+struct SelWork {
     uint8_t occ[2][SHCI_MAX_ORB], vir[2][SHCI_MAX_ORB];
+    int first[32];                          // index of a list's first entry minus those before it in the sequence
+    int holes[32];                          // its pair: p | q << 8 (key bits), 0x10000 for an opposite-spin pair, beta 0x20000
 };
 
 template <int W>
-__device__ __forceinline__ void list_orbitals(OrbLists &L, int spin, const Str<W> &s, int n) {
+__device__ __forceinline__ void list_orbitals(SelWork &L, int spin, const Str<W> &s, int n) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     int no = 0, nv = 0;
@@ -336,58 +476,79 @@ __device__ __forceinline__ void list_orbitals(OrbLists &L, int spin, const Str<W
     }
 }
 
+// What k_select is run for: the selection, or the terms of the second-order
+// energy and which of their values a fill pass writes.
+enum { SEL_DETS = 0, SEL_TERMS = 1, SEL_SAMPLE = 2, SEL_MAGS = 3 };
+
 // One warp per determinant.  First every single move (alpha then beta), a lane
 // per move.  Then the double excitations: for 32 occupied pairs at a time a
 // lane finds by bisection how many leading entries of its pair's sorted list
 // can meet the threshold, and the warp takes those entries of all 32 lists as
-// one sequence, 32 at a time (a lane finds its list in the prefix sums), so
-// that no lane waits for another's longer list and candidates leave as one
-// contiguous, ordered run.  Walking one list per lane and reserving slots one
-// by one took 17.7 ms (count) and 24.2 ms (fill) for the 1.8e8 terms of 200,003
-// determinants of 24 orbitals (eps 1e-5); this form 5.5 and 7.8.
-template <int W, int KW, bool FILL, bool PT>
+// one sequence, 32 at a time (the starts of the lists among the 32, as bits,
+// tell a lane its list), so that no lane waits for another's longer list and
+// candidates leave as one contiguous, ordered run.  A candidate is the
+// determinant's key with the holes' and particles' bits flipped, its sign the
+// parity of those bits in the prefix-parity word.
+// Walking one list per lane and reserving slots one by one took 17.7 ms
+// (count) and 24.2 ms (fill) for the 1.8e8 terms of 200,003 determinants of 24
+// orbitals (eps 1e-5); balanced, 5.5 and 7.8 with the FP64 pipe 75 % busy on
+// thresholds and single moves; with those taken off it (Cut, k_move_tables)
+// and bits instead of strings 2.6 and 3.4: bound by issue.
+template <int W, int KW, bool FILL, int FOR>
 __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
-    __shared__ OrbLists lists[SEL_THREADS / 32];
+    __shared__ SelWork work[SEL_THREADS / 32];
     const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    OrbLists &L = lists[threadIdx.x >> 5];
+    const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
+    SelWork &L = work[threadIdx.x >> 5];
     const int n = S.n, na = S.na, nb = S.nb;
     const int u_sa = na * (n - na), u_sb = nb * (n - nb);
     const int u_paa = na * (na - 1) / 2, u_pbb = nb * (nb - 1) / 2, u_pab = na * nb;
     const int pairs = u_paa + u_pbb + u_pab;
+    const int beta = beta_bit<W, KW>(n);
     const int64_t warps = (int64_t)gridDim.x * (SEL_THREADS / 32);
     for (int64_t i = ((int64_t)blockIdx.x * SEL_THREADS + threadIdx.x) >> 5; i < S.n_det; i += warps) {
         double cmax = 0.0, ci = 0.0, f1 = 0.0, f2 = 0.0;
-        if (PT) {
+        if (FOR != SEL_DETS) {
             ci = __ldg(&S.c[i]);
             cmax = fabs(ci);
-            if (FILL && S.f1) {
-                f1 = __ldg(&S.f1[i]);
-                f2 = __ldg(&S.f2[i]);
-            }
         } else {
             for (int l = 0; l < S.k; l++) cmax = fmax(cmax, fabs(__ldg(&S.c[(int64_t)l * S.n_det + i])));
         }
+        if (FILL && FOR == SEL_SAMPLE) {
+            f1 = __ldg(&S.f1[i]) * ci;
+            f2 = __ldg(&S.f2[i]) * ci * ci;
+        }
         int64_t pos = FILL ? __ldg(&S.off[i]) : 0;        // next slot, or candidates so far
         if (cmax > 0.0) {
+            const Cut cut = make_cut(S.eps1, cmax);
             const Str<W> A = load_str<W>(S.dets, 2 * i), B = load_str<W>(S.dets, 2 * i + 1);
-            // Record this round's candidates (a, b) with the elements hv.  Second-order
-            // mode (PT): only determinants of the current hash batch, with their terms.
-            auto emit = [&](bool keep, const Str<W> &a, const Str<W> &b, double hv) {
-                if (PT && S.nbatch > 1) keep = keep && det_batch<W>(a, b, S.nbatch) == S.batch;
+            const Key<KW> D = make_key<W, KW>(A, B, n);
+            const Key<KW> PD = parity_below<W, KW>(D);
+            // Record this round's candidates: the determinant with the bits of m flipped,
+            // and v, its element up to the parity of m's bits.  Terms (FOR != SEL_DETS):
+            // only determinants of the current hash batch.
+            auto emit = [&](bool keep, const Key<KW> &m, double v) {
+                Key<KW> x;
+#pragma unroll
+                for (int w = 0; w < KW; w++) x.w[w] = D.w[w] ^ m.w[w];
+                if (FOR != SEL_DETS && S.nbatch > 1 && keep) {
+                    Str<W> a, b;
+                    split_key<W, KW>(x, n, a, b);
+                    keep = det_batch<W>(a, b, S.nbatch) == S.batch;
+                }
                 const unsigned mask = __ballot_sync(0xffffffffu, keep);
                 if (FILL && keep) {
                     const int64_t slot = pos + __popc(mask & lt);
-                    store_key<KW>(S.out, slot, make_key<W, KW>(a, b, n));
-                    if (PT) {
-                        if (S.f1) {
-                            S.terms[slot] = f1 * ci * hv;
-                            S.terms2[slot] = f2 * ci * ci * hv * hv;
-                            S.mags[slot] = fabs(hv) * cmax;
+                    store_key<KW>(S.out, slot, x);
+                    if (FOR != SEL_DETS) {
+                        const double hv = flip_sign(v, common_parity<KW>(PD, m));
+                        if (FOR == SEL_SAMPLE) {
+                            S.terms[slot] = f1 * hv;
+                            S.terms2[slot] = f2 * hv * hv;
                         } else {
                             S.terms[slot] = hv * ci;
-                            if (S.mags) S.mags[slot] = fabs(hv) * cmax;
                         }
+                        if (FOR != SEL_TERMS) S.mags[slot] = fabs(hv) * cmax;
                     }
                 }
                 pos += __popc(mask);
@@ -398,29 +559,48 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
             __syncwarp();
             for (int spin = 0; spin < 2; spin++) {
                 const int units = spin ? u_sb : u_sa, nv = n - (spin ? nb : na);
-                const Str<W> &si = spin ? B : A;
+                const int np = n * (n + 1) / 2;
+                const double *own = nullptr, *other = nullptr;
+                if (S.ma) {
+                    const int64_t ua = __ldg(&S.ia[i]), ub = __ldg(&S.ib[i]);
+                    own = spin ? S.mb + 2 * ub * np : S.ma + 2 * ua * np;
+                    other = (spin ? S.ma + 2 * ua * np : S.mb + 2 * ub * np) + np;
+                }
                 for (int u0 = 0; u0 < units; u0 += 32) {
                     const int u = u0 + lane;
                     bool keep = false;
-                    Str<W> sj = si;
-                    double hv = 0.0;
+                    Key<KW> m{};
+                    double v = 0.0;
                     if (u < units) {
-                        flip_bit(sj, L.occ[spin][u / nv]);
-                        flip_bit(sj, L.vir[spin][u % nv]);
-                        hv = single_exc<W>(I, si, sj, spin ? A : B);
-                        keep = fabs(hv) * cmax >= S.eps1;
+                        const int x = u / nv;
+                        const int p = L.occ[spin][x], r = L.vir[spin][u - x * nv];
+                        set_bit(m, p + (spin ? beta : 0));
+                        set_bit(m, r + (spin ? beta : 0));
+                        if (own) {
+                            const int pr = pair_idx(p, r);
+                            v = flip_sign(__ldg(&own[pr]) + __ldg(&other[pr]), p < r);
+                        } else {
+                            const Str<W> &si = spin ? B : A;
+                            Str<W> sj = si;
+                            flip_bit(sj, p);
+                            flip_bit(sj, r);
+                            v = single_exc<W>(I, si, sj, spin ? A : B);
+                            if (FILL) v = flip_sign(v, common_parity<KW>(PD, m));    // emit applies it once more
+                        }
+                        keep = passes(cut, v);
                     }
-                    if (spin) emit(keep, A, sj, hv);
-                    else emit(keep, sj, B, hv);
+                    emit(keep, m, v);
                 }
             }
             for (int u0 = 0; u0 < pairs; u0 += 32) {
                 int v = u0 + lane;
-                int64_t e0 = 0;
-                int len = 0, spin = 2, p = 0, q = 0;      // spin 0: alpha pair, 1: beta pair, 2: alpha and beta
+                int e0 = 0, len = 0, holes = 0;
                 if (v < pairs) {
+                    int p, q;
+                    const int64_t *off = S.ss_off;
+                    const float *kf = S.ss_kf;
                     if (v < u_paa + u_pbb) {
-                        spin = v < u_paa ? 0 : 1;
+                        const int spin = v < u_paa ? 0 : 1;
                         if (spin) v -= u_paa;
                         // pair rank v -> (x < y): y is the largest with y (y - 1) / 2 <= v
                         int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)v)) * 0.5f);
@@ -428,18 +608,23 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
                         while ((y + 1) * y / 2 <= v) y++;
                         p = L.occ[spin][v - y * (y - 1) / 2];
                         q = L.occ[spin][y];
+                        holes = spin ? 0x20000 : 0;
                     } else {
                         v -= u_paa + u_pbb;
-                        p = L.occ[0][v / nb];
-                        q = L.occ[1][v % nb];
+                        const int x = v / nb;
+                        p = L.occ[0][x];
+                        q = L.occ[1][v - x * nb];
+                        holes = 0x10000;
+                        off = S.os_off;
+                        kf = S.os_kf;
                     }
-                    const int64_t *off = spin == 2 ? S.os_off : S.ss_off;
-                    const float *kf = spin == 2 ? S.os_kf : S.ss_kf;
-                    e0 = __ldg(&off[p * n + q]);
-                    int lo = 0, hi = (int)(__ldg(&off[p * n + q + 1]) - e0);
+                    holes |= p | (q << 8);
+                    const int64_t b = __ldg(&off[p * n + q]);
+                    e0 = (int)b;                          // at most 128^4 / 2 entries
+                    int lo = 0, hi = (int)(__ldg(&off[p * n + q + 1]) - b);
                     while (lo < hi) {                     // keys descend: first entry out of reach
                         const int mid = (lo + hi) >> 1;
-                        if (key_bound(__ldg(&kf[e0 + mid])) * cmax < S.eps1) hi = mid;
+                        if (__ldg(&kf[e0 + mid]) < cut.reach) hi = mid;
                         else lo = mid + 1;
                     }
                     len = lo;
@@ -451,57 +636,41 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
                     if (lane >= o) incl += y;
                 }
                 const int total = __shfl_sync(0xffffffffu, incl, 31);
-                const int pq = p | (q << 8) | (spin << 16);
+                const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+                __syncwarp();
+                if (len > 0) {
+                    const int at = __popc(some & lt);
+                    L.first[at] = e0 - (incl - len);
+                    L.holes[at] = holes;
+                }
+                __syncwarp();
+                const int start = len > 0 ? incl - len : 0x40000000;
+                int begun = 0;                            // lists that begin before this round
                 for (int t0 = 0; t0 < total; t0 += 32) {
                     const int t = t0 + lane;
-                    int src = 0;                          // the first lane with incl > t
-#pragma unroll
-                    for (int step = 16; step >= 1; step >>= 1) {
-                        const int y = __shfl_sync(0xffffffffu, incl, src + step - 1);
-                        if (y <= t) src += step;
-                    }
-                    src = min(src, 31);
-                    const int64_t first = __shfl_sync(0xffffffffu, e0, src);
-                    const int before = __shfl_sync(0xffffffffu, incl - len, src);
-                    const int x = __shfl_sync(0xffffffffu, pq, src);
+                    const unsigned rel = (unsigned)(start - t0);
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, rel < 32u ? 1u << rel : 0u);
+                    const int src = begun + __popc(starts & le) - 1;
+                    begun += __popc(starts);
                     bool keep = false;
-                    Str<W> a = A, b = B;
+                    Key<KW> m{};
                     double hv = 0.0;
                     if (t < total) {
-                        const int p1 = x & 255, q1 = (x >> 8) & 255, sp = x >> 16;
-                        const int64_t e = first + (t - before);
-                        const uint32_t rs = __ldg(sp == 2 ? &S.os_rs[e] : &S.ss_rs[e]);
-                        hv = __ldg(sp == 2 ? &S.os_v[e] : &S.ss_v[e]);
-                        const int r = (int)(rs & 0xFFFFu), s = (int)(rs >> 16);
-                        // the strings the two holes p1, q1 and particles r, s belong to
-                        const Str<W> &sa = sp == 1 ? B : A;
-                        const Str<W> &sb = sp == 0 ? A : B;
-                        keep = !has_bit(sa, r) && !has_bit(sb, s) && fabs(hv) * cmax >= S.eps1;
-                        if (keep) {
-                            int neg = 0;
-                            if (sp == 2) {
-                                flip_bit(a, p1);
-                                flip_bit(b, q1);
-                                if (FILL && PT)
-                                    neg = bits_between<W>(a, min(p1, r), max(p1, r)) + bits_between<W>(b, min(q1, s), max(q1, s));
-                                flip_bit(a, r);
-                                flip_bit(b, s);
-                            } else {
-                                // p1 -> r, then q1 -> s on the intermediate string
-                                Str<W> y = sa;
-                                if (FILL && PT) neg = bits_between<W>(y, min(p1, r), max(p1, r));
-                                flip_bit(y, p1);
-                                flip_bit(y, r);
-                                if (FILL && PT) neg += bits_between<W>(y, min(q1, s), max(q1, s));
-                                flip_bit(y, q1);
-                                flip_bit(y, s);
-                                if (sp) b = y;
-                                else a = y;
-                            }
-                            hv = flip_sign(hv, neg);
-                        }
+                        const int h = L.holes[src], e = L.first[src] + t;
+                        const bool opp = h & 0x10000;
+                        const uint32_t rs = __ldg(opp ? &S.os_rs[e] : &S.ss_rs[e]);
+                        hv = __ldg(opp ? &S.os_v[e] : &S.ss_v[e]);
+                        const int o1 = h & 0x20000 ? beta : 0, o2 = h & 0x30000 ? beta : 0;   // key bits of the two spins
+                        set_bit(m, (int)(rs & 0xFFFFu) + o1);
+                        set_bit(m, (int)(rs >> 16) + o2);
+                        bool free = true;                 // neither particle orbital is occupied
+#pragma unroll
+                        for (int w = 0; w < KW; w++) free = free && (m.w[w] & D.w[w]) == 0;
+                        keep = free && passes(cut, hv);
+                        set_bit(m, (h & 255) + o1);
+                        set_bit(m, ((h >> 8) & 255) + o2);
                     }
-                    emit(keep, a, b, hv);
+                    emit(keep, m, hv);
                 }
             }
         }
@@ -510,7 +679,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
 }
 
 // count pass over S's determinants and the offsets of their candidates; returns the total
-template <int W, int KW, bool PT>
+template <int W, int KW, bool TERMS>
 static int64_t count_candidates(shci_ctx *c, SelArgs &S, const DevInts &I, DevBuf<unsigned long long> &cnt,
                                 DevBuf<int64_t> &off, DevBuf<int64_t> &tmp) {
     cudaStream_t st = c->st;
@@ -521,7 +690,7 @@ static int64_t count_candidates(shci_ctx *c, SelArgs &S, const DevInts &I, DevBu
     S.cnt = cnt.p;
     S.off = off.p;
     const int blocks = (int)std::min<int64_t>(ceil_div(n, SEL_THREADS / 32), (int64_t)c->n_sm * (2048 / SEL_THREADS));
-    k_select<W, KW, false, PT><<<blocks, SEL_THREADS, 0, st>>>(S, I);
+    k_select<W, KW, false, TERMS ? SEL_TERMS : SEL_DETS><<<blocks, SEL_THREADS, 0, st>>>(S, I);
     KERNEL_CHECK();
     g_kernel_launches += 1;
     exclusive_scan<int64_t>(reinterpret_cast<const int64_t *>(cnt.p), off.p, n, tmp.p, st);
@@ -531,11 +700,11 @@ static int64_t count_candidates(shci_ctx *c, SelArgs &S, const DevInts &I, DevBu
     return total;
 }
 
-template <int W, int KW, bool PT>
+template <int W, int KW, int FOR>
 static void fill_candidates(shci_ctx *c, const SelArgs &S, const DevInts &I) {
     const int blocks = (int)std::min<int64_t>(ceil_div(S.n_det, SEL_THREADS / 32),
                                               (int64_t)c->n_sm * (2048 / SEL_THREADS));
-    k_select<W, KW, true, PT><<<blocks, SEL_THREADS, 0, c->st>>>(S, I);
+    k_select<W, KW, true, FOR><<<blocks, SEL_THREADS, 0, c->st>>>(S, I);
     KERNEL_CHECK();
     g_kernel_launches += 1;
 }
@@ -594,6 +763,8 @@ static void select_w(shci_ctx *c, int k, const double *cd, double eps1, DevBuf<u
     S.k = k;
     S.c = cd;
     const DevInts I = dev_ints(c);
+    MoveTables moves;
+    tabulate_moves<W>(c, S, I, (double)n, moves);
     DevBuf<unsigned long long> cnt;
     DevBuf<int64_t> off, tmp;
     const int64_t total = count_candidates<W, KW, false>(c, S, I, cnt, off, tmp);
@@ -604,7 +775,7 @@ static void select_w(shci_ctx *c, int k, const double *cd, double eps1, DevBuf<u
     DevBuf<uint64_t> cand;
     cand.alloc((size_t)total * KW);
     S.out = cand.p;
-    fill_candidates<W, KW, false>(c, S, I);
+    fill_candidates<W, KW, SEL_DETS>(c, S, I);
     radix_sort<KW>(cand.p, nullptr, total, c->sw, st, KeyMask<W, KW>(c->n_orb).w, RS_KEYS);
     DevBuf<uint64_t> vs;
     sorted_space<W, KW>(c, vs);
@@ -681,16 +852,19 @@ __device__ __forceinline__ void run_terms(const RunArgs &A, int64_t e, double *v
 // are summed by a segmented tree of shuffles, the last one's continuation by
 // the whole warp, 128 elements at a time; the runs' keys and sums are queued
 // and finished 32 at a time (is a in V, H_aa, the contribution).  A thread per
-// run, adding up its terms one by one, took 27 ms for 1.8e8 terms and 18
-// ms for a sample of 4e7, nearly all of it the longest runs' chains of
-// dependent loads; this form 4.9 and 6.3.  The order of every
-// sum is fixed.
+// run, adding up its terms one by one, took 27 ms for 1.8e8 terms and 18 ms
+// for a sample of 5e7, nearly all of it the longest runs' chains of dependent
+// loads; this form 4.8 and 5.5, with the FP64 pipe 78 % busy (the tree's
+// additions, H_aa, the division).  The order of every sum is fixed.
+constexpr int RUN_CHUNK = 16;
+
 template <int W, int KW, int MODE>
 __global__ void __launch_bounds__(SEL_THREADS) k_run_reduce(RunArgs A, DevInts I) {
     constexpr int NS = RunSums<MODE>::N;
     constexpr int NW = SEL_THREADS / 32;
     __shared__ __align__(16) uint64_t qkey[NW][64 * KW];
     __shared__ double qsum[NW][64 * NS];
+    __shared__ double ftab[NW][W == 1 ? 64 : SHCI_MAX_ORB];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     uint64_t *qk = qkey[wib];
@@ -698,30 +872,94 @@ __global__ void __launch_bounds__(SEL_THREADS) k_run_reduce(RunArgs A, DevInts I
     double acc0 = 0.0, acc1 = 0.0;
     unsigned long long cnt = 0;
     int qn = 0;
-    auto finish = [&](int m) {                            // the first m (<= 32) queued runs
-        if (lane < m) {
-            const Key<KW> x = load_key<KW>(qk, lane);
-            if (!in_sorted<KW>(A.vs, A.nv, x)) {
-                Str<W> a, b;
-                split_key<W, KW>(x, I.n, a, b);
-                const double den = A.e_var - hii<W>(I, a, b);
-                const double *v = qs + lane * NS;
-                if constexpr (MODE == RUN_PT) {
-                    acc0 += v[0] * v[0] / den;
-                } else if constexpr (MODE == RUN_SAMPLE) {
-                    acc0 += (v[0] * v[0] + v[1]) / den;
-                    acc1 += (v[2] * v[2] + v[3]) / den;
-                } else {
-                    const double corr = (v[0] * v[0] - v[1] * v[1]) / den;
-                    acc0 += corr;
-                    acc1 += corr * corr;
-                }
-                cnt++;
+    // H_aa of sorted runs: most of 32 consecutive ones share their beta string b
+    // (its bits are the key's high ones), so the warp tabulates, once per b,
+    // b's own energy and f_k = h_kk + sum_{l in b} J_kl; a run then adds f over
+    // its alpha electrons and their pairs: 21 FP64 additions instead of 78 for
+    // six electrons a spin.  Runs of a fourth string among the 32 sum in full.
+    double *f = ftab[wib];
+    Str<W> bcur{};
+    double ecur = 0.0;
+    bool have = false;
+    auto diagonal = [&](bool need, const Str<W> &a, const Str<W> &b) {
+        double e = 0.0;
+        unsigned todo = __ballot_sync(0xffffffffu, need);
+        for (int g = 0; todo != 0; g++) {
+            if (g == 3) {
+                if ((todo >> lane) & 1u) e = hii<W>(I, a, b);
+                break;
             }
+            Str<W> bg;
+            bool cur = have, mine = (todo >> lane) & 1u;
+#pragma unroll
+            for (int k = 0; k < W; k++) {
+                bg.w[k] = __shfl_sync(0xffffffffu, b.w[k], __ffs(todo) - 1);
+                cur = cur && bg.w[k] == bcur.w[k];
+                mine = mine && bg.w[k] == b.w[k];
+            }
+            if (!cur) {                                   // warp-uniform
+                __syncwarp();
+                double eb = 0.0;
+                for (int k = lane; k < I.n; k += 32) {
+                    const double hk = __ldg(&I.h[k * I.n + k]);
+                    double v = hk;
+                    for_bits_above<W>(bg, -1, [&](int l) { v += __ldg(&I.jdiag[k * I.n + l]); });
+                    f[k] = v;
+                    if (has_bit(bg, k)) {
+                        eb += hk;
+                        for_bits_above<W>(bg, k, [&](int l) { eb += __ldg(&I.jkdiag[k * I.n + l]); });
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) eb += __shfl_xor_sync(0xffffffffu, eb, o);
+                __syncwarp();
+                bcur = bg;
+                ecur = eb;
+                have = true;
+            }
+            if (mine) {
+                e = I.e_core + ecur;
+                for_bits_above<W>(a, -1, [&](int k) {
+                    e += f[k];
+                    for_bits_above<W>(a, k, [&](int l) { e += __ldg(&I.jkdiag[k * I.n + l]); });
+                });
+            }
+            todo &= ~__ballot_sync(0xffffffffu, mine);
+        }
+        return e;
+    };
+    auto finish = [&](int m) {                            // the first m (<= 32) queued runs
+        Key<KW> x{};
+        bool need = false;
+        if (lane < m) {
+            x = load_key<KW>(qk, lane);
+            need = !in_sorted<KW>(A.vs, A.nv, x);
+        }
+        Str<W> a, b;
+        split_key<W, KW>(x, I.n, a, b);
+        const double haa = diagonal(need, a, b);
+        if (need) {
+            const double den = A.e_var - haa;
+            const double *v = qs + lane * NS;
+            if constexpr (MODE == RUN_PT) {
+                acc0 += v[0] * v[0] / den;
+            } else if constexpr (MODE == RUN_SAMPLE) {
+                acc0 += (v[0] * v[0] + v[1]) / den;
+                acc1 += (v[2] * v[2] + v[3]) / den;
+            } else {
+                const double corr = (v[0] * v[0] - v[1] * v[1]) / den;
+                acc0 += corr;
+                acc1 += corr * corr;
+            }
+            cnt++;
         }
     };
+    // RUN_CHUNK consecutive windows at a time: a warp's queued runs are neighbours
     const int64_t windows = (A.total + 31) >> 5, warps = (int64_t)gridDim.x * NW;
-    for (int64_t w = ((int64_t)blockIdx.x * SEL_THREADS + threadIdx.x) >> 5; w < windows; w += warps) {
+    const int64_t first = ((int64_t)blockIdx.x * SEL_THREADS + threadIdx.x) >> 5;
+    for (int64_t step = 0;; step++) {
+        const int64_t w = (step / RUN_CHUNK * warps + first) * RUN_CHUNK + step % RUN_CHUNK;
+        if (w >= windows) break;
         const int64_t e = w * 32 + lane;
         const bool in = e < A.total;
         Key<KW> x{}, before{};
@@ -859,7 +1097,8 @@ static void reduce_terms(shci_ctx *c, SelArgs &S, const DevInts &I, int64_t tota
     S.terms = T.t1.p;
     S.terms2 = T.t2.p;
     S.mags = T.mag.p;
-    fill_candidates<W, KW, true>(c, S, I);
+    constexpr int FOR = MODE == RUN_PT ? SEL_TERMS : (MODE == RUN_SAMPLE ? SEL_SAMPLE : SEL_MAGS);
+    fill_candidates<W, KW, FOR>(c, S, I);
     radix_sort<KW>(T.cand.p, T.idx.p, total, c->sw, st, KeyMask<W, KW>(c->n_orb).w, RS_POSITION);
     const int blocks = c->n_sm * 8;
     T.part.alloc((size_t)2 * blocks);
@@ -900,6 +1139,8 @@ static double pt2_w(shci_ctx *c, const double *cd, double e_var, double eps2, in
     SelArgs S = sel_args(c, eps2);
     S.c = cd;
     const DevInts I = dev_ints(c);
+    MoveTables moves;
+    tabulate_moves<W>(c, S, I, (double)c->n_det, moves);
     TermWork T;
     // batches: enough that one batch's candidates and their sort fit a quarter of free memory
     constexpr double BYTES_PER_CAND = 2.0 * 8 * KW + 8 + 2 * 4;
@@ -958,126 +1199,47 @@ __global__ void k_sum_in_order(const double *__restrict__ part, int m, double *_
     *out = t;
 }
 
-// Walker's alias table for p_i = |c_i| / sum (Eq. 10), by Vose's two-list
-// method: q_i = n p_i, the lists of small (q < 1) and large columns in
-// ascending order, then pairs from the lists' ends.
-__global__ void k_alias_split(const double *__restrict__ c, int64_t n, const double *__restrict__ sum,
-                              double *__restrict__ q, int64_t *__restrict__ is_small) {
-    const double scale = (double)n / *sum;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        q[i] = fabs(c[i]) * scale;
-        is_small[i] = q[i] < 1.0 ? 1 : 0;
+// Walker's alias table for p_i = |c_i| / sum (Eq. 10), built by Vose's
+// two-list method: q_i = n p_i; the small column (q < 1) on top of its stack
+// takes the large column g on top of the other as its alias, g keeps
+// q_g + q_l - 1, and a g that falls below 1 goes onto the small stack.  Every
+// step needs the rounded result of the one before it and no two can be
+// exchanged, so this is one chain of n additions, and it runs on a host core.
+// On the GPU 100,003 columns took one thread 43.4 ms (dependent loads), one
+// warp that staged the columns in shared memory for one lane 10.3 ms (two
+// dependent FP64 additions, a test and a branch per column), and the same in
+// integers that give the additions' bits 12.8 to 14.9; the semistochastic
+// energy of that space went from 61.5 ms with the last form to 50.7 with this.
+static void alias_table(const double *c, int64_t n, double sum, double *prob, uint32_t *alias) {
+    const double scale = (double)n / sum;
+    std::vector<uint32_t> stack((size_t)n);              // small columns from the front, large ones from the back
+    int64_t ns = 0, nl = 0;
+    for (int64_t i = 0; i < n; i++) {
+        prob[i] = std::fabs(c[i]) * scale;
+        alias[i] = (uint32_t)i;
+        if (prob[i] < 1.0) ns++;
     }
-}
-
-// the lists, and the table's values for columns that are never paired: a large
-// column keeps itself (probability 1), a small one its q and itself
-__global__ void k_alias_lists(const double *__restrict__ q, int64_t n, const int64_t *__restrict__ pos,
-                              uint32_t *__restrict__ small, uint32_t *__restrict__ large, double *__restrict__ prob,
-                              int64_t *__restrict__ alias) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = pos[i];
-        const bool is_small = q[i] < 1.0;
-        if (is_small) small[s] = (uint32_t)i;
-        else large[i - s] = (uint32_t)i;
-        prob[i] = is_small ? q[i] : 1.0;
-        alias[i] = i;
+    std::vector<uint32_t> large((size_t)(n - ns));
+    ns = 0;
+    for (int64_t i = 0; i < n; i++) {
+        if (prob[i] < 1.0) stack[ns++] = (uint32_t)i;
+        else large[nl++] = (uint32_t)i;
     }
-}
-
-// The pairing: the small column on top of its stack takes the large column g
-// on top of the other as its alias, g keeps q_g + q_l - 1, and a g that falls
-// below 1 goes onto the small stack.  Each step needs the one before it, but a
-// demoted g is popped by the very next step, so both stacks are read strictly
-// from their ends: one warp stages ALIAS_CH columns of each in shared memory,
-// one lane runs the chain of additions over them, and the warp writes the
-// aliases.  Bound by that chain (two dependent FP64 additions per column).
-// With every access a dependent global load, 100,003 columns took 43.4 ms;
-// this form 10.3.
-constexpr int ALIAS_CH = 1024;
-
-__global__ void __launch_bounds__(32) k_alias_pair(const double *__restrict__ q, const uint32_t *__restrict__ small,
-                                                   const uint32_t *__restrict__ large, const int64_t *__restrict__ n_small,
-                                                   int64_t n, double *__restrict__ prob, int64_t *__restrict__ alias) {
-    __shared__ double sq[ALIAS_CH + 1], lq[ALIAS_CH];
-    __shared__ uint32_t sidx[ALIAS_CH], lidx[ALIAS_CH], spair[ALIAS_CH];
-    const int lane = threadIdx.x;
-    int64_t ns = *n_small, nl = n - ns;                  // columns not yet staged
-    int sc = 0, sk = 0, lc = 0, lk = 0;                  // staged and consumed
-    bool have = false, demoted = false;                  // a large column in hand; a demoted one on top of the small stack
-    double gq = 0.0, dq = 0.0;
-    uint32_t gi = 0, di = 0;
-    while (true) {
-        if (sk == sc && ns > 0) {
-            sc = (int)min((int64_t)ALIAS_CH, ns);
-            for (int x = lane; x < sc; x += 32) {
-                sidx[x] = small[ns - 1 - x];
-                sq[x] = q[sidx[x]];
-            }
-            ns -= sc;
-            sk = 0;
-        }
-        if (lk == lc && nl > 0) {
-            lc = (int)min((int64_t)ALIAS_CH, nl);
-            for (int x = lane; x < lc; x += 32) {
-                lidx[x] = large[nl - 1 - x];
-                lq[x] = q[lidx[x]];
-            }
-            nl -= lc;
-            lk = 0;
-        }
-        __syncwarp();
-        const int from = sk;
-        if (lane == 0) {
-            while (true) {
-                if (!have) {
-                    if (lk == lc) break;
-                    gi = lidx[lk];
-                    gq = lq[lk++];
-                    have = true;
-                }
-                if (demoted) {
-                    prob[di] = dq;
-                    alias[di] = gi;
-                    gq = (gq + dq) - 1.0;
-                    demoted = false;
-                } else {
-                    if (sk == sc) break;
-                    double next = sq[sk];
-                    do {                                  // q_g >= 1 and q_l >= 0: the sign needs no test
-                        const double l = next;
-                        spair[sk] = gi;
-                        next = sq[++sk];
-                        gq = (gq + l) - 1.0;
-                    } while (sk < sc && __double2hiint(gq) >= 0x3FF00000);
-                }
-                if (__double2hiint(gq) < 0x3FF00000) {    // below 1
-                    demoted = true;
-                    di = gi;
-                    dq = gq;
-                    have = false;
-                }
-            }
-        }
-        sk = __shfl_sync(0xffffffffu, sk, 0);
-        lk = __shfl_sync(0xffffffffu, lk, 0);
-        have = __shfl_sync(0xffffffffu, (int)have, 0);
-        demoted = __shfl_sync(0xffffffffu, (int)demoted, 0);
-        __syncwarp();
-        for (int x = from + lane; x < sk; x += 32) alias[sidx[x]] = spair[x];
-        __syncwarp();
-        if ((!demoted && sk == sc && ns == 0) || (!have && lk == lc && nl == 0)) break;
+    while (ns > 0 && nl > 0) {
+        const uint32_t l = stack[--ns], g = large[--nl];
+        alias[l] = g;                                    // prob[l] stays
+        prob[g] = (prob[g] + prob[l]) - 1.0;
+        if (prob[g] < 1.0) stack[ns++] = g;
+        else nl++;
     }
-    // rounding leftovers keep themselves: the demoted column on top, the small columns never paired
-    if (lane == 0 && demoted) prob[di] = 1.0;
-    for (int x = sk + lane; x < sc; x += 32) prob[sidx[x]] = 1.0;
-    for (int64_t x = lane; x < ns; x += 32) prob[small[x]] = 1.0;
+    while (nl > 0) prob[large[--nl]] = 1.0;
+    while (ns > 0) prob[stack[--ns]] = 1.0;              // rounding leftovers
 }
 
 // draw d: r = SplitMix64 output for the counter seed + (d + 1) * golden
 // gamma; column = high 32 bits * n >> 32, uniform u = low 32 bits / 2^32;
 // the column itself when u < prob[column], else its alias
-__global__ void k_alias_draw(const double *__restrict__ prob, const int64_t *__restrict__ alias, int64_t n,
+__global__ void k_alias_draw(const double *__restrict__ prob, const uint32_t *__restrict__ alias, int64_t n,
                              uint64_t seed, int64_t n_draws, int64_t *__restrict__ out) {
     for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < n_draws;
          d += (int64_t)gridDim.x * blockDim.x) {
@@ -1087,7 +1249,7 @@ __global__ void k_alias_draw(const double *__restrict__ prob, const int64_t *__r
         z ^= z >> 31;
         const int64_t col = (int64_t)(((z >> 32) * (uint64_t)n) >> 32);
         const double u = (double)(uint32_t)z * 0x1p-32;
-        out[d] = u < prob[col] ? col : alias[col];
+        out[d] = u < prob[col] ? col : (int64_t)alias[col];
     }
 }
 
@@ -1111,9 +1273,10 @@ static double abs_sum(shci_ctx *c, const double *cd, int64_t n) {
 // per-determinant compact arrays (strings, c_i, w/p, w (n_d - 1)/p - w^2/p^2)
 template <int W>
 __global__ void k_sample_prep(const uint64_t *__restrict__ sorted, int64_t n_d, const int64_t *__restrict__ pos,
-                              const uint64_t *__restrict__ dets, const double *__restrict__ c, double csum,
-                              uint64_t *__restrict__ sdets, double *__restrict__ sc, double *__restrict__ f1,
-                              double *__restrict__ f2) {
+                              const uint64_t *__restrict__ dets, const int32_t *__restrict__ ia,
+                              const int32_t *__restrict__ ib, const double *__restrict__ c, double csum,
+                              uint64_t *__restrict__ sdets, int32_t *__restrict__ sia, int32_t *__restrict__ sib,
+                              double *__restrict__ sc, double *__restrict__ f1, double *__restrict__ f2) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_d; e += (int64_t)gridDim.x * blockDim.x) {
         if (e > 0 && sorted[e - 1] == sorted[e]) continue;
         int64_t f = e + 1;
@@ -1122,6 +1285,8 @@ __global__ void k_sample_prep(const uint64_t *__restrict__ sorted, int64_t n_d, 
         const double w = (double)(f - e), p = fabs(c[i]) / csum;
 #pragma unroll
         for (int k = 0; k < 2 * W; k++) sdets[u * 2 * W + k] = dets[i * 2 * W + k];
+        sia[u] = ia[i];
+        sib[u] = ib[i];
         sc[u] = c[i];
         f1[u] = w / p;
         f2[u] = w * (double)(n_d - 1) / p - w * w / (p * p);
@@ -1154,6 +1319,7 @@ static void pt2_samples_w(shci_ctx *c, const double *cd, double e_var, double ep
     const DevInts I = dev_ints(c);
     DevBuf<uint64_t> sorted, sdets;
     DevBuf<int64_t> flag, pos, tmp;
+    DevBuf<int32_t> sia, sib;
     DevBuf<double> sc, f1, f2;
     sorted.alloc((size_t)n_d);
     flag.alloc((size_t)n_d + 1);
@@ -1163,6 +1329,11 @@ static void pt2_samples_w(shci_ctx *c, const double *cd, double e_var, double ep
     sc.alloc((size_t)n_d);
     f1.alloc((size_t)n_d);
     f2.alloc((size_t)n_d);
+    sia.alloc((size_t)n_d);
+    sib.alloc((size_t)n_d);
+    MoveTables moves;
+    SelArgs S0 = sel_args(c, eps2);
+    tabulate_moves<W>(c, S0, I, (double)std::min(n_d, n) * n_samples, moves);
     uint64_t vary = 1;                      // bits of an index of V
     while ((int64_t)vary < n - 1) vary = 2 * vary + 1;
     const int gb = (int)std::min<int64_t>(ceil_div(n_d, SEL_THREADS), (int64_t)c->n_sm * 16);
@@ -1174,12 +1345,14 @@ static void pt2_samples_w(shci_ctx *c, const double *cd, double e_var, double ep
         exclusive_scan<int64_t>(flag.p, pos.p, n_d, tmp.p, st);
         int64_t n_dist = 0;
         CUDA_TRY(cudaMemcpyAsync(&n_dist, pos.p + n_d, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        k_sample_prep<W><<<gb, SEL_THREADS, 0, st>>>(sorted.p, n_d, pos.p, c->dets.p, cd, csum, sdets.p, sc.p, f1.p,
-                                                     f2.p);
+        k_sample_prep<W><<<gb, SEL_THREADS, 0, st>>>(sorted.p, n_d, pos.p, c->dets.p, c->ia.p, c->ib.p, cd, csum,
+                                                     sdets.p, sia.p, sib.p, sc.p, f1.p, f2.p);
         KERNEL_CHECK();
         g_kernel_launches += 2;
         CUDA_TRY(cudaStreamSynchronize(st));
-        SelArgs S = sel_args(c, eps2);
+        SelArgs S = S0;
+        S.ia = sia.p;
+        S.ib = sib.p;
         S.n_det = n_dist;
         S.dets = sdets.p;
         S.c = sc.p;
@@ -1268,36 +1441,34 @@ void alias_draw(shci_ctx *c, const double *coef, int64_t n_draws, uint64_t seed,
     cudaStream_t st = c->st;
     const int64_t n = c->n_det;
     if (n > 0xFFFFFFFFll) throw ShciError{SHCI_ERR_INVALID, "too many determinants for the sampler"};
-    const double *cd = coef;
+    const double *cd = coef, *hc = coef;                 // on the device, on the host
     DevBuf<double> cbuf;
+    std::vector<double> copy;
     if (mem == SHCI_MEM_HOST) {
         cbuf.alloc((size_t)n);
         CUDA_TRY(cudaMemcpyAsync(cbuf.p, coef, sizeof(double) * n, cudaMemcpyHostToDevice, st));
         cd = cbuf.p;
+    } else {
+        copy.resize((size_t)n);
+        CUDA_TRY(cudaMemcpyAsync(copy.data(), coef, sizeof(double) * n, cudaMemcpyDeviceToHost, st));
+        hc = copy.data();
     }
-    const double csum = abs_sum(c, cd, n);
+    const double csum = abs_sum(c, cd, n);               // waits for the stream: the copy is done
     if (!(csum > 0.0)) throw ShciError{SHCI_ERR_INVALID, "all coefficients are zero"};
-    DevBuf<double> prob, q, sum;
-    DevBuf<int64_t> alias, flag, pos, tmp, obuf;
-    DevBuf<uint32_t> small, large;
+    std::vector<double> hp((size_t)n);
+    std::vector<uint32_t> ha((size_t)n);
+    alias_table(hc, n, csum, hp.data(), ha.data());
+    DevBuf<double> prob;
+    DevBuf<uint32_t> alias;
+    DevBuf<int64_t> obuf;
     prob.alloc((size_t)n);
-    q.alloc((size_t)n);
-    sum.alloc(1);
     alias.alloc((size_t)n);
-    flag.alloc((size_t)n + 1);
-    pos.alloc((size_t)n + 1);
-    tmp.alloc((size_t)scan_tmp_len(n + 1));
-    small.alloc((size_t)n);
-    large.alloc((size_t)n);
-    CUDA_TRY(cudaMemcpyAsync(sum.p, &csum, sizeof(double), cudaMemcpyHostToDevice, st));
-    const int gn = (int)std::min<int64_t>(ceil_div(n, SEL_THREADS), (int64_t)c->n_sm * 16);
-    k_alias_split<<<gn, SEL_THREADS, 0, st>>>(cd, n, sum.p, q.p, flag.p);
-    exclusive_scan<int64_t>(flag.p, pos.p, n, tmp.p, st);
-    k_alias_lists<<<gn, SEL_THREADS, 0, st>>>(q.p, n, pos.p, small.p, large.p, prob.p, alias.p);
-    k_alias_pair<<<1, 32, 0, st>>>(q.p, small.p, large.p, pos.p + n, n, prob.p, alias.p);
-    KERNEL_CHECK();
-    g_kernel_launches += 3;
-    if (n_draws == 0) return;
+    CUDA_TRY(cudaMemcpyAsync(prob.p, hp.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(alias.p, ha.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, st));
+    if (n_draws == 0) {
+        CUDA_TRY(cudaStreamSynchronize(st));
+        return;
+    }
     int64_t *o = out;
     if (mem == SHCI_MEM_HOST) {
         obuf.alloc((size_t)n_draws);
@@ -1366,6 +1537,8 @@ static void psto_w(shci_ctx *c, const double *cd, double e_var, double eps_psto,
     S.c = cd;
     S.nbatch = nbatch;
     const DevInts I = dev_ints(c);
+    MoveTables moves;
+    tabulate_moves<W>(c, S, I, (double)c->n_det * nbatch, moves);
     TermWork T;
     sorted_space<W, KW>(c, T.vs);
     double sum = 0.0, sum2 = 0.0;
@@ -1493,13 +1666,12 @@ void pt2_semistochastic(shci_ctx *c, const double *coef, double e_var, double ep
     if (e2_err) *e2_err = n_samples > 1 ? std::sqrt(var / (n_samples - 1) / n_samples) : 0.0;
 }
 
-void select_dets(shci_ctx *c, int k, const double *coef, double eps1, int64_t cap, uint64_t *out, int64_t *n_out,
-                 int mem) {
+void select_dets(shci_ctx *c, int k, const double *coef, double eps1, int mem, int64_t *n_out,
+                 const std::function<std::pair<uint64_t *, int64_t>(int64_t)> &place) {
     if (!c->built) throw ShciError{SHCI_ERR_STATE, "build the connectivity before selecting"};
     if (k < 1 || k > SHCI_MAX_K) throw ShciError{SHCI_ERR_INVALID, "k must be in [1, 8]"};
     if (!(eps1 > 0.0) || !std::isfinite(eps1)) throw ShciError{SHCI_ERR_INVALID, "eps1 must be positive and finite"};
     if (!coef || !n_out) throw ShciError{SHCI_ERR_INVALID, "null pointer"};
-    if (cap < 0) throw ShciError{SHCI_ERR_INVALID, "cap must be >= 0"};
     if (mem != SHCI_MEM_HOST && mem != SHCI_MEM_DEVICE) throw ShciError{SHCI_ERR_INVALID, "unknown mem_space"};
     if (c->n_orb > 128) throw ShciError{SHCI_ERR_INVALID, "selection supports up to 128 orbitals"};
     cudaStream_t st = c->st;
@@ -1526,11 +1698,11 @@ void select_dets(shci_ctx *c, int k, const double *coef, double eps1, int64_t ca
 #undef CALL
     *n_out = n_new;
     const int KW = 2 * c->W;
-    if (n_new > 0 && cap > 0) {
-        if (!out) throw ShciError{SHCI_ERR_INVALID, "null output pointer"};
-        const int64_t m = std::min(cap, n_new);
-        CUDA_TRY(cudaMemcpyAsync(out, result.p, sizeof(uint64_t) * m * KW,
-                                 mem == SHCI_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
+    if (n_new > 0) {
+        const std::pair<uint64_t *, int64_t> to = place(n_new);
+        if (to.second > 0)
+            CUDA_TRY(cudaMemcpyAsync(to.first, result.p, sizeof(uint64_t) * to.second * KW,
+                                     mem == SHCI_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
     }
     CUDA_TRY(cudaEventRecord(e1, st));
     CUDA_TRY(cudaEventSynchronize(e1));
