@@ -80,6 +80,35 @@ __device__ __forceinline__ void red_add(double *p, double v) {
     asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v) : "memory");
 }
 
+// Sums of NV values over the warp: afterwards lane holds in v[0] the sum of
+// value `return`, each value in 32 / P lanes (P: NV rounded up to a power of
+// two; values past NV are zero).  At each of the first log2(P) levels a lane
+// keeps one half of the values it holds, so P - 1 + log2(32 / P) additions
+// instead of 5 NV: FP64 additions are what such a reduction costs.
+template <int NV>
+__device__ __forceinline__ int warp_sum_many(const double (&in)[NV], double &sum) {
+    constexpr int P = NV <= 1 ? 1 : (NV <= 2 ? 2 : (NV <= 4 ? 4 : (NV <= 8 ? 8 : (NV <= 16 ? 16 : 32))));
+    const int lane = threadIdx.x & 31;
+    double v[P];
+#pragma unroll
+    for (int e = 0; e < P; e++) v[e] = e < NV ? in[e < NV ? e : 0] : 0.0;
+    int own = 0, mask = 16;
+#pragma unroll
+    for (int half = P >> 1; half >= 1; half >>= 1, mask >>= 1) {
+        const bool upper = (lane & mask) != 0;
+#pragma unroll
+        for (int e = 0; e < half; e++) {
+            const double send = upper ? v[e] : v[e + half];
+            const double keep = upper ? v[e + half] : v[e];
+            v[e] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+        }
+        own += upper ? half : 0;
+    }
+    for (; mask >= 1; mask >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
+    sum = v[0];
+    return own;
+}
+
 __device__ __forceinline__ int popc2(uint64_t a, uint64_t b) { return __popcll(a ^ b); }
 
 template <int W>

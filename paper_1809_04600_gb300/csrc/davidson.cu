@@ -85,11 +85,9 @@ __global__ void __launch_bounds__(DV_THREADS) k_gram_f(const double *__restrict_
         const int r = min(a0 + a, na - 1);
         rowp[a] = r < mv ? V + (int64_t)r * n : T + (int64_t)(r - mv) * n;
     }
-    double acc[NA][NB];
+    double acc[NE];
 #pragma unroll
-    for (int a = 0; a < NA; a++)
-#pragma unroll
-        for (int b = 0; b < NB; b++) acc[a][b] = 0.0;
+    for (int e = 0; e < NE; e++) acc[e] = 0.0;
     const int64_t stride = (int64_t)gridDim.x * DV_THREADS;
     for (int64_t i = blockIdx.x * (int64_t)DV_THREADS + tid; i < n; i += stride) {
         double bv[NB];
@@ -100,20 +98,15 @@ __global__ void __launch_bounds__(DV_THREADS) k_gram_f(const double *__restrict_
             if (a < cnt) {
                 const double av = rowp[a][i];
 #pragma unroll
-                for (int b = 0; b < NB; b++) acc[a][b] = fma(av, bv[b], acc[a][b]);
+                for (int b = 0; b < NB; b++) acc[a * NB + b] = fma(av, bv[b], acc[a * NB + b]);
             }
         }
     }
     __shared__ double red[NE][DV_THREADS / 32];
-#pragma unroll
-    for (int a = 0; a < NA; a++) {
-#pragma unroll
-        for (int b = 0; b < NB; b++) {
-            double v = acc[a][b];
-#pragma unroll
-            for (int o2 = 16; o2 >= 1; o2 >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o2);
-            if (lane == 0) red[a * NB + b][w] = v;
-        }
+    {
+        double v;
+        const int e = warp_sum_many<NE>(acc, v);
+        if (e < NE) red[e][w] = v;
     }
     __syncthreads();
     const int64_t gbase = (int64_t)blockIdx.y * gridDim.x * NE;
@@ -166,15 +159,23 @@ __global__ void __launch_bounds__(DV_THREADS) k_gram_f(const double *__restrict_
         return;
     }
     // EP_ORTHO: C = R[0..mv), S = R[mv..mv + NB); projected Gram S' = S - C^T C
-    // (V orthonormal), then Cholesky-QR coefficients M of (T - V C) and C M
-    for (int e = tid; e < NB * NB; e += DV_THREADS) {
+    // (V orthonormal), then Cholesky-QR coefficients M of (T - V C) and C M.
+    // R is staged in shared memory and each entry of C^T C summed by a warp:
+    // one thread's chain of loads and FP64 additions over mv rows took longer
+    // than the whole product of a 44,100-element block.
+    __shared__ double Rs[(SHCI_MAX_SUB + NB) * NB];
+    for (int e = tid; e < na * NB; e += DV_THREADS) Rs[e] = __ldcg(&o.R[e]);
+    __syncthreads();
+    for (int e = w; e < NB * NB; e += DV_THREADS / 32) {
         const int j = e / NB, l = e % NB;
-        double v = __ldcg(&o.R[(mv + j) * NB + l]);
-        for (int a = 0; a < mv; a++) v -= __ldcg(&o.R[a * NB + j]) * __ldcg(&o.R[a * NB + l]);
-        Ss[e] = v;
+        double v = 0.0;
+        for (int a = lane; a < mv; a += 32) v = fma(Rs[a * NB + j], Rs[a * NB + l], v);
+#pragma unroll
+        for (int x = 16; x >= 1; x >>= 1) v += __shfl_xor_sync(0xffffffffu, v, x);
+        if (lane == 0) Ss[e] = Rs[(mv + j) * NB + l] - v;
     }
     if (o.pass == 1 && tid < NB) {
-        pres[tid] = __ldcg(&o.R[(mv + tid) * NB + tid]);
+        pres[tid] = Rs[(mv + tid) * NB + tid];
         o.pre[tid] = pres[tid];
     } else if (tid < NB) {
         pres[tid] = __ldcg(&o.pre[tid]);
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(DV_THREADS) k_gram_f(const double *__restrict_
     for (int e = tid; e < mv * NB; e += DV_THREADS) {
         const int a = e / NB, l = e % NB;
         double v = 0.0;
-        for (int j = 0; j < NB; j++) v = fma(__ldcg(&o.R[a * NB + j]), Ms[j * NB + l], v);
+        for (int j = 0; j < NB; j++) v = fma(Rs[a * NB + j], Ms[j * NB + l], v);
         o.CM[e] = v;
     }
 }
@@ -318,15 +319,20 @@ __global__ void __launch_bounds__(DV_THREADS) k_ritz(const double *__restrict__ 
 #pragma unroll
         for (int l = 0; l < K; l++) { x[l] = 0.0; h[l] = 0.0; }
         int a = 0;
-        for (; a + 2 <= m; a += 2) {
-            const double v0 = V[(int64_t)a * n + i], w0 = AV[(int64_t)a * n + i];
-            const double v1 = V[(int64_t)(a + 1) * n + i], w1 = AV[(int64_t)(a + 1) * n + i];
+        for (; a + 4 <= m; a += 4) {
+            double v[4], w[4];
 #pragma unroll
-            for (int l = 0; l < K; l++) {
-                x[l] = fma(ys[a * K + l], v0, x[l]);
-                h[l] = fma(ys[a * K + l], w0, h[l]);
-                x[l] = fma(ys[(a + 1) * K + l], v1, x[l]);
-                h[l] = fma(ys[(a + 1) * K + l], w1, h[l]);
+            for (int u = 0; u < 4; u++) {
+                v[u] = V[(int64_t)(a + u) * n + i];
+                w[u] = AV[(int64_t)(a + u) * n + i];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+#pragma unroll
+                for (int l = 0; l < K; l++) {
+                    x[l] = fma(ys[(a + u) * K + l], v[u], x[l]);
+                    h[l] = fma(ys[(a + u) * K + l], w[u], h[l]);
+                }
             }
         }
         for (; a < m; a++) {
@@ -358,12 +364,10 @@ __global__ void __launch_bounds__(DV_THREADS) k_ritz(const double *__restrict__ 
     if (MODE == 0) {
         __shared__ double red[K][DV_THREADS / 32];
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-        for (int l = 0; l < K; l++) {
-            double v = rn[l];
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) red[l][w] = v;
+        {
+            double v;
+            const int l = warp_sum_many<K>(rn, v);
+            if (l < K) red[l][w] = v;
         }
         __syncthreads();
         if (threadIdx.x < K) {
@@ -397,7 +401,7 @@ __global__ void __launch_bounds__(DV_THREADS) k_ritz(const double *__restrict__ 
 __global__ void k_jacobi(const double *__restrict__ G, int ld, int m, int m_prev, double *__restrict__ eval,
                          double *__restrict__ evec) {
     extern __shared__ double jsm[];
-    jacobi_solve(G, ld, m, m_prev, eval, evec, jsm);
+    subspace_eig(G, ld, m, m_prev, eval, evec, jsm);
 }
 
 // ---------------------------------------------------------------- start vectors
@@ -547,7 +551,7 @@ struct Dav {
         constexpr int NA = GramShape<NB>::NA;
         const int na = mv + mt;
         const int groups = (na + NA - 1) / NA;
-        const int slices = std::max(1, std::min<int>((int)ceil_div(n, DV_THREADS * 4), n_slots / groups));
+        const int slices = std::max(1, std::min<int>((int)ceil_div(n, DV_THREADS * 2), n_slots / groups));
         dim3 grid(slices, groups);
         k_gram_f<NB><<<grid, DV_THREADS, 0, st>>>(V, mv, T, mt, B, n, c->dw.partial.p, ctr, o, skip);
         KERNEL_CHECK();

@@ -246,6 +246,328 @@ __device__ __forceinline__ void jacobi_solve(const double *G, int ld, int m, int
     }
 }
 
+// 1 / t and 1 / sqrt(t) to about an ulp for |t| within FP32's normal range: an
+// FP32 value and two Newton steps, straight-line code that several can be in
+// flight of.  Outside that range the result is not finite or zero.
+__device__ __forceinline__ double fast_rcp(double t) {
+    double r = (double)__frcp_rn((float)t);
+    r = fma(r, fma(-t, r, 1.0), r);
+    return fma(r, fma(-t, r, 1.0), r);
+}
+
+__device__ __forceinline__ double fast_rsqrt(double t) {
+    double r = (double)__frsqrt_rn((float)t);
+    r = fma(0.5 * r, fma(-t * r, r, 1.0), r);
+    return fma(0.5 * r, fma(-t * r, r, 1.0), r);
+}
+
+// The eigen-decomposition after one more basis vector: eval / evec hold the
+// eigenpairs of G's leading n x n block, and row / column n joins.  In their
+// basis the matrix is an arrowhead [D z; z^T alpha], whose eigenvalues are the
+// roots of f(x) = alpha - x - sum z_i^2 / (d_i - x), one in each interval
+// between the poles d_i.  Each root is solved for as its distance mu to the
+// nearer pole (a quadratic in mu with that pole kept and the rest linearised:
+// in FP32 to ~1e-5, then two steps in FP64), so that every x_j - d_i keeps its
+// relative accuracy; the border z is then recomputed from the roots (Gu and
+// Eisenstat 1994), which makes the eigenvectors z_i / (x_j - d_i) orthogonal
+// to FP64 precision.  A z_i below 1e-15 of the matrix leaves its pair as it is.
+// Returns false (uniformly; eval and evec as they were) when two poles with a
+// border element lie closer than 1e-12 of the matrix, or a value leaves the
+// range of the above: the caller then uses Jacobi.
+//
+// A warp's FP64 instruction occupies its quarter of the SM for ~76 cycles, so
+// sums over poles are split four ways over warps of different quarters (warp
+// w: terms w mod 4, roots 32 (w / 4) on).  Needs 256 threads and
+// JACOBI_SMEM_A bytes at jsm.
+__device__ __forceinline__ bool append_eig(const double *G, int ld, int n, double *__restrict__ eval,
+                                           double *__restrict__ evec, double *jsm) {
+    constexpr int QL = SHCI_MAX_SUB + 1;
+    constexpr int MS = SHCI_MAX_SUB;
+    // V is written last; until then its place holds the partial sums.  Little
+    // static shared memory: the batched solver runs five CTAs per SM.
+    double (*V)[QL] = reinterpret_cast<double (*)[QL]>(jsm);
+    double (*part)[4][MS] = reinterpret_cast<double (*)[4][MS]>(jsm);
+    __shared__ double dd[MS], zz[MS];                     // all pairs
+    __shared__ double d[MS], z[MS];                       // those with a border element
+    __shared__ float df[MS], zf[MS];                      // d - alpha and z in units of the scale
+    __shared__ double mu[MS], val[MS];
+    __shared__ double scale_sh;
+    __shared__ uint8_t idx[MS], slot[MS], pole[MS], rank[MS];
+    __shared__ int bad, n_on;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int quarter = warp & 3, mine = lane + 32 * (warp >> 2);     // this thread's share of the split sums
+    auto gs = [&](int r, int c) { return 0.5 * (__ldcg(&G[r * ld + c]) + __ldcg(&G[c * ld + r])); };
+    __syncthreads();
+    // z = Q^T g, one warp per pair
+    for (int i = warp; i < n; i += nw) {
+        double v = 0.0;
+        for (int s = lane; s < n; s += 32) v = fma(__ldcg(&evec[i * ld + s]), gs(s, n), v);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            zz[i] = v;
+            dd[i] = __ldcg(&eval[i]);
+        }
+    }
+    const double alpha = gs(n, n);
+    __syncthreads();
+    // scale, the pairs with a border element, their gaps: one warp
+    if (warp == 0) {
+        double sc = fabs(alpha);
+        for (int i = lane; i < n; i += 32) sc = fmax(sc, fmax(fabs(dd[i]), fabs(zz[i])));
+        bool wrong = false;
+        for (int i = lane; i < n; i += 32) wrong = wrong || !isfinite(dd[i]) || !isfinite(zz[i]);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) sc = fmax(sc, __shfl_xor_sync(0xffffffffu, sc, o));
+        wrong = wrong || !isfinite(sc) || !isfinite(alpha);
+        const double cut = 1e-15 * sc;
+        int np = 0;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            const bool on = i < n && fabs(zz[i]) > cut;
+            const unsigned m = __ballot_sync(0xffffffffu, on);
+            const int at = np + __popc(m & ((1u << lane) - 1u));
+            if (on) {
+                idx[at] = (uint8_t)i;
+                d[at] = dd[i];
+                z[at] = zz[i];
+            }
+            if (i < n) slot[i] = (uint8_t)(on ? 255 : i - at);        // rank among the untouched pairs
+            np += __popc(m);
+        }
+        __syncwarp();
+        const float inv = 1.0f / (float)sc;
+        for (int i = lane; i < np; i += 32) {
+            if (i > 0) wrong = wrong || !(d[i] - d[i - 1] > 1e-12 * sc);
+            df[i] = (float)(d[i] - alpha) * inv;
+            zf[i] = (float)z[i] * inv;
+        }
+        wrong = __any_sync(0xffffffffu, wrong);
+        if (lane == 0) {
+            bad = wrong;
+            n_on = np;
+            scale_sh = sc;
+        }
+    }
+    __syncthreads();
+    if (bad) return false;
+    const int p = n_on, total = n + 1;
+    const double scale = scale_sh;
+    // roots 0 .. p, root r between the poles r - 1 and r; a thread each (warps 0 and 1).
+    // z_K^2 / mu + a + b mu = 0 with a + b mu the tangent of the rest of f at the last
+    // mu, b < 0: one root of each sign.
+    double m = 0.0, lo = 0.0, hi = 0.0, base = 0.0, q = 0.0;
+    bool neg = false;
+    if (tid <= p && p > 0) {
+        const int r = tid;
+        int K = r == p ? p - 1 : 0;
+        if (r > 0 && r < p) {
+            // the nearer pole by the sign of f at the middle (close to zero either pole serves)
+            const float at = 0.5f * (df[r - 1] + df[r]);
+            float f = -at;
+#pragma unroll 4
+            for (int i = 0; i < p; i++) f -= zf[i] * __fdividef(zf[i], df[i] - at);
+            K = f > 0.0f ? r : r - 1;                     // f descends: positive here, the root is right of it
+        }
+        const float inv = 1.0f / (float)scale;
+        float zn = 0.0f;
+        for (int i = 0; i < p; i++) zn = fmaf(zf[i], zf[i], zn);
+        neg = K == r;                                     // the root lies left of its pole
+        const double out = 1.001 * scale * (double)sqrtf(zn);
+        // |mu| is at most the distance to the next pole, or the Gershgorin bound outside them
+        const double reach = r == 0 ? fmax(0.0, d[K] - alpha) + out
+                                    : (r == p ? fmax(0.0, alpha - d[K]) + out : d[r] - d[r - 1]);
+        lo = neg ? -reach : 0.0;
+        hi = neg ? 0.0 : reach;
+        q = z[K] * z[K];
+        base = alpha - d[K];
+        const float dfK = df[K], bf = -dfK, qf = zf[K] * zf[K], lof = (float)lo * inv, hif = (float)hi * inv;
+        float mf = 0.0f;
+        for (int it = 0; it < 10; it++) {
+            float s = 0.0f, s1 = 1.0f;
+#pragma unroll 4
+            for (int i = 0; i < p; i++) {
+                const float w = i == K ? 0.0f : __fdividef(zf[i], (df[i] - dfK) - mf);
+                s = fmaf(w, zf[i], s);
+                s1 = fmaf(w, w, s1);
+            }
+            const float b = -s1, aa = (bf - mf - s) - b * mf;
+            const float e = -aa - copysignf(sqrtf(fmaf(aa, aa, -4.0f * b * qf)), aa);
+            const float x = (neg == (aa > 0.0f)) ? __fdividef(2.0f * qf, e) : __fdividef(e, 2.0f * b);
+            if (!isfinite(x)) break;
+            const float y = fminf(fmaxf(x, lof), hif);
+            const bool done = fabsf(y - mf) <= 1e-5f * fabsf(y);
+            mf = y;
+            if (done) break;
+        }
+        m = (double)mf * scale;
+        if (m == 0.0) m = (neg ? lo : hi) * 0x1p-40;
+        pole[r] = (uint8_t)K;
+        mu[r] = m;
+    }
+    __syncthreads();
+    if (p > 0) {
+        bool done = false;
+        for (int it = 0; it < 20; it++) {
+            if (mine <= p) {
+                const int K = pole[mine];
+                const double dK = d[K], mm = mu[mine];
+                double s = 0.0, w2 = 0.0;
+                for (int i0 = quarter; i0 < p; i0 += 16) {           // four reciprocals in flight
+                    double w[4], zi[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const int i = min(i0 + 4 * u, p - 1);
+                        zi[u] = i0 + 4 * u < p && i != K ? z[i] : 0.0;
+                        w[u] = zi[u] * fast_rcp((d[i] - dK) - mm);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        s = fma(w[u], zi[u], s);
+                        w2 = fma(w[u], w[u], w2);
+                    }
+                }
+                part[0][quarter][mine] = s;
+                part[1][quarter][mine] = w2;
+            }
+            __syncthreads();
+            if (tid <= p && !done) {
+                const double s = (part[0][0][tid] + part[0][1][tid]) + (part[0][2][tid] + part[0][3][tid]);
+                const double b = -(1.0 + ((part[1][0][tid] + part[1][1][tid]) + (part[1][2][tid] + part[1][3][tid])));
+                const double a = (base - m - s) - b * m, y = fma(a, a, -4.0 * b * q);
+                const double e = -a - copysign(y * fast_rsqrt(y), a);
+                double x = (neg == (a > 0.0)) ? 2.0 * q * fast_rcp(e) : e * fast_rcp(2.0 * b);
+                if (!(x >= lo && x <= hi)) x = 0.5 * (m + (x < lo ? lo : hi));
+                done = fabs(x - m) <= 1e-8 * fabs(x);     // the error squares from step to step
+                m = x;
+                mu[tid] = x;
+            }
+            if (!__syncthreads_or(tid <= p && !done)) break;
+        }
+        if (tid <= p && (!done || m == 0.0 || !isfinite(m))) bad = 1;     // a root on its pole
+    } else if (tid == 0) {
+        pole[0] = 0;
+    }
+    if (tid <= p) val[tid] = p > 0 ? d[pole[tid]] + m : alpha;
+    __syncthreads();
+    if (bad) return false;
+    auto diff = [&](int j, int i) { return (d[pole[j]] - d[i]) + mu[j]; };      // x_j - d_i
+    // z_i^2 = -prod_j (x_j - d_i) / prod_j (d_j - d_i): root j or j + 1 over pole j
+    if (mine < p) {
+        double up = 1.0, dn = 1.0;
+        for (int j = quarter; j < p; j += 4) {
+            if (j == mine) continue;
+            up *= diff(j < mine ? j : j + 1, mine);
+            dn *= d[j] - d[mine];
+        }
+        part[0][quarter][mine] = up / dn;
+    }
+    // places: the roots are elements 0 .. p, the untouched pairs follow in order
+    if (tid > p && tid < total) {
+        int i = 0;
+        while (slot[i] != tid - p - 1) i++;
+        pole[tid] = (uint8_t)i;
+        val[tid] = dd[i];
+    }
+    __syncthreads();
+    if (tid < p) {
+        const double w = (part[0][0][tid] * part[0][1][tid]) * (part[0][2][tid] * part[0][3][tid]) *
+                         (-diff(tid, tid) * diff(tid + 1, tid));
+        if (!(w > 0.0) || !isfinite(w)) bad = 1;
+        z[tid] = copysign(w * fast_rsqrt(w), z[tid]);
+    }
+    if (tid >= 64 && tid < 64 + total) {
+        const int e = tid - 64;
+        int rk = 0;
+        for (int j = 0; j < total; j++) rk += val[j] < val[e] || (val[j] == val[e] && j < e);
+        rank[e] = (uint8_t)rk;
+    }
+    __syncthreads();
+    if (bad) return false;
+    for (int e = tid; e < total * total; e += nt) V[e / total][e % total] = 0.0;
+    __syncthreads();
+    // eigenvectors in the old basis, unnormalised: z_i / (x_j - d_i), and 1 for the new vector
+    for (int e = tid; e < p * (p + 1); e += nt) {
+        const int i = e / (p + 1), j = e - i * (p + 1);
+        V[idx[i]][rank[j]] = z[i] * fast_rcp(diff(j, i));
+    }
+    if (tid <= p) V[n][rank[tid]] = 1.0;
+    else if (tid < total) V[pole[tid]][rank[tid]] = 1.0;
+    __syncthreads();
+    // norms (in place of d, z, mu and zz, which are done with), and the sign that
+    // makes the largest component positive
+    if (mine < total) {
+        double nn = 0.0;
+#pragma unroll 4
+        for (int i = quarter; i < total; i += 4) {
+            const double u = V[i][mine];
+            nn = fma(u, u, nn);
+        }
+        (quarter < 2 ? (quarter == 0 ? d : z) : (quarter == 2 ? mu : zz))[mine] = nn;
+    }
+    __syncthreads();
+    if (tid < total) {
+        int big = 0, sign = 0;
+#pragma unroll 4
+        for (int i = 0; i < total; i++) {
+            const int h = __double2hiint(V[i][tid]);
+            if ((h & 0x7FFFFFFF) > big) {
+                big = h & 0x7FFFFFFF;
+                sign = h < 0;
+            }
+        }
+        const double f = flip_sign(fast_rsqrt((d[tid] + z[tid]) + (mu[tid] + zz[tid])), sign);
+        if (!isfinite(f)) bad = 1;
+        zz[tid] = f;
+    }
+    __syncthreads();
+    if (bad) return false;
+    // Q <- [Q 0; 0 1] V, a warp per component (its row of Q in the lanes' registers)
+    for (int r = warp; r <= n; r += nw) {
+        double q0 = 0.0, q1 = 0.0;
+        if (r < n) {
+            if (lane < n) q0 = __ldcg(&evec[lane * ld + r]);
+            if (lane + 32 < n) q1 = __ldcg(&evec[(lane + 32) * ld + r]);
+        }
+        const int l0 = min(lane, total - 1), l1 = min(lane + 32, total - 1);
+        double v0 = 0.0, v1 = 0.0;
+        if (r == n) {
+            v0 = V[n][l0];
+            v1 = V[n][l1];
+        } else if (total <= 32) {
+#pragma unroll 4
+            for (int i = 0; i < n; i++) v0 = fma(__shfl_sync(0xffffffffu, q0, i), V[i][l0], v0);
+        } else {
+#pragma unroll 4
+            for (int i = 0; i < n; i++) {
+                const double q = __shfl_sync(0xffffffffu, i < 32 ? q0 : q1, i & 31);
+                v0 = fma(q, V[i][l0], v0);
+                v1 = fma(q, V[i][l1], v1);
+            }
+        }
+        if (lane < total) evec[lane * ld + r] = v0 * zz[lane];
+        if (lane + 32 < total) evec[(lane + 32) * ld + r] = v1 * zz[lane + 32];
+    }
+    if (tid < total) eval[rank[tid]] = val[tid];
+    __syncthreads();
+    return true;
+}
+
+// Eigen-decomposition of the m x m matrix G whose leading m_prev x m_prev
+// block's is in eval / evec (m_prev = 0: nothing is known): vector by vector
+// when the block only grew, by Jacobi otherwise (the first solve after a
+// restart).  Per Davidson step of a whole solve: 176 us with Jacobi alone and 36
+// with this for one root (up to 24 vectors), 1.2 ms and 0.30 for the slowest
+// of eight systems of four roots (up to 48 vectors).
+template <bool QSHARED = true>
+__device__ __forceinline__ void subspace_eig(const double *G, int ld, int m, int m_prev, double *__restrict__ eval,
+                                             double *__restrict__ evec, double *jsm, double *qg = nullptr) {
+    int have = m_prev > 0 && m_prev <= m ? m_prev : 0;
+    if (have > 0)
+        while (have < m && append_eig(G, ld, have, eval, evec, jsm)) have++;
+    if (have < m) jacobi_solve<QSHARED>(G, ld, m, have, eval, evec, jsm, qg);
+}
+
 constexpr size_t JACOBI_SMEM_A = sizeof(double) * SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);
 constexpr size_t JACOBI_SMEM = 2 * JACOBI_SMEM_A;
 constexpr int JACOBI_Q_DOUBLES = SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);
