@@ -1366,6 +1366,7 @@ int shci_batch_create(shci_ctx *ctx, int n_sys, const shci_system_desc *systems,
             S.ea.item_first = c->item_a_first.p;
             S.ea.n_items = c->n_items_a;
             S.ea.accumulate = 0;
+            S.ea.by_words = 0;              // one pass over the alpha groups does the opposite-spin doubles too
             S.eb = shci::enum_args(c);
             S.eb.item_group = c->item_b_group.p;
             S.eb.item_first = c->item_b_first.p;

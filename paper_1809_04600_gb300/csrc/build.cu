@@ -197,16 +197,19 @@ __global__ void k_new_start(const uint64_t *__restrict__ keys, const uint32_t *_
     }
 }
 
-// incremental update: row lengths and the offsets of the two new parts of each
-// row (old elements first, then the beta-grouped and alpha-grouped new ones)
+// incremental update: row lengths and the offsets of the three new parts of each
+// row (old elements first, then the beta-grouped, alpha-grouped and
+// opposite-spin new ones)
 __global__ void k_extend_rows(const int64_t *__restrict__ old_rowptr, int64_t n_old, const int64_t *__restrict__ cnt_b,
-                              const int64_t *__restrict__ cnt_a, int64_t n, int64_t *__restrict__ len,
-                              int64_t *__restrict__ off_b, int64_t *__restrict__ off_a) {
+                              const int64_t *__restrict__ cnt_a, const int64_t *__restrict__ cnt_o, int64_t n,
+                              int64_t *__restrict__ len, int64_t *__restrict__ off_b, int64_t *__restrict__ off_a,
+                              int64_t *__restrict__ off_o) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t old = i < n_old ? old_rowptr[i + 1] - old_rowptr[i] : 0;
         off_b[i] = old;
         off_a[i] = old + cnt_b[i];
-        len[i] = old + cnt_b[i] + cnt_a[i];
+        off_o[i] = old + cnt_b[i] + cnt_a[i];
+        len[i] = old + cnt_b[i] + cnt_a[i] + cnt_o[i];
     }
 }
 
@@ -303,12 +306,18 @@ __global__ void k_diag(const uint64_t *__restrict__ dets, int64_t n, DevInts I, 
 
 // (kernels in enumerate.cuh)
 
-__global__ void k_add_i64(int64_t *__restrict__ a, const int64_t *__restrict__ b, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[i] += b[i];
+// a row's parts (beta-grouped, alpha-grouped, opposite-spin) to the offsets of
+// the second and third and the row's length
+__global__ void k_row_parts(const int64_t *__restrict__ cnt_b, int64_t *__restrict__ cnt_ab, int64_t *__restrict__ cnt,
+                            int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t ab = cnt_b[i] + cnt_ab[i];
+        cnt_ab[i] = ab;
+        cnt[i] += ab;
+    }
 }
 
-static void make_items(shci_ctx *c, const int64_t *off, int64_t n_groups, DevBuf<int32_t> &item_group,
+static void make_items(shci_ctx *c, const int64_t *off, int64_t n_groups, int chunk, DevBuf<int32_t> &item_group,
                        DevBuf<int32_t> &item_first, int64_t &n_items) {
     cudaStream_t st = c->st;
     DevBuf<int64_t> cnt, start, tmp;
@@ -316,14 +325,14 @@ static void make_items(shci_ctx *c, const int64_t *off, int64_t n_groups, DevBuf
     start.alloc((size_t)n_groups + 1);
     tmp.alloc((size_t)scan_tmp_len(n_groups + 1));
     unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n_groups, 256), 4096));
-    k_items_count<<<g, 256, 0, st>>>(off, n_groups, cnt.p);
+    k_items_count<<<g, 256, 0, st>>>(off, n_groups, chunk, cnt.p);
     exclusive_scan<int64_t>(cnt.p, start.p, n_groups, tmp.p, st);
     CUDA_TRY(cudaMemcpyAsync(&n_items, start.p + n_groups, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
     if (n_items > 0x7FFFFFFFll) throw ShciError{SHCI_ERR_INVALID, "too many work items"};
     item_group.alloc((size_t)std::max<int64_t>(n_items, 1));
     item_first.alloc((size_t)std::max<int64_t>(n_items, 1));
-    k_items_fill<<<g, 256, 0, st>>>(off, start.p, n_groups, item_group.p, item_first.p);
+    k_items_fill<<<g, 256, 0, st>>>(off, start.p, n_groups, chunk, item_group.p, item_first.p);
     KERNEL_CHECK();
     g_kernel_launches += 2;
 }
@@ -370,6 +379,17 @@ static void extend_pass(shci_ctx *c, EnumArgs E, const DevInts &I, bool alpha_pa
     E.row_det = rdet;
     E.row_str = rstr;
     launch_enum<W, MODE, 0>(c, E, I, alpha_part);
+}
+
+template <int W, int MODE>
+static void extend_opposite(shci_ctx *c, EnumArgs E, const DevInts &I, const PartItems &items, const int32_t *rdet) {
+    if (items.n == 0) return;
+    E.item_group = items.group.p;
+    E.item_first = items.first.p;
+    E.item_end = items.end.p;
+    E.n_items = items.n;
+    E.row_det = rdet;
+    launch_opposite<W, MODE, 0>(c, E, I);
 }
 
 // ====================================================================== host pipeline
@@ -422,6 +442,65 @@ static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf
                                                    sidx.p);
     KERNEL_CHECK();
     LAUNCHED(3);
+}
+
+// determinants per string
+__global__ void k_string_counts(const int32_t *__restrict__ sidx, int64_t n, uint32_t *__restrict__ cnt) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        atomicAdd(&cnt[sidx[i]], 1u);
+}
+
+// keys that ascend as the counts descend
+__global__ void k_count_keys(const uint32_t *__restrict__ cnt, int64_t U, uint32_t top, uint64_t *__restrict__ keys) {
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < U; u += (int64_t)gridDim.x * blockDim.x)
+        keys[u] = top - cnt[u];
+}
+
+// string order[r] gets number r
+template <int W>
+__global__ void k_renumber(const uint32_t *__restrict__ order, int64_t U, const uint64_t *__restrict__ old,
+                           uint64_t *__restrict__ str, uint32_t *__restrict__ number) {
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < U; r += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t u = order[r];
+#pragma unroll
+        for (int w = 0; w < W; w++) str[r * W + w] = old[(int64_t)u * W + w];
+        number[u] = (uint32_t)r;
+    }
+}
+
+__global__ void k_apply_number(const uint32_t *__restrict__ number, int64_t n, int32_t *__restrict__ sidx) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        sidx[i] = (int32_t)number[sidx[i]];
+}
+
+// Number the unique strings by decreasing number of determinants (ties as
+// before, ascending): a group's members then fill few words of the bitmaps
+// over the other spin's numbers, and the enumeration's largest work items come
+// first.
+template <int W>
+static void number_by_size(shci_ctx *c, int64_t U, DevBuf<uint64_t> &ustr, DevBuf<int32_t> &sidx) {
+    const int64_t n = c->n_det;
+    cudaStream_t st = c->st;
+    if (U <= 1) return;
+    DevBuf<uint32_t> cnt, order, number;
+    DevBuf<uint64_t> keys, str;
+    cnt.alloc((size_t)U);
+    order.alloc((size_t)U);
+    number.alloc((size_t)U);
+    keys.alloc((size_t)U);
+    str.alloc((size_t)U * W);
+    CUDA_TRY(cudaMemsetAsync(cnt.p, 0, sizeof(uint32_t) * U, st));
+    k_string_counts<<<grid_for(n), 256, 0, st>>>(sidx.p, n, cnt.p);
+    const uint64_t top = composite_mask(0, n + 1) & 0xFFFFFFFFull;       // at least n, all ones
+    k_count_keys<<<grid_for(U), 256, 0, st>>>(cnt.p, U, (uint32_t)top, keys.p);
+    KERNEL_CHECK();
+    radix_sort<1>(keys.p, order.p, U, c->sw, st, &top, RS_POSITION);
+    k_renumber<W><<<grid_for(U), 256, 0, st>>>(order.p, U, ustr.p, str.p, number.p);
+    k_apply_number<<<grid_for(n), 256, 0, st>>>(number.p, n, sidx.p);
+    KERNEL_CHECK();
+    LAUNCHED(4);
+    ustr.swap(str);
+    CUDA_TRY(cudaStreamSynchronize(st));
 }
 
 template <int W>
@@ -537,6 +616,134 @@ __global__ void k_occ_prefix(const unsigned long long *__restrict__ occ, int64_t
 }
 
 
+// flag[p] = 1 when member p (members sorted by group, then beta index) is the
+// first of its group in its 64-bit word
+__global__ void k_word_heads(const int32_t *__restrict__ mdet, int64_t m, const int32_t *__restrict__ ia,
+                             const int32_t *__restrict__ ib, int64_t *__restrict__ flag) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t d = mdet[p];
+        int64_t f = 1;
+        if (p > 0) {
+            const int32_t e = mdet[p - 1];
+            f = ia[d] != ia[e] || (ib[d] >> 6) != (ib[e] >> 6);
+        }
+        flag[p] = f;
+    }
+}
+
+__global__ void k_word_fill(const int32_t *__restrict__ mdet, int64_t m, const int32_t *__restrict__ ia,
+                            const int32_t *__restrict__ ib, const int64_t *__restrict__ pos,
+                            unsigned long long *__restrict__ word, int2 *__restrict__ info) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x) {
+        if (pos[p + 1] == pos[p]) continue;
+        const int32_t d = mdet[p];
+        const int w = ib[d] >> 6;
+        unsigned long long x = 1ull << (ib[d] & 63);
+        for (int64_t q = p + 1; q < m && pos[q + 1] == pos[q]; q++) x |= 1ull << (ib[mdet[q]] & 63);
+        word[pos[p]] = x;
+        info[pos[p]] = make_int2(w, (int)p);
+    }
+}
+
+// first word of each group (member offsets to word offsets)
+__global__ void k_word_off(const int64_t *__restrict__ off, int64_t n_groups, const int64_t *__restrict__ pos,
+                           int64_t *__restrict__ woff) {
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g <= n_groups; g += (int64_t)gridDim.x * blockDim.x)
+        woff[g] = pos[off[g]];
+}
+
+// The word list of m members sorted by alpha group (offsets off[Ua + 1]), then
+// by beta index.
+static void make_words(shci_ctx *c, const int64_t *off, const int32_t *mdet, int64_t m, WordList &L) {
+    cudaStream_t st = c->st;
+    L.off.alloc((size_t)c->Ua + 1);
+    if (m == 0) {
+        CUDA_TRY(cudaMemsetAsync(L.off.p, 0, sizeof(int64_t) * (c->Ua + 1), st));
+        L.word.alloc(1);
+        L.info.alloc(1);
+        return;
+    }
+    c->i64a.alloc((size_t)m + 1);
+    c->i64b.alloc((size_t)m + 1);
+    c->i64c.alloc((size_t)scan_tmp_len(m + 1));
+    k_word_heads<<<grid_for(m), 256, 0, st>>>(mdet, m, c->ia.p, c->ib.p, c->i64a.p);
+    exclusive_scan<int64_t>(c->i64a.p, c->i64b.p, m, c->i64c.p, st);
+    int64_t words = 0;
+    CUDA_TRY(cudaMemcpyAsync(&words, c->i64b.p + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    L.word.alloc((size_t)words);
+    L.info.alloc((size_t)words);
+    k_word_fill<<<grid_for(m), 256, 0, st>>>(mdet, m, c->ia.p, c->ib.p, c->i64b.p, L.word.p, L.info.p);
+    k_word_off<<<grid_for(c->Ua + 1), 256, 0, st>>>(off, c->Ua, c->i64b.p, L.off.p);
+    KERNEL_CHECK();
+    LAUNCHED(3);
+}
+
+// dense bitmap of each beta string's singles
+__global__ void k_singles_set(const int64_t *__restrict__ off, const int32_t *__restrict__ idx, int64_t U, int64_t words,
+                              unsigned long long *__restrict__ bm) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < U;
+         b += ((int64_t)gridDim.x * blockDim.x) >> 5)
+        for (int64_t e = off[b] + lane; e < off[b + 1]; e += 32)
+            atomicOr(&bm[b * words + (idx[e] >> 6)], 1ull << (idx[e] & 63));
+}
+
+// entries before each word: off[b] + set bits of b's earlier words
+__global__ void k_singles_prefix(const int64_t *__restrict__ off, int64_t U, int64_t words,
+                                 const unsigned long long *__restrict__ bm, int32_t *__restrict__ pref) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < U;
+         b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        int run = (int)off[b];
+        for (int64_t w0 = 0; w0 < words; w0 += 32) {
+            const int64_t w = w0 + lane;
+            const int c = w < words ? __popcll(bm[b * words + w]) : 0;
+            const int incl = warp_incl_scan(c);
+            if (w < words) pref[b * words + w] = run + incl - c;
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+}
+
+// the beta part of every single kb -> b, at its place in bitmap order
+template <int W>
+__global__ void k_singles_info(const int64_t *__restrict__ off, const int32_t *__restrict__ idx, int64_t U, int64_t words,
+                               const unsigned long long *__restrict__ bm, const int32_t *__restrict__ pref,
+                               const uint64_t *__restrict__ str, uint32_t *__restrict__ info) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < U;
+         b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const Str<W> sb = load_str<W>(str, b);
+        for (int64_t e = off[b] + lane; e < off[b + 1]; e += 32) {
+            const int kb = idx[e];
+            int rs, neg;
+            move_info<W>(sb, load_str<W>(str, kb), rs, neg);
+            const int64_t at = b * words + (kb >> 6);
+            info[pref[at] + __popcll(bm[at] & ((1ull << (kb & 63)) - 1ull))] = ((uint32_t)rs << 1) | (uint32_t)(neg & 1);
+        }
+    }
+}
+
+template <int W>
+static void opposite_words(shci_ctx *c) {
+    cudaStream_t st = c->st;
+    const size_t cells = (size_t)(c->Ub * c->occ_words);
+    c->sbm.alloc(cells);
+    c->sbp.alloc(cells);
+    c->bs_info.alloc((size_t)std::max<int64_t>(c->n_beta_singles, 1));
+    CUDA_TRY(cudaMemsetAsync(c->sbm.p, 0, sizeof(unsigned long long) * cells, st));
+    const unsigned g = grid_for(c->Ub * 32);
+    k_singles_set<<<g, 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->occ_words, c->sbm.p);
+    k_singles_prefix<<<g, 256, 0, st>>>(c->bs_off.p, c->Ub, c->occ_words, c->sbm.p, c->sbp.p);
+    k_singles_info<W><<<g, 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->occ_words, c->sbm.p, c->sbp.p, c->bstr.p,
+                                         c->bs_info.p);
+    KERNEL_CHECK();
+    LAUNCHED(3);
+    make_words(c, c->ga_off.p, c->ga_det.p, c->n_det, c->ow);
+    c->opp_words = true;
+}
+
 // Beta-single lists and the occupancy bitmap for the opposite-spin doubles.
 // SHCI_OPP_SPIN=scan: no bitmap, every alpha single's group is scanned;
 // lookup: every (alpha single, beta single) pair is looked up; auto (default):
@@ -553,6 +760,10 @@ static void opposite_spin_setup(shci_ctx *c) {
     std::string pref = env ? env : "auto";
     c->opp_lookup = false;
     c->opp_hybrid = false;
+    c->opp_words = false;
+    c->sbm.reset();
+    c->sbp.reset();
+    c->bs_info.reset();
     if (pref == "scan" || bytes > 4.0e9) {
         c->occ.reset();
         c->occ_pref.reset();
@@ -572,6 +783,8 @@ static void opposite_spin_setup(shci_ctx *c) {
     const char *fenv = getenv("SHCI_OPP_FACTOR");
     c->opp_factor = fenv ? (float)atof(fenv) : 0.5f;
     if (!(c->opp_factor >= 0.0f)) c->opp_factor = 0.5f;
+    if (pref != "lookup" && (double)c->Ub * c->occ_words * 12.0 <= 4.0e9 && c->n_beta_singles <= 0x7FFFFFFFll)
+        opposite_words<W>(c);
 }
 
 // SHCI_AUTO: store both triangles of H when their nnz_full elements (12 bytes
@@ -612,6 +825,8 @@ static void lists_w(shci_ctx *c) {
 
     unique_strings<W>(c, 0, c->astr, c->ia, c->Ua);
     unique_strings<W>(c, 1, c->bstr, c->ib, c->Ub);
+    number_by_size<W>(c, c->Ua, c->astr, c->ia);
+    number_by_size<W>(c, c->Ub, c->bstr, c->ib);
     group_by<W>(c, c->ia.p, c->ib.p, c->Ua, c->Ub, 1, c->ga_off, c->ga_det, c->ga_str);
     group_by<W>(c, c->ib.p, c->ia.p, c->Ub, c->Ua, 0, c->gb_off, c->gb_det, c->gb_str);
     CUDA_TRY(cudaMemcpyAsync(&flags, c->counter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -627,8 +842,9 @@ static void lists_w(shci_ctx *c) {
     LAUNCHED(1);
 
     // work items: chunks of ENUM_NW rows of one alpha (beta) group
-    make_items(c, c->ga_off.p, c->Ua, c->item_a_group, c->item_a_first, c->n_items_a);
-    make_items(c, c->gb_off.p, c->Ub, c->item_b_group, c->item_b_first, c->n_items_b);
+    make_items(c, c->ga_off.p, c->Ua, ENUM_NW, c->item_a_group, c->item_a_first, c->n_items_a);
+    make_items(c, c->gb_off.p, c->Ub, ENUM_NW, c->item_b_group, c->item_b_first, c->n_items_b);
+    if (c->opp_words) make_items(c, c->ga_off.p, c->Ua, OPP_ROWS, c->item_o_group, c->item_o_first, c->n_items_o);
 }
 
 // count pass: entries of the beta-grouped part and of the alpha-grouped part
@@ -651,10 +867,15 @@ static void count_w(shci_ctx *c, bool upper) {
     A.cnt = c->cnt_b.p;
     if (upper) launch_enum<W, ENUM_COUNT_UP, 0>(c, A, I, false);
     else launch_enum<W, ENUM_COUNT, 0>(c, A, I, false);
-    A.cnt = c->i64a.p;
+    c->cnt_ab.alloc((size_t)n);
+    A.cnt = c->cnt_ab.p;
     if (upper) launch_enum<W, ENUM_COUNT_UP, 0>(c, A, I, true);
     else launch_enum<W, ENUM_COUNT, 0>(c, A, I, true);
-    k_add_i64<<<grid_for(n), 256, 0, st>>>(c->i64a.p, c->cnt_b.p, n);
+    A.cnt = c->i64a.p;
+    if (!c->opp_words) CUDA_TRY(cudaMemsetAsync(c->i64a.p, 0, sizeof(int64_t) * n, st));
+    else if (upper) launch_opposite<W, ENUM_COUNT_UP, 0>(c, A, I);
+    else launch_opposite<W, ENUM_COUNT, 0>(c, A, I);
+    k_row_parts<<<grid_for(n), 256, 0, st>>>(c->cnt_b.p, c->cnt_ab.p, c->i64a.p, n);
     KERNEL_CHECK();
     LAUNCHED(1);
     exclusive_scan<int64_t>(c->i64a.p, c->rowptr.p, n, c->i64c.p, st);
@@ -690,6 +911,11 @@ static void store_w(shci_ctx *c, int mode) {
     A.part_off = c->cnt_b.p;
     if (upper) launch_enum<W, ENUM_FILL_UP, 0>(c, A, I, true);
     else launch_enum<W, ENUM_FILL, 0>(c, A, I, true);
+    if (c->opp_words) {
+        A.part_off = c->cnt_ab.p;
+        if (upper) launch_opposite<W, ENUM_FILL_UP, 0>(c, A, I);
+        else launch_opposite<W, ENUM_FILL, 0>(c, A, I);
+    }
     CUDA_TRY(cudaStreamSynchronize(c->st));
 }
 
@@ -718,6 +944,34 @@ void store(shci_ctx *c, int mode) {
     if (c->W == 1) store_w<1>(c, mode);
     else store_w<2>(c, mode);
     c->built = true;
+}
+
+// the new members of the alpha groups, in the groups' order: flags, then places
+__global__ void k_new_flags(const int32_t *__restrict__ mdet, int64_t n, int64_t n_old, int64_t *__restrict__ flag) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
+        flag[p] = mdet[p] >= n_old;
+}
+
+__global__ void k_new_members(const int32_t *__restrict__ mdet, int64_t n, const int64_t *__restrict__ pos,
+                              int32_t *__restrict__ out) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
+        if (pos[p + 1] != pos[p]) out[pos[p]] = mdet[p];
+}
+
+static void new_members(shci_ctx *c, int64_t n_old, DevBuf<int64_t> &off, DevBuf<int32_t> &mdet) {
+    cudaStream_t st = c->st;
+    const int64_t n = c->n_det;
+    c->i64a.alloc((size_t)n + 1);
+    c->i64b.alloc((size_t)n + 1);
+    c->i64c.alloc((size_t)scan_tmp_len(n + 1));
+    off.alloc((size_t)c->Ua + 1);
+    mdet.alloc((size_t)std::max<int64_t>(n - n_old, 1));
+    k_new_flags<<<grid_for(n), 256, 0, st>>>(c->ga_det.p, n, n_old, c->i64a.p);
+    exclusive_scan<int64_t>(c->i64a.p, c->i64b.p, n, c->i64c.p, st);
+    k_new_members<<<grid_for(n), 256, 0, st>>>(c->ga_det.p, n, c->i64b.p, mdet.p);
+    k_word_off<<<grid_for(c->Ua + 1), 256, 0, st>>>(c->ga_off.p, c->Ua, c->i64b.p, off.p);
+    KERNEL_CHECK();
+    LAUNCHED(3);
 }
 
 // Incremental update after V grew from n_old determinants (Sec. III,
@@ -784,15 +1038,28 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     Ao.n_old = n_old;
     Ao.ga_new = ga_new.p;
     Ao.gb_new = gb_new.p;
+    // and the words of the new members alone
+    WordList new_words;
+    DevBuf<int32_t> new_det;
+    if (c->opp_words) {
+        new_members(c, n_old, off_tmp, new_det);
+        make_words(c, off_tmp.p, new_det.p, n - n_old, new_words);
+        Ao.ow_off = new_words.off.p;
+        Ao.ow_word = new_words.word.p;
+        Ao.ow_info = new_words.info.p;
+        Ao.ow_det = new_det.p;
+    }
 
     pm.mark(1);
     // count pass: new elements of each row, beta-grouped and alpha-grouped
     DevBuf<unsigned long long> cand;
     cand.alloc(1);
     CUDA_TRY(cudaMemsetAsync(cand.p, 0, sizeof(unsigned long long), st));
-    DevBuf<int64_t> cnt_a, len, off_a, off_b, rowptr;
+    DevBuf<int64_t> cnt_a, cnt_o, len, off_a, off_b, off_o, rowptr;
     c->cnt_b.alloc((size_t)n);
     cnt_a.alloc((size_t)n);
+    cnt_o.alloc((size_t)n);
+    off_o.alloc((size_t)n);
     len.alloc((size_t)n + 1);
     off_a.alloc((size_t)n);
     off_b.alloc((size_t)n);
@@ -807,7 +1074,14 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     An.cnt = Ao.cnt = cnt_a.p;
     extend_pass<W, ENUM_COUNT_INC>(c, An, I, true, ia_new, gad.p, gas.p);
     extend_pass<W, ENUM_COUNT_INC>(c, Ao, I, true, ia_old, gad.p, gas.p);
-    k_extend_rows<<<grid_for(n), 256, 0, st>>>(c->rowptr.p, n_old, c->cnt_b.p, cnt_a.p, n, len.p, off_b.p, off_a.p);
+    An.cnt = Ao.cnt = cnt_o.p;
+    CUDA_TRY(cudaMemsetAsync(cnt_o.p, 0, sizeof(int64_t) * n, st));
+    if (c->opp_words) {
+        extend_opposite<W, ENUM_COUNT_INC>(c, An, I, ia_new, gad.p);
+        extend_opposite<W, ENUM_COUNT_INC>(c, Ao, I, ia_old, gad.p);
+    }
+    k_extend_rows<<<grid_for(n), 256, 0, st>>>(c->rowptr.p, n_old, c->cnt_b.p, cnt_a.p, cnt_o.p, n, len.p, off_b.p,
+                                               off_a.p, off_o.p);
     KERNEL_CHECK();
     LAUNCHED(1);
     exclusive_scan<int64_t>(len.p, rowptr.p, n, c->i64c.p, st);
@@ -849,6 +1123,11 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
         An.part_off = Ao.part_off = off_a.p;
         extend_pass<W, ENUM_FILL_INC>(c, An, I, true, ia_new, gad.p, gas.p);
         extend_pass<W, ENUM_FILL_INC>(c, Ao, I, true, ia_old, gad.p, gas.p);
+        if (c->opp_words) {
+            An.part_off = Ao.part_off = off_o.p;
+            extend_opposite<W, ENUM_FILL_INC>(c, An, I, ia_new, gad.p);
+            extend_opposite<W, ENUM_FILL_INC>(c, Ao, I, ia_old, gad.p);
+        }
         c->col.swap(col);
         c->val.swap(val);
     } else {

@@ -33,6 +33,14 @@ struct HBList {
     int64_t entries = 0;
 };
 
+// Nonzero 64-bit words of the bitmaps over beta indices of each alpha group's
+// members: off[Ua + 1], the words, and each word's index and first member.
+struct WordList {
+    DevBuf<int64_t> off;
+    DevBuf<unsigned long long> word;
+    DevBuf<int2> info;
+};
+
 struct shci_ctx {
     int device = 0;
     cudaStream_t st = nullptr;
@@ -75,10 +83,19 @@ struct shci_ctx {
     bool opp_lookup = false;               // the occupancy bitmap is built
     bool opp_hybrid = false;               // scan or look up per alpha single
     float opp_factor = 0.5f;               // scan a group of up to this many x the beta singles
+    // opposite-spin doubles by bitmap words (opposite.cuh)
+    bool opp_words = false;
+    WordList ow;
+    DevBuf<unsigned long long> sbm;        // [Ub][occ_words] beta-singles bitmap
+    DevBuf<int32_t> sbp;                   // [Ub][occ_words] entries of bs_info before each word
+    DevBuf<uint32_t> bs_info;              // per beta single in bitmap order: pair index << 1 | sign
+    DevBuf<int32_t> item_o_group, item_o_first;
+    int64_t n_items_o = 0;
     // enumeration work items: chunks of rows of one alpha (beta) group
     DevBuf<int32_t> item_a_group, item_a_first, item_b_group, item_b_first;
     int64_t n_items_a = 0, n_items_b = 0;
     DevBuf<int64_t> cnt_b;                 // entries of the beta-grouped part of each row (build scratch)
+    DevBuf<int64_t> cnt_ab;                // and of the beta- and alpha-grouped parts
 
     // stored H, both triangles, diagonal separate; after an incremental
     // update a row holds its old elements first, then the new ones

@@ -80,6 +80,20 @@ struct EnumArgs {
     const unsigned long long *occ;          // [Ua][occ_words] occupancy bitmap over (alpha, beta)
     const int32_t *occ_pref;                // [Ua][occ_words] set bits before each word in its row
     int64_t occ_words;
+    // opposite-spin doubles by bitmap words (opposite.cuh) instead of in the
+    // alpha-grouped pass: nonzero words of each alpha group's members (word,
+    // its index and its first member's position in ow_det), the dense bitmap
+    // of each beta string's singles with the entries before each word, and per
+    // entry the beta part of the element (pair index << 1 | sign)
+    int by_words;
+    const int64_t *ow_off;
+    const unsigned long long *ow_word;
+    const int2 *ow_info;
+    const int32_t *ow_det;
+    const unsigned long long *sbm;
+    const int32_t *sbp;
+    int64_t sb_words;
+    const uint32_t *bs_info;
     const int32_t *item_group;              // work item -> group index
     const int32_t *item_first;              // work item -> first member offset within the group
     int64_t n_items;
@@ -509,7 +523,7 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
         if (valid) {
             const int64_t n_beg = A.ga_new[a];
             old_row_suffix<W, MODE, K>(R, A, I, Q, Bi, Ai, A.ga_str, A.ga_det, n_beg, g_beg + g_len, cand_local);
-            const int64_t s_beg = A.as_off[a], s_end = A.as_off[a + 1];
+            const int64_t s_beg = A.as_off[a], s_end = A.by_words ? s_beg : A.as_off[a + 1];
             for (int64_t s0 = s_beg; s0 < s_end; s0 += 32) {
                 // one alpha single per lane: its group's new members and pair context
                 int64_t kb = 0;
@@ -581,6 +595,10 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
             }
         }
         __syncthreads();
+    }
+    if (A.by_words) {                       // the opposite-spin doubles have a pass of their own
+        row_end<W, MODE, K>(R, A, I, Q, Bi, Ai, i, valid);
+        return;
     }
     // opposite-spin doubles: candidates in the groups of the alpha singles of a,
     // found by scanning each group k (tiles shared by the CTA's warps) or by
@@ -787,19 +805,20 @@ __global__ void __launch_bounds__(ENUM_THREADS, EnumMinBlocks<MODE>::value) k_en
     if (ModeOf<MODE>::count && (threadIdx.x & 31) == 0 && cand_local) atomicAdd(A.cand, cand_local);
 }
 
-// work items: one per chunk of ENUM_NW members of each group
-static __global__ void k_items_count(const int64_t *__restrict__ off, int64_t n_groups, int64_t *__restrict__ cnt) {
+// work items: one per chunk of `chunk` members of each group
+static __global__ void k_items_count(const int64_t *__restrict__ off, int64_t n_groups, int chunk,
+                                     int64_t *__restrict__ cnt) {
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x)
-        cnt[g] = (off[g + 1] - off[g] + ENUM_NW - 1) / ENUM_NW;
+        cnt[g] = (off[g + 1] - off[g] + chunk - 1) / chunk;
 }
 
 static __global__ void k_items_fill(const int64_t *__restrict__ off, const int64_t *__restrict__ start, int64_t n_groups,
-                                    int32_t *__restrict__ item_group, int32_t *__restrict__ item_first) {
+                                    int chunk, int32_t *__restrict__ item_group, int32_t *__restrict__ item_first) {
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x) {
-        int64_t c = (off[g + 1] - off[g] + ENUM_NW - 1) / ENUM_NW;
+        int64_t c = (off[g + 1] - off[g] + chunk - 1) / chunk;
         for (int64_t t = 0; t < c; t++) {
             item_group[start[g] + t] = (int32_t)g;
-            item_first[start[g] + t] = (int32_t)(t * ENUM_NW);
+            item_first[start[g] + t] = (int32_t)(t * chunk);
         }
     }
 }

@@ -229,8 +229,9 @@ void sigma(shci_ctx *c, int k, const double *x, double *y, bool inter) {
 // On-the-fly sigma (the "direct" method the paper proposes for larger spaces,
 // Sec. VIII): every product re-enumerates the connected pairs with the helper
 // lists and recomputes H_ij, so H is never stored.  Pass 1 (rows grouped by
-// alpha string) writes y = diag * x + same-spin-beta and opposite-spin terms;
-// pass 2 (rows grouped by beta string) adds the same-spin-alpha terms.
+// alpha string) writes y = diag * x + same-spin-beta terms, pass 2 adds the
+// opposite-spin terms (opposite.cuh; without its bitmaps pass 1 does), pass 3
+// (rows grouped by beta string) the same-spin-alpha terms.
 template <int W, int K>
 static void otf_k(shci_ctx *c, const double *x, double *y) {
     EnumArgs A = enum_args(c);
@@ -240,6 +241,7 @@ static void otf_k(shci_ctx *c, const double *x, double *y) {
     DevInts I = dev_ints(c);
     A.accumulate = 0;
     launch_enum<W, ENUM_SIGMA, K>(c, A, I, true);
+    if (c->opp_words) launch_opposite<W, ENUM_SIGMA, K>(c, A, I);
     A.accumulate = 1;
     launch_enum<W, ENUM_SIGMA, K>(c, A, I, false);
 }
