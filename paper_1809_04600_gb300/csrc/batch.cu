@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(BT, MINB) k_batch_davidson(BatchArgs B) {
                 if (a < m) S.G[(m + q) * S.m_max + a] = v;   // the new corner: one writer per entry
             }
             __syncthreads();
-            subspace_eig<false>(S.G, S.m_max, mt, st.m_eig, S.eval, S.evec, sh, S.jq);
+            subspace_eig<false, false>(S.G, S.m_max, mt, st.m_eig, S.eval, S.evec, sh, S.jq);
             __syncthreads();
             if (tid == 0) {
                 st.m = mt;

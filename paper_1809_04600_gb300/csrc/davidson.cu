@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(DV_THREADS) k_ritz(const double *__restrict__ 
 __global__ void k_jacobi(const double *__restrict__ G, int ld, int m, int m_prev, double *__restrict__ eval,
                          double *__restrict__ evec) {
     extern __shared__ double jsm[];
-    subspace_eig(G, ld, m, m_prev, eval, evec, jsm);
+    subspace_eig<true, true>(G, ld, m, m_prev, eval, evec, jsm);
 }
 
 // ---------------------------------------------------------------- start vectors

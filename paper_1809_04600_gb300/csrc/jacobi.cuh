@@ -553,19 +553,191 @@ __device__ __forceinline__ bool append_eig(const double *G, int ld, int n, doubl
     return true;
 }
 
+// Signs of the eigenvectors.  An eigenvector's sign is free, but a caller that
+// follows a root from call to call relies on it not changing with the method,
+// and the Jacobi iteration's is the outcome of all its rotations.  So those are
+// carried out, on the bordered matrix in the old eigenvectors' basis, in FP32
+// and without the rotations too small to matter for a sign (angles below
+// 1e-4): X holds the eigenvectors they lead to, ~1e-5 accurate, by columns.
+// FP32 runs at 75 times the FP64 rate, so this takes a third of the FP64
+// iteration's time.  A, Qf: 64 x 65 floats each in shared memory; X overwrites A.
+__device__ __forceinline__ void jacobi_signs(const double *G, int ld, int m, int mp, const double *eval,
+                                             const double *evec, float (*A)[SHCI_MAX_SUB + 1],
+                                             float (*Qf)[SHCI_MAX_SUB + 1]) {
+    __shared__ float cs[SHCI_MAX_SUB / 2], sn[SHCI_MAX_SUB / 2];
+    __shared__ uint8_t pp[SHCI_MAX_SUB / 2], qq[SHCI_MAX_SUB / 2], act[SHCI_MAX_SUB / 2];
+    __shared__ int8_t pos[SHCI_MAX_SUB / 2];
+    __shared__ int n_act[2];
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int mm = (m + 1) & ~1, half = mm / 2;
+    auto gs = [&](int r, int c) { return 0.5 * (__ldcg(&G[r * ld + c]) + __ldcg(&G[c * ld + r])); };
+    const double shift = __ldcg(&eval[0]);
+    __syncthreads();
+    for (int e = tid; e < mm * mm; e += nt) {
+        const int r = e / mm, c = e % mm;
+        float v = 0.0f;
+        if (r == c) v = r < mp ? (float)(__ldcg(&eval[r]) - shift) : (r < m ? (float)(gs(r, r) - shift) : 3.0e18f);
+        else if (r >= mp && c >= mp && r < m && c < m) v = (float)gs(r, c);
+        A[r][c] = v;
+        Qf[r][c] = r == c ? 1.0f : 0.0f;
+    }
+    __syncthreads();
+    // the border in the old basis, a warp per entry
+    for (int e = warp; e < mp * (m - mp); e += nw) {
+        const int i = e % mp, c = mp + e / mp;
+        double v = 0.0;
+        for (int s = lane; s < mp; s += 32) v = fma(__ldcg(&evec[i * ld + s]), gs(s, c), v);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            A[i][c] = (float)v;
+            A[c][i] = (float)v;
+        }
+    }
+    __syncthreads();
+    for (int sweep = 0; sweep < 10; sweep++) {
+        bool some = false;                                // a sweep without rotations is not made
+        for (int e = tid; e < mm * mm; e += nt) {
+            const int p = e / mm, q = e - p * mm;
+            const float apq = fabsf(A[p][q]);
+            some = some || (p < q && apq > 1e-4f * fabsf(A[q][q] - A[p][p]) && apq > 1e-30f);
+        }
+        if (!__syncthreads_or(some)) break;               // uniform
+        int xr = tid, yr = mm - 1 - tid;                  // the pairs and order of jacobi_solve
+        for (int round = 0; round < mm - 1; round++) {
+            if (tid < 32) {
+                int active = 0;
+                if (tid < half) {
+                    int p = xr, q = yr;
+                    if (p > q) { const int t = p; p = q; q = t; }
+                    if (tid > 0 && ++xr == mm) xr = 1;
+                    if (++yr == mm) yr = 1;
+                    const float apq = A[p][q], diff = A[q][q] - A[p][p];
+                    float c = 1.0f, s = 0.0f;
+                    if (fabsf(apq) > 1e-4f * fabsf(diff)) {
+                        active = fabsf(apq) > 1e-30f;
+                        const float tau = diff / (2.0f * apq);
+                        const float t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
+                        c = rsqrtf(1.0f + t * t);
+                        s = t * c;
+                    }
+                    cs[tid] = c;
+                    sn[tid] = s;
+                    pp[tid] = (uint8_t)p;
+                    qq[tid] = (uint8_t)q;
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, active);
+                const int at = __popc(mask & ((1u << tid) - 1u));
+                if (active) act[at] = (uint8_t)tid;
+                if (tid < half) pos[tid] = (int8_t)(active ? at : -1);
+                if (tid == 0) n_act[round & 1] = __popc(mask);
+            }
+            __syncthreads();
+            const int na = n_act[round & 1];
+            if (na == 0) continue;                        // uniform
+            for (int e = tid; e < na * half; e += nt) {
+                const int x = e / half, u = e - x * half, t = act[x], pu = pos[u];
+                if (pu >= 0 && pu < x) continue;
+                const int p = pp[t], q = qq[t], r = pp[u], v = qq[u];
+                const float ct = cs[t], st = sn[t];
+                const float cu = pu >= 0 ? cs[u] : 1.0f, su = pu >= 0 ? sn[u] : 0.0f;
+                const float apr = A[p][r], apv = A[p][v], aqr = A[q][r], aqv = A[q][v];
+                const float bpr = ct * apr - st * aqr, bpv = ct * apv - st * aqv;
+                const float bqr = st * apr + ct * aqr, bqv = st * apv + ct * aqv;
+                const float npr = cu * bpr - su * bpv, npv = su * bpr + cu * bpv;
+                const float nqr = cu * bqr - su * bqv, nqv = su * bqr + cu * bqv;
+                if (t == u) {
+                    A[p][p] = npr;
+                    A[q][q] = nqv;
+                    A[p][q] = npv;
+                    A[q][p] = npv;
+                } else {
+                    A[p][r] = npr;
+                    A[p][v] = npv;
+                    A[q][r] = nqr;
+                    A[q][v] = nqv;
+                    A[r][p] = npr;
+                    A[v][p] = npv;
+                    A[r][q] = nqr;
+                    A[v][q] = nqv;
+                }
+            }
+            for (int e = tid; e < mm * na; e += nt) {
+                const int i = e / na, t = act[e - i * na], p = pp[t], q = qq[t];
+                const float c = cs[t], s = sn[t], qp = Qf[i][p], qv = Qf[i][q];
+                Qf[i][p] = c * qp - s * qv;
+                Qf[i][q] = s * qp + c * qv;
+            }
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    // X = [evec 0; 0 1] Qf
+    for (int e = tid; e < m * m; e += nt) {
+        const int r = e / m, c = e % m;
+        float v = 0.0f;
+        if (r >= mp) {
+            v = Qf[r][c];
+        } else {
+            for (int i = 0; i < mp; i++) v = fmaf((float)__ldcg(&evec[i * ld + r]), Qf[i][c], v);
+        }
+        A[r][c] = v;
+    }
+    __syncthreads();
+}
+
+// the sign of each new eigenvector is that of the column of X it is nearest to
+__device__ __forceinline__ void apply_signs(int ld, int m, double *__restrict__ evec,
+                                            const float (*X)[SHCI_MAX_SUB + 1]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    for (int l = warp; l < m; l += nw) {
+        const float e0 = lane < m ? (float)__ldcg(&evec[l * ld + lane]) : 0.0f;
+        const float e1 = lane + 32 < m ? (float)__ldcg(&evec[l * ld + lane + 32]) : 0.0f;
+        float d0 = 0.0f, d1 = 0.0f;                       // against columns lane and lane + 32
+        const int c0 = min(lane, m - 1), c1 = min(lane + 32, m - 1);
+        for (int r = 0; r < m; r++) {
+            const float e = __shfl_sync(0xffffffffu, r < 32 ? e0 : e1, r & 31);
+            d0 = fmaf(e, X[r][c0], d0);
+            d1 = fmaf(e, X[r][c1], d1);
+        }
+        float best = fabsf(d0) >= fabsf(d1) ? d0 : d1;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            const float y = __shfl_xor_sync(0xffffffffu, best, o);
+            if (fabsf(y) > fabsf(best)) best = y;
+        }
+        if (best < 0.0f) {
+            if (lane < m) evec[l * ld + lane] = -__ldcg(&evec[l * ld + lane]);
+            if (lane + 32 < m) evec[l * ld + lane + 32] = -__ldcg(&evec[l * ld + lane + 32]);
+        }
+    }
+    __syncthreads();
+}
+
 // Eigen-decomposition of the m x m matrix G whose leading m_prev x m_prev
 // block's is in eval / evec (m_prev = 0: nothing is known): vector by vector
 // when the block only grew, by Jacobi otherwise (the first solve after a
-// restart).  Per Davidson step of a whole solve: 176 us with Jacobi alone and 36
-// with this for one root (up to 24 vectors), 1.2 ms and 0.30 for the slowest
-// of eight systems of four roots (up to 48 vectors).
-template <bool QSHARED = true>
+// restart).  SIGNS: with the signs of the Jacobi iteration (jsm: JACOBI_SMEM
+// bytes); a batch returns energies only and does without.  Per Davidson step
+// of a whole solve: 176 us with Jacobi alone and 88 with this, 52 of it for the
+// signs, for one root (up to 24 vectors), 1.2 ms and 0.30 for the slowest of
+// eight batched systems of four roots (up to 48 vectors, no signs).
+template <bool QSHARED, bool SIGNS>
 __device__ __forceinline__ void subspace_eig(const double *G, int ld, int m, int m_prev, double *__restrict__ eval,
                                              double *__restrict__ evec, double *jsm, double *qg = nullptr) {
-    int have = m_prev > 0 && m_prev <= m ? m_prev : 0;
-    if (have > 0)
-        while (have < m && append_eig(G, ld, have, eval, evec, jsm)) have++;
+    const int old = m_prev > 0 && m_prev <= m ? m_prev : 0;
+    int have = old;
+    if (have == 0 || have == m) {
+        jacobi_solve<QSHARED>(G, ld, m, have, eval, evec, jsm, qg);
+        return;
+    }
+    typedef float (*Rows)[SHCI_MAX_SUB + 1];
+    Rows X = reinterpret_cast<Rows>(jsm + SHCI_MAX_SUB * (SHCI_MAX_SUB + 1));     // behind append_eig's matrix
+    if (SIGNS) jacobi_signs(G, ld, m, old, eval, evec, X, reinterpret_cast<Rows>(jsm));
+    while (have < m && append_eig(G, ld, have, eval, evec, jsm)) have++;
     if (have < m) jacobi_solve<QSHARED>(G, ld, m, have, eval, evec, jsm, qg);
+    else if (SIGNS) apply_signs(ld, m, evec, X);
 }
 
 constexpr size_t JACOBI_SMEM_A = sizeof(double) * SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);
