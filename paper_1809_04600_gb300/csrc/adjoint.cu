@@ -81,7 +81,10 @@ static void backward_w(shci_ctx *c, const double *cv, double *gdh, double *geri,
     A.geri_len = eri_len;
     DevInts I = dev_ints(c);
     launch_enum<W, ENUM_GRAD, 1>(c, A, I, true);
-    if (c->opp_words) launch_opposite<W, ENUM_GRAD, 1>(c, A, I);
+    if (c->opp_pass) {
+        group_vectors(c, A, 1);
+        launch_opposite<W, ENUM_GRAD, 1>(c, A, I);
+    }
     launch_enum<W, ENUM_GRAD, 1>(c, A, I, false);
 }
 

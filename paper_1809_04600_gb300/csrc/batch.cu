@@ -418,7 +418,7 @@ __device__ void diag_rows(const BSys &S, int nb, int64_t r0, int cnt) {
 // registers allocated apart from the rest of the persistent kernel.
 __device__ __noinline__ void batch_alpha_item(const BSys &S, int64_t local, EnumSmem<1> &es, int nb) {
     unsigned long long cand = 0;
-    enum_alpha_item<1, ENUM_SIGMA, BK>(S.ea, S.I, local, es.T, es.Q[threadIdx.x >> 5], cand, nb);
+    enum_alpha_item<1, ENUM_SIGMA, BK, true>(S.ea, S.I, local, es.T, es.Q[threadIdx.x >> 5], cand, nb);
 }
 
 __device__ __noinline__ void batch_beta_item(const BSys &S, int64_t local, EnumSmem<1> &es, int nb) {
@@ -1331,6 +1331,7 @@ int shci_batch_create(shci_ctx *ctx, int n_sys, const shci_system_desc *systems,
             c->device = ctx->device;
             c->st = ctx->st;
             c->own_stream = false;
+            c->batch_member = true;
             c->n_sm = ctx->n_sm;
             CUDA_TRY(cudaEventCreate(&c->ev0));
             CUDA_TRY(cudaEventCreate(&c->ev1));
@@ -1366,7 +1367,6 @@ int shci_batch_create(shci_ctx *ctx, int n_sys, const shci_system_desc *systems,
             S.ea.item_first = c->item_a_first.p;
             S.ea.n_items = c->n_items_a;
             S.ea.accumulate = 0;
-            S.ea.by_words = 0;              // one pass over the alpha groups does the opposite-spin doubles too
             S.eb = shci::enum_args(c);
             S.eb.item_group = c->item_b_group.p;
             S.eb.item_first = c->item_b_first.p;

@@ -8,6 +8,7 @@
 #include <numeric>
 
 #include "enum_launch.cuh"
+#include "move_tables.cuh"
 
 std::atomic<long long> g_kernel_launches{0};
 #define LAUNCHED(n) (g_kernel_launches += (n))
@@ -75,6 +76,7 @@ void load_integrals(shci_ctx *c, int n_orb, double e_core, const double *h, cons
     c->e_core = e_core;
     c->have_ints = true;
     c->hb_valid = false;
+    c->have_moves = false;
 }
 
 DevInts dev_ints(const shci_ctx *c) {
@@ -141,13 +143,15 @@ __global__ void k_head_flags(const uint64_t *__restrict__ keys, int64_t n, int64
 template <int W>
 __global__ void k_unique_write(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ vals,
                                const int64_t *__restrict__ flags, const int64_t *__restrict__ excl, int64_t n,
-                               uint64_t *__restrict__ ustr, int32_t *__restrict__ sidx) {
+                               uint64_t *__restrict__ ustr, int32_t *__restrict__ sidx, int32_t *__restrict__ first) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t id = excl[i] + flags[i] - 1;
         if (flags[i]) {
 #pragma unroll
             for (int k = 0; k < W; k++) ustr[id * W + k] = keys[i * W + k];
+            first[id] = (int32_t)i;
         }
+        if (i == n - 1) first[id + 1] = (int32_t)n;
         sidx[vals[i]] = (int32_t)id;
     }
 }
@@ -320,7 +324,7 @@ __global__ void k_row_parts(const int64_t *__restrict__ cnt_b, int64_t *__restri
 static void make_items(shci_ctx *c, const int64_t *off, int64_t n_groups, int chunk, DevBuf<int32_t> &item_group,
                        DevBuf<int32_t> &item_first, int64_t &n_items) {
     cudaStream_t st = c->st;
-    DevBuf<int64_t> cnt, start, tmp;
+    DevBuf<int64_t> &cnt = c->i64a, &start = c->i64b, &tmp = c->i64c;
     cnt.alloc((size_t)n_groups + 1);
     start.alloc((size_t)n_groups + 1);
     tmp.alloc((size_t)scan_tmp_len(n_groups + 1));
@@ -346,14 +350,14 @@ struct PartItems {
 };
 
 static void make_items_part(shci_ctx *c, const int64_t *off, const int64_t *g_new, int64_t n_groups, int part,
-                            PartItems &P) {
+                            int chunk, PartItems &P) {
     cudaStream_t st = c->st;
-    DevBuf<int64_t> cnt, start, tmp;
+    DevBuf<int64_t> &cnt = c->i64a, &start = c->i64b, &tmp = c->i64c;
     cnt.alloc((size_t)n_groups + 1);
     start.alloc((size_t)n_groups + 1);
     tmp.alloc((size_t)scan_tmp_len(n_groups + 1));
     unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n_groups, 256), 4096));
-    k_items_count_part<<<g, 256, 0, st>>>(off, g_new, n_groups, part, cnt.p);
+    k_items_count_part<<<g, 256, 0, st>>>(off, g_new, n_groups, part, chunk, cnt.p);
     exclusive_scan<int64_t>(cnt.p, start.p, n_groups, tmp.p, st);
     CUDA_TRY(cudaMemcpyAsync(&P.n, start.p + n_groups, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -361,7 +365,7 @@ static void make_items_part(shci_ctx *c, const int64_t *off, const int64_t *g_ne
     P.group.alloc((size_t)std::max<int64_t>(P.n, 1));
     P.first.alloc((size_t)std::max<int64_t>(P.n, 1));
     P.end.alloc((size_t)std::max<int64_t>(P.n, 1));
-    k_items_fill_part<<<g, 256, 0, st>>>(off, g_new, start.p, n_groups, part, P.group.p, P.first.p, P.end.p);
+    k_items_fill_part<<<g, 256, 0, st>>>(off, g_new, start.p, n_groups, part, chunk, P.group.p, P.first.p, P.end.p);
     KERNEL_CHECK();
     g_kernel_launches += 2;
 }
@@ -398,7 +402,11 @@ static inline unsigned grid_for(int64_t n, int threads = 256) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, threads), 152 * 32));
 }
 
-// bits a spin string can have set, per word
+// bits a spin string can have set, per word.  A sort of one-word strings takes
+// them as known, which saves the reduction over the keys and its read-back.
+// Strings of two words have more digits, many of them all zero where few
+// orbitals are in use: there the reduction pays (76 orbitals, 1000 strings: 20
+// passes instead of 80 in a growth's four sorts of strings).
 template <int W>
 struct OrbMask {
     uint64_t w[W];
@@ -408,6 +416,7 @@ struct OrbMask {
             w[k] = bits == 64 ? ~0ull : (1ull << bits) - 1;
         }
     }
+    const uint64_t *known() const { return W == 1 ? w : nullptr; }
 };
 
 // bits in which the composite keys (major << 32 | minor) of the given ranges can differ
@@ -428,7 +437,7 @@ static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf
     c->sort_vals.alloc((size_t)n);
     k_extract_strings<W><<<grid_for(n), 256, 0, st>>>(c->dets.p, n, spin, c->sort_keys.p, c->sort_vals.p);
     KERNEL_CHECK();
-    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st, OrbMask<W>(c->n_orb).w);
+    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, n, c->sw, st, OrbMask<W>(c->n_orb).known());
     c->i64a.alloc((size_t)n + 1);
     c->i64b.alloc((size_t)n + 1);
     c->i64c.alloc((size_t)scan_tmp_len(n + 1));
@@ -438,22 +447,18 @@ static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf
     CUDA_TRY(cudaStreamSynchronize(st));
     ustr.alloc((size_t)U * W);
     sidx.alloc((size_t)n);
+    c->i32a.alloc((size_t)U + 1);
     k_unique_write<W><<<grid_for(n), 256, 0, st>>>(c->sort_keys.p, c->sort_vals.p, c->i64a.p, c->i64b.p, n, ustr.p,
-                                                   sidx.p);
+                                                   sidx.p, c->i32a.p);
     KERNEL_CHECK();
     LAUNCHED(3);
 }
 
-// determinants per string
-__global__ void k_string_counts(const int32_t *__restrict__ sidx, int64_t n, uint32_t *__restrict__ cnt) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[sidx[i]], 1u);
-}
-
-// keys that ascend as the counts descend
-__global__ void k_count_keys(const uint32_t *__restrict__ cnt, int64_t U, uint32_t top, uint64_t *__restrict__ keys) {
+// keys that ascend as the strings' determinant counts descend; first: where
+// each string's run begins among the sorted determinants
+__global__ void k_count_keys(const int32_t *__restrict__ first, int64_t U, uint32_t top, uint64_t *__restrict__ keys) {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < U; u += (int64_t)gridDim.x * blockDim.x)
-        keys[u] = top - cnt[u];
+        keys[u] = top - (uint32_t)(first[u + 1] - first[u]);
 }
 
 // string order[r] gets number r
@@ -479,28 +484,21 @@ __global__ void k_apply_number(const uint32_t *__restrict__ number, int64_t n, i
 // first.
 template <int W>
 static void number_by_size(shci_ctx *c, int64_t U, DevBuf<uint64_t> &ustr, DevBuf<int32_t> &sidx) {
+    // right after unique_strings: c->i32a holds the runs' beginnings, the sort buffers are free
     const int64_t n = c->n_det;
     cudaStream_t st = c->st;
     if (U <= 1) return;
-    DevBuf<uint32_t> cnt, order, number;
-    DevBuf<uint64_t> keys, str;
-    cnt.alloc((size_t)U);
-    order.alloc((size_t)U);
-    number.alloc((size_t)U);
-    keys.alloc((size_t)U);
-    str.alloc((size_t)U * W);
-    CUDA_TRY(cudaMemsetAsync(cnt.p, 0, sizeof(uint32_t) * U, st));
-    k_string_counts<<<grid_for(n), 256, 0, st>>>(sidx.p, n, cnt.p);
+    c->u32a.alloc((size_t)U);
+    c->str_tmp.alloc((size_t)U * W);
     const uint64_t top = composite_mask(0, n + 1) & 0xFFFFFFFFull;       // at least n, all ones
-    k_count_keys<<<grid_for(U), 256, 0, st>>>(cnt.p, U, (uint32_t)top, keys.p);
+    k_count_keys<<<grid_for(U), 256, 0, st>>>(c->i32a.p, U, (uint32_t)top, c->sort_keys.p);
     KERNEL_CHECK();
-    radix_sort<1>(keys.p, order.p, U, c->sw, st, &top, RS_POSITION);
-    k_renumber<W><<<grid_for(U), 256, 0, st>>>(order.p, U, ustr.p, str.p, number.p);
-    k_apply_number<<<grid_for(n), 256, 0, st>>>(number.p, n, sidx.p);
+    radix_sort<1>(c->sort_keys.p, c->sort_vals.p, U, c->sw, st, &top, RS_POSITION);
+    k_renumber<W><<<grid_for(U), 256, 0, st>>>(c->sort_vals.p, U, ustr.p, c->str_tmp.p, c->u32a.p);
+    k_apply_number<<<grid_for(n), 256, 0, st>>>(c->u32a.p, n, sidx.p);
     KERNEL_CHECK();
-    LAUNCHED(4);
-    ustr.swap(str);
-    CUDA_TRY(cudaStreamSynchronize(st));
+    LAUNCHED(3);
+    ustr.swap(c->str_tmp);
 }
 
 template <int W>
@@ -567,9 +565,9 @@ static int64_t string_singles(shci_ctx *c, const uint64_t *ustr, int64_t U, int 
     c->sort_vals.alloc((size_t)std::max<int64_t>(nk, c->n_det));
     k_minus_one_keys<W><<<grid_for(U), 256, 0, st>>>(ustr, U, ne, c->sort_keys.p, c->sort_vals.p);
     KERNEL_CHECK();
-    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, nk, c->sw, st, OrbMask<W>(c->n_orb).w);
-    DevBuf<int64_t> seg_start;
-    DevBuf<int32_t> seg_len;
+    radix_sort<W>(c->sort_keys.p, c->sort_vals.p, nk, c->sw, st, OrbMask<W>(c->n_orb).known());
+    DevBuf<int64_t> &seg_start = c->seg_start;
+    DevBuf<int32_t> &seg_len = c->seg_len;
     seg_start.alloc((size_t)nk);
     seg_len.alloc((size_t)nk);
     k_segment_info<W><<<grid_for(nk), 256, 0, st>>>(c->sort_keys.p, c->sort_vals.p, nk, seg_start.p, seg_len.p);
@@ -594,154 +592,77 @@ static void alpha_singles(shci_ctx *c) {
 }
 
 // occupancy bitmap over (unique alpha, unique beta) and, per 64-bit word, the
-// number of set bits before it in its row: the rank of a present (a, b) among
-// the members of alpha group a (sorted by beta index) is its member offset
-__global__ void k_occ_set(const int32_t *__restrict__ ia, const int32_t *__restrict__ ib, int64_t n, int64_t ow,
-                          unsigned long long *__restrict__ occ) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+// place in the alpha-group lists of its first determinant: members of a group
+// are sorted by beta index
+__global__ void k_occ_set(const int32_t *__restrict__ ia, const int32_t *__restrict__ ib, int64_t from, int64_t n,
+                          int64_t ow, OccCell *__restrict__ occ) {
+    for (int64_t i = from + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = ib[i];
-        atomicOr(&occ[(int64_t)ia[i] * ow + (b >> 6)], 1ull << (b & 63));
+        atomicOr(&occ[(int64_t)ia[i] * ow + (b >> 6)].bits, 1ull << (b & 63));
     }
 }
 
-__global__ void k_occ_prefix(const unsigned long long *__restrict__ occ, int64_t Ua, int64_t ow,
-                             int32_t *__restrict__ pref) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < Ua; a += (int64_t)gridDim.x * blockDim.x) {
-        int32_t run = 0;
-        for (int64_t w = 0; w < ow; w++) {
-            pref[a * ow + w] = run;
-            run += __popcll(occ[a * ow + w]);
-        }
-    }
-}
-
-
-// flag[p] = 1 when member p (members sorted by group, then beta index) is the
-// first of its group in its 64-bit word
-__global__ void k_word_heads(const int32_t *__restrict__ mdet, int64_t m, const int32_t *__restrict__ ia,
-                             const int32_t *__restrict__ ib, int64_t *__restrict__ flag) {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t d = mdet[p];
-        int64_t f = 1;
-        if (p > 0) {
-            const int32_t e = mdet[p - 1];
-            f = ia[d] != ia[e] || (ib[d] >> 6) != (ib[e] >> 6);
-        }
-        flag[p] = f;
-    }
-}
-
-__global__ void k_word_fill(const int32_t *__restrict__ mdet, int64_t m, const int32_t *__restrict__ ia,
-                            const int32_t *__restrict__ ib, const int64_t *__restrict__ pos,
-                            unsigned long long *__restrict__ word, int2 *__restrict__ info) {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x) {
-        if (pos[p + 1] == pos[p]) continue;
-        const int32_t d = mdet[p];
-        const int w = ib[d] >> 6;
-        unsigned long long x = 1ull << (ib[d] & 63);
-        for (int64_t q = p + 1; q < m && pos[q + 1] == pos[q]; q++) x |= 1ull << (ib[mdet[q]] & 63);
-        word[pos[p]] = x;
-        info[pos[p]] = make_int2(w, (int)p);
-    }
-}
-
-// first word of each group (member offsets to word offsets)
-__global__ void k_word_off(const int64_t *__restrict__ off, int64_t n_groups, const int64_t *__restrict__ pos,
-                           int64_t *__restrict__ woff) {
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g <= n_groups; g += (int64_t)gridDim.x * blockDim.x)
-        woff[g] = pos[off[g]];
-}
-
-// The word list of m members sorted by alpha group (offsets off[Ua + 1]), then
-// by beta index.
-static void make_words(shci_ctx *c, const int64_t *off, const int32_t *mdet, int64_t m, WordList &L) {
-    cudaStream_t st = c->st;
-    L.off.alloc((size_t)c->Ua + 1);
-    if (m == 0) {
-        CUDA_TRY(cudaMemsetAsync(L.off.p, 0, sizeof(int64_t) * (c->Ua + 1), st));
-        L.word.alloc(1);
-        L.info.alloc(1);
-        return;
-    }
-    c->i64a.alloc((size_t)m + 1);
-    c->i64b.alloc((size_t)m + 1);
-    c->i64c.alloc((size_t)scan_tmp_len(m + 1));
-    k_word_heads<<<grid_for(m), 256, 0, st>>>(mdet, m, c->ia.p, c->ib.p, c->i64a.p);
-    exclusive_scan<int64_t>(c->i64a.p, c->i64b.p, m, c->i64c.p, st);
-    int64_t words = 0;
-    CUDA_TRY(cudaMemcpyAsync(&words, c->i64b.p + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    L.word.alloc((size_t)words);
-    L.info.alloc((size_t)words);
-    k_word_fill<<<grid_for(m), 256, 0, st>>>(mdet, m, c->ia.p, c->ib.p, c->i64b.p, L.word.p, L.info.p);
-    k_word_off<<<grid_for(c->Ua + 1), 256, 0, st>>>(off, c->Ua, c->i64b.p, L.off.p);
-    KERNEL_CHECK();
-    LAUNCHED(3);
-}
-
-// dense bitmap of each beta string's singles
-__global__ void k_singles_set(const int64_t *__restrict__ off, const int32_t *__restrict__ idx, int64_t U, int64_t words,
-                              unsigned long long *__restrict__ bm) {
+__global__ void k_occ_place(const int64_t *__restrict__ off, int64_t Ua, int64_t ow, OccCell *__restrict__ occ) {
     const int lane = threadIdx.x & 31;
-    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < U;
-         b += ((int64_t)gridDim.x * blockDim.x) >> 5)
-        for (int64_t e = off[b] + lane; e < off[b + 1]; e += 32)
-            atomicOr(&bm[b * words + (idx[e] >> 6)], 1ull << (idx[e] & 63));
-}
-
-// entries before each word: off[b] + set bits of b's earlier words
-__global__ void k_singles_prefix(const int64_t *__restrict__ off, int64_t U, int64_t words,
-                                 const unsigned long long *__restrict__ bm, int32_t *__restrict__ pref) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < U;
-         b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        int run = (int)off[b];
-        for (int64_t w0 = 0; w0 < words; w0 += 32) {
+    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < Ua;
+         a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        int run = (int)off[a];
+        for (int64_t w0 = 0; w0 < ow; w0 += 32) {
             const int64_t w = w0 + lane;
-            const int c = w < words ? __popcll(bm[b * words + w]) : 0;
+            const int c = w < ow ? __popcll(occ[a * ow + w].bits) : 0;
             const int incl = warp_incl_scan(c);
-            if (w < words) pref[b * words + w] = run + incl - c;
+            if (w < ow) occ[a * ow + w].place = run + incl - c;
             run += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
 }
 
-// the beta part of every single kb -> b, at its place in bitmap order
+// the bitmap of determinants [from, n), whose members begin at off
+static void occupancy(shci_ctx *c, int64_t from, const int64_t *off, DevBuf<OccCell> &occ) {
+    cudaStream_t st = c->st;
+    const size_t cells = (size_t)(c->Ua * c->occ_words);
+    occ.alloc(cells);
+    CUDA_TRY(cudaMemsetAsync(occ.p, 0, sizeof(OccCell) * cells, st));
+    k_occ_set<<<grid_for(c->n_det - from), 256, 0, st>>>(c->ia.p, c->ib.p, from, c->n_det, c->occ_words, occ.p);
+    k_occ_place<<<grid_for(c->Ua * 32), 256, 0, st>>>(off, c->Ua, c->occ_words, occ.p);
+    KERNEL_CHECK();
+    LAUNCHED(2);
+}
+
+// beta index of each member
+__global__ void k_member_index(const int32_t *__restrict__ mdet, int64_t m, const int32_t *__restrict__ ib,
+                               int32_t *__restrict__ out) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x)
+        out[p] = ib[mdet[p]];
+}
+
+// every single kb -> b: kb, and the beta part of its elements
 template <int W>
-__global__ void k_singles_info(const int64_t *__restrict__ off, const int32_t *__restrict__ idx, int64_t U, int64_t words,
-                               const unsigned long long *__restrict__ bm, const int32_t *__restrict__ pref,
-                               const uint64_t *__restrict__ str, uint32_t *__restrict__ info) {
+__global__ void k_singles_info(const int64_t *__restrict__ off, const int32_t *__restrict__ idx, int64_t U,
+                               const uint64_t *__restrict__ str, int2 *__restrict__ pair) {
     const int lane = threadIdx.x & 31;
     for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < U;
          b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const Str<W> sb = load_str<W>(str, b);
         for (int64_t e = off[b] + lane; e < off[b + 1]; e += 32) {
-            const int kb = idx[e];
             int rs, neg;
-            move_info<W>(sb, load_str<W>(str, kb), rs, neg);
-            const int64_t at = b * words + (kb >> 6);
-            info[pref[at] + __popcll(bm[at] & ((1ull << (kb & 63)) - 1ull))] = ((uint32_t)rs << 1) | (uint32_t)(neg & 1);
+            move_info<W>(sb, load_str<W>(str, idx[e]), rs, neg);
+            pair[e] = make_int2(idx[e], (rs << 1) | (neg & 1));
         }
     }
 }
 
+// what the opposite-spin pass needs beside the bitmap
 template <int W>
-static void opposite_words(shci_ctx *c) {
+static void opposite_pass_setup(shci_ctx *c) {
     cudaStream_t st = c->st;
-    const size_t cells = (size_t)(c->Ub * c->occ_words);
-    c->sbm.alloc(cells);
-    c->sbp.alloc(cells);
-    c->bs_info.alloc((size_t)std::max<int64_t>(c->n_beta_singles, 1));
-    CUDA_TRY(cudaMemsetAsync(c->sbm.p, 0, sizeof(unsigned long long) * cells, st));
-    const unsigned g = grid_for(c->Ub * 32);
-    k_singles_set<<<g, 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->occ_words, c->sbm.p);
-    k_singles_prefix<<<g, 256, 0, st>>>(c->bs_off.p, c->Ub, c->occ_words, c->sbm.p, c->sbp.p);
-    k_singles_info<W><<<g, 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->occ_words, c->sbm.p, c->sbp.p, c->bstr.p,
-                                         c->bs_info.p);
+    c->bs_pair.alloc((size_t)std::max<int64_t>(c->n_beta_singles, 1));
+    c->ga_ib.alloc((size_t)c->n_det);
+    k_singles_info<W><<<grid_for(c->Ub * 32), 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->bstr.p, c->bs_pair.p);
+    k_member_index<<<grid_for(c->n_det), 256, 0, st>>>(c->ga_det.p, c->n_det, c->ib.p, c->ga_ib.p);
     KERNEL_CHECK();
-    LAUNCHED(3);
-    make_words(c, c->ga_off.p, c->ga_det.p, c->n_det, c->ow);
-    c->opp_words = true;
+    LAUNCHED(2);
+    c->opp_pass = true;
 }
 
 // Beta-single lists and the occupancy bitmap for the opposite-spin doubles.
@@ -760,22 +681,14 @@ static void opposite_spin_setup(shci_ctx *c) {
     std::string pref = env ? env : "auto";
     c->opp_lookup = false;
     c->opp_hybrid = false;
-    c->opp_words = false;
-    c->sbm.reset();
-    c->sbp.reset();
-    c->bs_info.reset();
+    c->opp_pass = false;
     if (pref == "scan" || bytes > 4.0e9) {
         c->occ.reset();
-        c->occ_pref.reset();
+        c->bs_pair.reset();
+        c->ga_ib.reset();
         return;
     }
-    c->occ.alloc((size_t)(c->Ua * c->occ_words));
-    c->occ_pref.alloc((size_t)(c->Ua * c->occ_words));
-    CUDA_TRY(cudaMemsetAsync(c->occ.p, 0, sizeof(unsigned long long) * c->Ua * c->occ_words, st));
-    k_occ_set<<<grid_for(c->n_det), 256, 0, st>>>(c->ia.p, c->ib.p, c->n_det, c->occ_words, c->occ.p);
-    k_occ_prefix<<<grid_for(c->Ua), 256, 0, st>>>(c->occ.p, c->Ua, c->occ_words, c->occ_pref.p);
-    KERNEL_CHECK();
-    LAUNCHED(2);
+    occupancy(c, 0, c->ga_off.p, c->occ);
     c->opp_lookup = true;
     c->opp_hybrid = pref != "lookup";
     // the crossover of the per-alpha-single choice (SHCI_OPP_FACTOR overrides):
@@ -783,8 +696,7 @@ static void opposite_spin_setup(shci_ctx *c) {
     const char *fenv = getenv("SHCI_OPP_FACTOR");
     c->opp_factor = fenv ? (float)atof(fenv) : 0.5f;
     if (!(c->opp_factor >= 0.0f)) c->opp_factor = 0.5f;
-    if (pref != "lookup" && (double)c->Ub * c->occ_words * 12.0 <= 4.0e9 && c->n_beta_singles <= 0x7FFFFFFFll)
-        opposite_words<W>(c);
+    if (pref != "lookup") opposite_pass_setup<W>(c);
 }
 
 // SHCI_AUTO: store both triangles of H when their nnz_full elements (12 bytes
@@ -810,6 +722,7 @@ static int64_t stored_entries(const shci_ctx *c) {
 template <int W>
 static void lists_w(shci_ctx *c) {
     cudaStream_t st = c->st;
+    c->have_moves = false;                  // V's strings change
     const int64_t n = c->n_det;
     c->counter.alloc(4);
     CUDA_TRY(cudaMemsetAsync(c->counter.p, 0, 4 * sizeof(int), st));
@@ -824,8 +737,8 @@ static void lists_w(shci_ctx *c) {
     if (flags & 4) throw ShciError{SHCI_ERR_INVALID, "a determinant occupies an orbital >= n_orb"};
 
     unique_strings<W>(c, 0, c->astr, c->ia, c->Ua);
-    unique_strings<W>(c, 1, c->bstr, c->ib, c->Ub);
     number_by_size<W>(c, c->Ua, c->astr, c->ia);
+    unique_strings<W>(c, 1, c->bstr, c->ib, c->Ub);
     number_by_size<W>(c, c->Ub, c->bstr, c->ib);
     group_by<W>(c, c->ia.p, c->ib.p, c->Ua, c->Ub, 1, c->ga_off, c->ga_det, c->ga_str);
     group_by<W>(c, c->ib.p, c->ia.p, c->Ub, c->Ua, 0, c->gb_off, c->gb_det, c->gb_str);
@@ -844,7 +757,37 @@ static void lists_w(shci_ctx *c) {
     // work items: chunks of ENUM_NW rows of one alpha (beta) group
     make_items(c, c->ga_off.p, c->Ua, ENUM_NW, c->item_a_group, c->item_a_first, c->n_items_a);
     make_items(c, c->gb_off.p, c->Ub, ENUM_NW, c->item_b_group, c->item_b_first, c->n_items_b);
-    if (c->opp_words) make_items(c, c->ga_off.p, c->Ua, OPP_ROWS, c->item_o_group, c->item_o_first, c->n_items_o);
+    if (c->opp_pass) {
+        const int rows = opp_item_rows(n, c->n_sm);
+        make_items(c, c->ga_off.p, c->Ua, rows, c->item_o_group, c->item_o_first, c->n_items_o);
+    }
+}
+
+// Tabulate the single moves of V's strings for the passes that evaluate
+// elements, when that is little work beside them: a table entry costs about
+// what a single in full does, a row of V has some ten to thirty, evaluated
+// once to store H and in every product on the fly (but a batch's systems share
+// the memory).  At most a 32nd of the free memory (64 MB in any case).  1e6
+// determinants of 24 orbitals: the same-spin kernels of a product on the fly
+// 4.5 to 1.7 ms each, those that write H 7.9 and 6.3 to 3.6 and 3.9.
+template <int W>
+static void connectivity_moves(shci_ctx *c, int mode) {
+    c->have_moves = false;
+    const double entries = (double)(c->Ua + c->Ub) * c->n_orb * (c->n_orb + 1) / 2;
+    const double per_row = mode == SHCI_ON_THE_FLY && !c->batch_member ? 128.0 : 24.0;
+    bool fits = entries <= per_row * (double)c->n_det;
+    if (fits && entries * 16.0 > 6.4e7) {
+        size_t fr = 0, tot = 0;
+        CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+        fits = entries * 16.0 <= (double)fr / 32.0;
+    }
+    if (!fits) {
+        c->move_a.reset();
+        c->move_b.reset();
+        return;
+    }
+    make_move_tables<W>(c, dev_ints(c), c->move_a, c->move_b);
+    c->have_moves = true;
 }
 
 // count pass: entries of the beta-grouped part and of the alpha-grouped part
@@ -855,7 +798,7 @@ static void count_w(shci_ctx *c, bool upper) {
     cudaStream_t st = c->st;
     const int64_t n = c->n_det;
     DevInts I = dev_ints(c);
-    DevBuf<unsigned long long> cand;
+    DevBuf<unsigned long long> &cand = c->cand;
     cand.alloc(1);
     CUDA_TRY(cudaMemsetAsync(cand.p, 0, sizeof(unsigned long long), st));
     c->rowptr.alloc((size_t)n + 1);
@@ -872,7 +815,7 @@ static void count_w(shci_ctx *c, bool upper) {
     if (upper) launch_enum<W, ENUM_COUNT_UP, 0>(c, A, I, true);
     else launch_enum<W, ENUM_COUNT, 0>(c, A, I, true);
     A.cnt = c->i64a.p;
-    if (!c->opp_words) CUDA_TRY(cudaMemsetAsync(c->i64a.p, 0, sizeof(int64_t) * n, st));
+    if (!c->opp_pass) CUDA_TRY(cudaMemsetAsync(c->i64a.p, 0, sizeof(int64_t) * n, st));
     else if (upper) launch_opposite<W, ENUM_COUNT_UP, 0>(c, A, I);
     else launch_opposite<W, ENUM_COUNT, 0>(c, A, I);
     k_row_parts<<<grid_for(n), 256, 0, st>>>(c->cnt_b.p, c->cnt_ab.p, c->i64a.p, n);
@@ -897,6 +840,7 @@ static void store_w(shci_ctx *c, int mode) {
     const bool upper = mode == SHCI_STORED_UPPER;
     if (c->rows_upper != upper) count_w<W>(c, upper);
     c->mode = mode;
+    if (!c->have_moves) connectivity_moves<W>(c, mode);
     const int64_t nnz = stored_entries(c);
     c->col.alloc((size_t)std::max<int64_t>(nnz, 1));
     c->val.alloc((size_t)std::max<int64_t>(nnz, 1));
@@ -911,7 +855,7 @@ static void store_w(shci_ctx *c, int mode) {
     A.part_off = c->cnt_b.p;
     if (upper) launch_enum<W, ENUM_FILL_UP, 0>(c, A, I, true);
     else launch_enum<W, ENUM_FILL, 0>(c, A, I, true);
-    if (c->opp_words) {
+    if (c->opp_pass) {
         A.part_off = c->cnt_ab.p;
         if (upper) launch_opposite<W, ENUM_FILL_UP, 0>(c, A, I);
         else launch_opposite<W, ENUM_FILL, 0>(c, A, I);
@@ -930,6 +874,7 @@ static void build_w(shci_ctx *c, int mode) {
         c->mode = mode;
         c->col.reset();
         c->val.reset();
+        connectivity_moves<W>(c, mode);
     }
     CUDA_TRY(cudaStreamSynchronize(c->st));
 }
@@ -958,6 +903,13 @@ __global__ void k_new_members(const int32_t *__restrict__ mdet, int64_t n, const
         if (pos[p + 1] != pos[p]) out[pos[p]] = mdet[p];
 }
 
+// group offsets among them
+__global__ void k_part_off(const int64_t *__restrict__ off, int64_t n_groups, const int64_t *__restrict__ pos,
+                           int64_t *__restrict__ out) {
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g <= n_groups; g += (int64_t)gridDim.x * blockDim.x)
+        out[g] = pos[off[g]];
+}
+
 static void new_members(shci_ctx *c, int64_t n_old, DevBuf<int64_t> &off, DevBuf<int32_t> &mdet) {
     cudaStream_t st = c->st;
     const int64_t n = c->n_det;
@@ -969,7 +921,7 @@ static void new_members(shci_ctx *c, int64_t n_old, DevBuf<int64_t> &off, DevBuf
     k_new_flags<<<grid_for(n), 256, 0, st>>>(c->ga_det.p, n, n_old, c->i64a.p);
     exclusive_scan<int64_t>(c->i64a.p, c->i64b.p, n, c->i64c.p, st);
     k_new_members<<<grid_for(n), 256, 0, st>>>(c->ga_det.p, n, c->i64b.p, mdet.p);
-    k_word_off<<<grid_for(c->Ua + 1), 256, 0, st>>>(c->ga_off.p, c->Ua, c->i64b.p, off.p);
+    k_part_off<<<grid_for(c->Ua + 1), 256, 0, st>>>(c->ga_off.p, c->Ua, c->i64b.p, off.p);
     KERNEL_CHECK();
     LAUNCHED(3);
 }
@@ -1020,11 +972,17 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     DevBuf<uint64_t> gas, gbs;
     group_by_index<W>(c, c->ia.p, c->Ua, 1, n_old, off_tmp, gad, gas, ga_new);
     group_by_index<W>(c, c->ib.p, c->Ub, 0, n_old, off_tmp, gbd, gbs, gb_new);
-    PartItems ia_old, ia_new, ib_old, ib_new;
-    make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 0, ia_old);
-    make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 1, ia_new);
-    make_items_part(c, c->gb_off.p, gb_new.p, c->Ub, 0, ib_old);
-    make_items_part(c, c->gb_off.p, gb_new.p, c->Ub, 1, ib_new);
+    PartItems ia_old, ia_new, ib_old, ib_new, io_old, io_new;
+    make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 0, ENUM_NW, ia_old);
+    make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 1, ENUM_NW, ia_new);
+    make_items_part(c, c->gb_off.p, gb_new.p, c->Ub, 0, ENUM_NW, ib_old);
+    make_items_part(c, c->gb_off.p, gb_new.p, c->Ub, 1, ENUM_NW, ib_new);
+    if (c->opp_pass) {
+        const int rows = opp_item_rows(n, c->n_sm);
+        make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 0, rows, io_old);
+        make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 1, rows, io_new);
+    }
+    connectivity_moves<W>(c, c->mode);
     // new rows: every candidate, the context's lists
     EnumArgs An = enum_args(c);
     // old rows: new candidates only, determinant-ordered lists
@@ -1038,21 +996,25 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     Ao.n_old = n_old;
     Ao.ga_new = ga_new.p;
     Ao.gb_new = gb_new.p;
-    // and the words of the new members alone
-    WordList new_words;
-    DevBuf<int32_t> new_det;
-    if (c->opp_words) {
+    // and the opposite-spin pass's view of the new members alone
+    DevBuf<int32_t> new_det, new_ib;
+    DevBuf<OccCell> new_occ;
+    if (c->opp_pass) {
         new_members(c, n_old, off_tmp, new_det);
-        make_words(c, off_tmp.p, new_det.p, n - n_old, new_words);
-        Ao.ow_off = new_words.off.p;
-        Ao.ow_word = new_words.word.p;
-        Ao.ow_info = new_words.info.p;
+        new_ib.alloc((size_t)(n - n_old));
+        k_member_index<<<grid_for(n - n_old), 256, 0, st>>>(new_det.p, n - n_old, c->ib.p, new_ib.p);
+        KERNEL_CHECK();
+        LAUNCHED(1);
+        occupancy(c, n_old, off_tmp.p, new_occ);
+        Ao.ow_off = off_tmp.p;
+        Ao.ow_ib = new_ib.p;
         Ao.ow_det = new_det.p;
+        Ao.occ = new_occ.p;
     }
 
     pm.mark(1);
     // count pass: new elements of each row, beta-grouped and alpha-grouped
-    DevBuf<unsigned long long> cand;
+    DevBuf<unsigned long long> &cand = c->cand;
     cand.alloc(1);
     CUDA_TRY(cudaMemsetAsync(cand.p, 0, sizeof(unsigned long long), st));
     DevBuf<int64_t> cnt_a, cnt_o, len, off_a, off_b, off_o, rowptr;
@@ -1076,9 +1038,9 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     extend_pass<W, ENUM_COUNT_INC>(c, Ao, I, true, ia_old, gad.p, gas.p);
     An.cnt = Ao.cnt = cnt_o.p;
     CUDA_TRY(cudaMemsetAsync(cnt_o.p, 0, sizeof(int64_t) * n, st));
-    if (c->opp_words) {
-        extend_opposite<W, ENUM_COUNT_INC>(c, An, I, ia_new, gad.p);
-        extend_opposite<W, ENUM_COUNT_INC>(c, Ao, I, ia_old, gad.p);
+    if (c->opp_pass) {
+        extend_opposite<W, ENUM_COUNT_INC>(c, An, I, io_new, gad.p);
+        extend_opposite<W, ENUM_COUNT_INC>(c, Ao, I, io_old, gad.p);
     }
     k_extend_rows<<<grid_for(n), 256, 0, st>>>(c->rowptr.p, n_old, c->cnt_b.p, cnt_a.p, cnt_o.p, n, len.p, off_b.p,
                                                off_a.p, off_o.p);
@@ -1123,10 +1085,10 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
         An.part_off = Ao.part_off = off_a.p;
         extend_pass<W, ENUM_FILL_INC>(c, An, I, true, ia_new, gad.p, gas.p);
         extend_pass<W, ENUM_FILL_INC>(c, Ao, I, true, ia_old, gad.p, gas.p);
-        if (c->opp_words) {
+        if (c->opp_pass) {
             An.part_off = Ao.part_off = off_o.p;
-            extend_opposite<W, ENUM_FILL_INC>(c, An, I, ia_new, gad.p);
-            extend_opposite<W, ENUM_FILL_INC>(c, Ao, I, ia_old, gad.p);
+            extend_opposite<W, ENUM_FILL_INC>(c, An, I, io_new, gad.p);
+            extend_opposite<W, ENUM_FILL_INC>(c, Ao, I, io_old, gad.p);
         }
         c->col.swap(col);
         c->val.swap(val);

@@ -232,7 +232,7 @@ __device__ __forceinline__ double hij_offdiag(const DevInts &I, const Str<W> &ai
         int neg = bits_between<W>(common, lo, hi) & 1;
         const double *jk = I.jk1 + (int64_t)(p * n + q) * n;
         const double *jo = I.j1 + (int64_t)(p * n + q) * n;
-        double v = __ldg(&I.h[p * n + q]);
+        double v = __ldg(&I.h[p * n + q]), vo = 0.0;
 #pragma unroll
         for (int k = 0; k < W; k++) {
             uint64_t m = common.w[k];
@@ -245,10 +245,10 @@ __device__ __forceinline__ double hij_offdiag(const DevInts &I, const Str<W> &ai
             while (o) {
                 int b = __ffsll((long long)o) - 1;
                 o &= o - 1;
-                v += __ldg(&jo[64 * k + b]);
+                vo += __ldg(&jo[64 * k + b]);
             }
         }
-        return flip_sign(v, neg);
+        return flip_sign(v + vo, neg);
     }
     if (na == 1 && nb == 1) {
         Str<W> pa, qa, pb, qb;

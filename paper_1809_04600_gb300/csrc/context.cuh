@@ -33,18 +33,15 @@ struct HBList {
     int64_t entries = 0;
 };
 
-// Nonzero 64-bit words of the bitmaps over beta indices of each alpha group's
-// members: off[Ua + 1], the words, and each word's index and first member.
-struct WordList {
-    DevBuf<int64_t> off;
-    DevBuf<unsigned long long> word;
-    DevBuf<int2> info;
-};
+namespace shci {
+struct OccCell;                            // enumerate.cuh
+}
 
 struct shci_ctx {
     int device = 0;
     cudaStream_t st = nullptr;
     bool own_stream = false;
+    bool batch_member = false;             // one of many systems that share the device's memory
     std::string err;
     int n_sm = 0;
 
@@ -77,20 +74,21 @@ struct shci_ctx {
     // beta-single lists and the (alpha, beta) occupancy bitmap for opposite-spin lookups
     DevBuf<int64_t> bs_off;
     DevBuf<int32_t> bs_idx;
-    DevBuf<unsigned long long> occ;
-    DevBuf<int32_t> occ_pref;
+    DevBuf<shci::OccCell> occ;
     int64_t occ_words = 0, n_beta_singles = 0;
     bool opp_lookup = false;               // the occupancy bitmap is built
     bool opp_hybrid = false;               // scan or look up per alpha single
     float opp_factor = 0.5f;               // scan a group of up to this many x the beta singles
-    // opposite-spin doubles by bitmap words (opposite.cuh)
-    bool opp_words = false;
-    WordList ow;
-    DevBuf<unsigned long long> sbm;        // [Ub][occ_words] beta-singles bitmap
-    DevBuf<int32_t> sbp;                   // [Ub][occ_words] entries of bs_info before each word
-    DevBuf<uint32_t> bs_info;              // per beta single in bitmap order: pair index << 1 | sign
+    // opposite-spin doubles in a pass of their own (opposite.cuh)
+    bool opp_pass = false;
+    DevBuf<int32_t> ga_ib;                 // beta index of each alpha group's members
+    DevBuf<int2> bs_pair;                  // beta singles: index, pair index << 1 | sign
+    DevBuf<double> x_grouped;              // vectors of a product in the order of the alpha groups' members
     DevBuf<int32_t> item_o_group, item_o_first;
     int64_t n_items_o = 0;
+    // single moves tabulated per string (move_tables.cuh)
+    bool have_moves = false;
+    DevBuf<double> move_a, move_b;
     // enumeration work items: chunks of rows of one alpha (beta) group
     DevBuf<int32_t> item_a_group, item_a_first, item_b_group, item_b_first;
     int64_t n_items_a = 0, n_items_b = 0;
@@ -109,7 +107,11 @@ struct shci_ctx {
     DevBuf<uint64_t> sort_keys;
     DevBuf<uint32_t> sort_vals;
     DevBuf<int64_t> i64a, i64b, i64c;
-    DevBuf<int32_t> i32a;
+    DevBuf<int32_t> i32a, seg_len;
+    DevBuf<int64_t> seg_start;
+    DevBuf<uint32_t> u32a;
+    DevBuf<uint64_t> str_tmp;
+    DevBuf<unsigned long long> cand;       // candidates screened by a count pass
     DevBuf<int> counter;                   // dynamic work counters / flags
     DevBuf<double> vec_a, vec_b;           // layout conversion for the ABI sigma
 

@@ -25,21 +25,21 @@ inline EnumArgs enum_args(const shci_ctx *c) {
     A.opp_lookup = c->opp_lookup ? 1 : 0;
     A.opp_hybrid = c->opp_hybrid ? 1 : 0;
     A.opp_factor = c->opp_factor;
+    A.ia = c->ia.p;
     A.ib = c->ib.p;
     A.bs_off = c->bs_off.p;
     A.bs_idx = c->bs_idx.p;
     A.occ = c->occ.p;
-    A.occ_pref = c->occ_pref.p;
     A.occ_words = c->occ_words;
-    A.by_words = c->opp_words ? 1 : 0;
-    A.ow_off = c->ow.off.p;
-    A.ow_word = c->ow.word.p;
-    A.ow_info = c->ow.info.p;
+    A.ow_off = c->ga_off.p;
+    A.ow_ib = c->ga_ib.p;
     A.ow_det = c->ga_det.p;
-    A.sbm = c->sbm.p;
-    A.sbp = c->sbp.p;
-    A.sb_words = c->occ_words;
-    A.bs_info = c->bs_info.p;
+    A.n_beta_str = c->Ub;
+    A.opp_rows = opp_item_rows(c->n_det, c->n_sm);
+    A.bs_pair = c->bs_pair.p;
+    A.ma = c->have_moves ? c->move_a.p : nullptr;
+    A.mb = c->have_moves ? c->move_b.p : nullptr;
+    A.n_pair = c->n_orb * (c->n_orb + 1) / 2;
     return A;
 }
 
@@ -54,10 +54,30 @@ void launch_enum(shci_ctx *c, EnumArgs A, const DevInts &I, bool alpha_part) {
         A.n_items = alpha_part ? c->n_items_a : c->n_items_b;
     }
     const int blocks = c->n_sm * (2048 / ENUM_THREADS);
-    if (alpha_part) k_enum_alpha<W, MODE, K><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
+    if (alpha_part && c->opp_pass) k_enum_alpha<W, MODE, K, false><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
+    else if (alpha_part) k_enum_alpha<W, MODE, K, true><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
     else k_enum_beta<W, MODE, K><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
     KERNEL_CHECK();
     g_kernel_launches += 1;
+}
+
+// out[p] = x of the member at place p, k interleaved values each
+static __global__ void k_group_vectors(const int32_t *__restrict__ mdet, int64_t n, int k, const double *__restrict__ x,
+                                       double *__restrict__ out) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * k; e += (int64_t)gridDim.x * blockDim.x)
+        out[e] = __ldg(&x[(int64_t)mdet[e / k] * k + e % k]);
+}
+
+// A.x in the order of the alpha groups' members, for the opposite-spin pass on
+// the fly: a pair's place is then where its coefficient is.
+inline void group_vectors(shci_ctx *c, EnumArgs &A, int k) {
+    const int64_t n = c->n_det;
+    c->x_grouped.alloc((size_t)n * k);
+    const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(n * k, 256), (int64_t)c->n_sm * 16);
+    k_group_vectors<<<blocks, 256, 0, c->st>>>(c->ga_det.p, n, k, A.x, c->x_grouped.p);
+    KERNEL_CHECK();
+    g_kernel_launches += 1;
+    A.x_grouped = c->x_grouped.p;
 }
 
 // The opposite-spin pass (opposite.cuh) over the context's items, or the
@@ -71,9 +91,13 @@ void launch_opposite(shci_ctx *c, EnumArgs A, const DevInts &I) {
         A.n_items = c->n_items_o;
         A.row_det = c->ga_det.p;
     }
-    const int blocks = (int)std::min<int64_t>(A.n_items, (int64_t)c->n_sm * OppMinBlocks<MODE, K>::value);
-    if (blocks == 0) return;
-    k_opposite<W, MODE, K><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
+    if (A.n_items == 0) return;
+    const size_t smem = sizeof(uint32_t) * opp_table(c->Ub);
+    CUDA_TRY(cudaFuncSetAttribute(k_opposite<W, MODE, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_opposite<W, MODE, K>, ENUM_THREADS, smem));
+    const int blocks = (int)std::min<int64_t>(A.n_items, (int64_t)c->n_sm * std::max(per_sm, 1));
+    k_opposite<W, MODE, K><<<blocks, ENUM_THREADS, smem, c->st>>>(A, I);
     KERNEL_CHECK();
     g_kernel_launches += 1;
 }

@@ -2,7 +2,9 @@
 // 1 and 2) with a per-pair action: count, write H_ij (stored H), or
 // accumulate H_ij c_j (on-the-fly sigma).
 //
-// Two kernels cover every pair (i, j), i != j, of one row i exactly once:
+// Two kernels cover every pair (i, j), i != j, of one row i exactly once (three
+// where opposite.cuh's pass takes the opposite-spin doubles, and k_enum_alpha
+// the other pairs of its part):
 //   k_enum_alpha: rows grouped by alpha string a.  Candidates are the
 //     determinants whose alpha string is a itself (same-spin beta
 //     excitations) or one of a's alpha singles k (opposite-spin doubles when
@@ -45,8 +47,26 @@ struct ModeOf {
     static constexpr bool up = MODE == ENUM_COUNT_UP || MODE == ENUM_FILL_UP;
 };
 
-
 constexpr int GRAD_REPLICAS = 32;           // gradient copies that spread the atomics
+
+// One 64-bit word of an alpha group's row of the occupancy bitmap over (alpha,
+// beta) and the place of its first set bit's determinant in the group lists:
+// one 16-byte load answers a lookup.
+struct __align__(16) OccCell {
+    unsigned long long bits;
+    int32_t place;
+    int32_t unused;
+};
+
+// cell w of a row by one load
+__device__ __forceinline__ OccCell occ_load(const OccCell *row, int64_t w) {
+    const int4 v = __ldg(reinterpret_cast<const int4 *>(row + w));
+    OccCell c;
+    c.bits = ((unsigned long long)(unsigned)v.y << 32) | (unsigned)v.x;
+    c.place = v.z;
+    c.unused = 0;
+    return c;
+}
 
 struct EnumArgs {
     const uint64_t *dets;
@@ -74,26 +94,25 @@ struct EnumArgs {
     const int32_t *item_end;
     int64_t n_old;
     const int64_t *ga_new, *gb_new;
-    const int32_t *ib;                      // beta string index of each determinant
+    const int32_t *ia, *ib;                 // string indices of each determinant
     const int64_t *bs_off;                  // beta singles
     const int32_t *bs_idx;
-    const unsigned long long *occ;          // [Ua][occ_words] occupancy bitmap over (alpha, beta)
-    const int32_t *occ_pref;                // [Ua][occ_words] set bits before each word in its row
+    const OccCell *occ;                     // [Ua][occ_words] occupancy bitmap over (alpha, beta)
     int64_t occ_words;
-    // opposite-spin doubles by bitmap words (opposite.cuh) instead of in the
-    // alpha-grouped pass: nonzero words of each alpha group's members (word,
-    // its index and its first member's position in ow_det), the dense bitmap
-    // of each beta string's singles with the entries before each word, and per
-    // entry the beta part of the element (pair index << 1 | sign)
-    int by_words;
+    // opposite-spin doubles in a pass of their own (opposite.cuh) instead of in
+    // the alpha-grouped one: each alpha group's members (offsets, beta index,
+    // determinant) as occ places them, the number of beta strings, and the beta
+    // singles as (index, pair index << 1 | sign).  On the fly x is in the order
+    // of the alpha groups' members (x_grouped).
     const int64_t *ow_off;
-    const unsigned long long *ow_word;
-    const int2 *ow_info;
-    const int32_t *ow_det;
-    const unsigned long long *sbm;
-    const int32_t *sbp;
-    int64_t sb_words;
-    const uint32_t *bs_info;
+    const int32_t *ow_ib, *ow_det;
+    int64_t n_beta_str;
+    int opp_rows;                           // rows of an item
+    const int2 *bs_pair;
+    const double *x_grouped;
+    // single moves tabulated per string (k_move_tables), or null
+    const double *ma, *mb;
+    int n_pair;
     const int32_t *item_group;              // work item -> group index
     const int32_t *item_first;              // work item -> first member offset within the group
     int64_t n_items;
@@ -148,7 +167,8 @@ __device__ __forceinline__ double single_exc(const DevInts &I, const Str<W> &si,
     const int neg = bits_between<W>(common, p < q ? p : q, p < q ? q : p);
     const double *jk = I.jk1 + (int64_t)(p * n + q) * n;
     const double *jo = I.j1 + (int64_t)(p * n + q) * n;
-    double v = __ldg(&I.h[p * n + q]);
+    // a sum per string, added last: the order of the tabulated moves
+    double v = __ldg(&I.h[p * n + q]), vo = 0.0;
 #pragma unroll
     for (int k = 0; k < W; k++) {
         uint64_t m = common.w[k];
@@ -161,10 +181,10 @@ __device__ __forceinline__ double single_exc(const DevInts &I, const Str<W> &si,
         while (o) {
             int b = __ffsll((long long)o) - 1;
             o &= o - 1;
-            v += __ldg(&jo[64 * k + b]);
+            vo += __ldg(&jo[64 * k + b]);
         }
     }
-    return flip_sign(v, neg);
+    return flip_sign(v + vo, neg);
 }
 
 // same-spin double: holes q1 < q2 in sj, particles p1 < p2 in si
@@ -213,9 +233,16 @@ __device__ __forceinline__ double eri_pairs(const DevInts &I, int pq, int rs) {
 // row's beta and alpha strings); sj: D_j's string of the differing spin.
 // ctx & 1 marks an opposite-spin double whose alpha part (pair index ctx >> 2,
 // sign bit (ctx >> 1) & 1) was computed once for the whole candidate group.
+// own / oth: the row's entries of the move tables (the differing string's
+// first part, the other string's second), or null.
 template <int W>
 __device__ __forceinline__ double eval_pair(const DevInts &I, const Str<W> &si, const Str<W> &other,
-                                            const Str<W> &sj, int ctx) {
+                                            const Str<W> &sj, int ctx, const double *own, const double *oth) {
+    if (!(ctx & 1) && own && xor_popc<W>(si, sj) == 2) {
+        int pq, neg;
+        move_info<W>(si, sj, pq, neg);
+        return flip_sign(__ldg(&own[pq]) + __ldg(&oth[pq]), neg);
+    }
     if (ctx & 1) {
         int pq_b, neg_b;
         move_info<W>(si, sj, pq_b, neg_b);
@@ -311,6 +338,7 @@ struct RowAcc {
     int64_t i = 0;          // the row's determinant (gradient mode)
     int ka = K;             // vectors in use (sigma mode)
     double ci = 0.0;        // its coefficient (gradient mode)
+    const double *own = nullptr, *oth = nullptr;   // its entries of the move tables
     double acc[K > 0 ? K : 1];
 };
 
@@ -338,7 +366,7 @@ __device__ __forceinline__ void flush(RowAcc<MODE, K> &R, const EnumArgs &A, con
 #pragma unroll
         for (int k = 0; k < W; k++) sj.w[k] = Q.s[lane * W + k];
         const int32_t j = Q.j[lane];
-        const double v = eval_pair<W>(I, si, other, sj, Q.ctx[lane]);
+        const double v = eval_pair<W>(I, si, other, sj, Q.ctx[lane], R.own, R.oth);
         if (ModeOf<MODE>::fill) {
             A.col[R.pos + lane] = j;
             A.val[R.pos + lane] = v;
@@ -496,7 +524,8 @@ __device__ __forceinline__ void old_row_suffix(RowAcc<MODE, K> &R, const EnumArg
 // row's own alpha group) and opposite-spin doubles (candidates in the alpha
 // groups of the alpha singles of the row's alpha string).  One work item:
 // up to ENUM_NW rows of one alpha group, one per warp; called by the whole CTA.
-template <int W, int MODE, int K>
+// OPP: the opposite-spin doubles too (otherwise a pass of their own finds them).
+template <int W, int MODE, int K, bool OPP>
 __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts &I, int64_t item, Tile<W> &T,
                                                 WarpQueue<W> &Q, unsigned long long &cand_local, int k_active = 0) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -515,6 +544,10 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
     const Str<W> Bi = valid ? load_str<W>(rstr, g_beg + r) : Str<W>{};
     RowAcc<MODE, K> R;
     row_begin(R, A, i, valid);
+    if (!ModeOf<MODE>::count && MODE != ENUM_GRAD && A.ma && valid) {
+        R.own = A.mb + 2 * (int64_t)A.ib[i] * A.n_pair;
+        R.oth = A.ma + (2 * (int64_t)a + 1) * A.n_pair;
+    }
     R.ka = k_active ? k_active : (A.k_active ? A.k_active : K);
     if (XM && A.n_old > 0) {
         // old rows: the new members of the own group (same-spin beta
@@ -523,7 +556,7 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
         if (valid) {
             const int64_t n_beg = A.ga_new[a];
             old_row_suffix<W, MODE, K>(R, A, I, Q, Bi, Ai, A.ga_str, A.ga_det, n_beg, g_beg + g_len, cand_local);
-            const int64_t s_beg = A.as_off[a], s_end = A.by_words ? s_beg : A.as_off[a + 1];
+            const int64_t s_beg = A.as_off[a], s_end = OPP ? A.as_off[a + 1] : s_beg;
             for (int64_t s0 = s_beg; s0 < s_end; s0 += 32) {
                 // one alpha single per lane: its group's new members and pair context
                 int64_t kb = 0;
@@ -596,7 +629,7 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
         }
         __syncthreads();
     }
-    if (A.by_words) {                       // the opposite-spin doubles have a pass of their own
+    if constexpr (!OPP) {
         row_end<W, MODE, K>(R, A, I, Q, Bi, Ai, i, valid);
         return;
     }
@@ -638,7 +671,7 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
         const bool lookup = A.opp_lookup && (!A.opp_hybrid || (float)k_len > A.opp_factor * (float)sb_max);
         if (lookup) {
             if (!valid) continue;
-            const unsigned long long *row = A.occ + (int64_t)k * A.occ_words;
+            const OccCell *row = A.occ + (int64_t)k * A.occ_words;
             cand_local += lane == 0 ? sb_len : 0;
             // LU lookups per lane per step, each stage's loads issued together
             // (independent L2 gathers in flight instead of one dependent chain)
@@ -655,7 +688,7 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
                     kb[u] = y < sb_len ? __ldg(&A.bs_idx[sb_beg + y]) : -1;
                 }
 #pragma unroll
-                for (int u = 0; u < LU; u++) word[u] = kb[u] >= 0 ? __ldg(&row[kb[u] >> 6]) : 0ull;
+                for (int u = 0; u < LU; u++) word[u] = kb[u] >= 0 ? __ldg(&row[kb[u] >> 6].bits) : 0ull;
 #pragma unroll
                 for (int u = 0; u < LU; u++) {
                     match[u] = kb[u] >= 0 && ((word[u] >> (kb[u] & 63)) & 1ull);
@@ -666,11 +699,11 @@ __device__ __forceinline__ void enum_alpha_item(const EnumArgs &A, const DevInts
                     int64_t m[LU];
 #pragma unroll
                     for (int u = 0; u < LU; u++)
-                        m[u] = match[u] ? __ldg(&A.occ_pref[(int64_t)k * A.occ_words + (kb[u] >> 6)]) : 0;
+                        m[u] = match[u] ? __ldg(&row[kb[u] >> 6].place) : 0;
 #pragma unroll
                     for (int u = 0; u < LU; u++) {
                         if (match[u]) {
-                            m[u] += k_beg + __popcll(word[u] & ((1ull << (kb[u] & 63)) - 1ull));
+                            m[u] += __popcll(word[u] & ((1ull << (kb[u] & 63)) - 1ull));
                             j[u] = __ldg(&A.ga_det[m[u]]);
                             Bj[u] = load_str<W>(A.ga_str, m[u]);
                         }
@@ -723,6 +756,10 @@ __device__ __forceinline__ void enum_beta_item(const EnumArgs &A, const DevInts 
     const Str<W> Ai = valid ? load_str<W>(rstr, g_beg + r) : Str<W>{};
     RowAcc<MODE, K> R;
     row_begin(R, A, i, valid);
+    if (!ModeOf<MODE>::count && MODE != ENUM_GRAD && A.ma && valid) {
+        R.own = A.ma + 2 * (int64_t)A.ia[i] * A.n_pair;
+        R.oth = A.mb + (2 * (int64_t)b + 1) * A.n_pair;
+    }
     R.ka = k_active ? k_active : (A.k_active ? A.k_active : K);
     if (XM && A.n_old > 0) {
         // old rows: the new members of the own beta group (same-spin alpha excitations)
@@ -773,7 +810,7 @@ struct EnumMinBlocks {
 };
 
 // persistent grids: CTAs take work items from an atomic counter
-template <int W, int MODE, int K>
+template <int W, int MODE, int K, bool OPP>
 __global__ void __launch_bounds__(ENUM_THREADS, EnumMinBlocks<MODE>::value) k_enum_alpha(EnumArgs A, DevInts I) {
     __shared__ EnumSmem<W> S;
     __shared__ int item_sh;
@@ -784,7 +821,7 @@ __global__ void __launch_bounds__(ENUM_THREADS, EnumMinBlocks<MODE>::value) k_en
         const int64_t item = item_sh;
         __syncthreads();
         if (item >= A.n_items) break;
-        enum_alpha_item<W, MODE, K>(A, I, item, S.T, S.Q[threadIdx.x >> 5], cand_local);
+        enum_alpha_item<W, MODE, K, OPP>(A, I, item, S.T, S.Q[threadIdx.x >> 5], cand_local);
     }
     if (ModeOf<MODE>::count && (threadIdx.x & 31) == 0 && cand_local) atomicAdd(A.cand, cand_local);
 }
@@ -826,23 +863,23 @@ static __global__ void k_items_fill(const int64_t *__restrict__ off, const int64
 // incremental update: items over one part of each determinant-ordered group,
 // the old members [0, g_new - off) (part 0) or the new ones (part 1)
 static __global__ void k_items_count_part(const int64_t *__restrict__ off, const int64_t *__restrict__ g_new,
-                                          int64_t n_groups, int part, int64_t *__restrict__ cnt) {
+                                          int64_t n_groups, int part, int chunk, int64_t *__restrict__ cnt) {
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x) {
         const int64_t m = part ? off[g + 1] - g_new[g] : g_new[g] - off[g];
-        cnt[g] = (m + ENUM_NW - 1) / ENUM_NW;
+        cnt[g] = (m + chunk - 1) / chunk;
     }
 }
 
 static __global__ void k_items_fill_part(const int64_t *__restrict__ off, const int64_t *__restrict__ g_new,
-                                         const int64_t *__restrict__ start, int64_t n_groups, int part,
+                                         const int64_t *__restrict__ start, int64_t n_groups, int part, int chunk,
                                          int32_t *__restrict__ item_group, int32_t *__restrict__ item_first,
                                          int32_t *__restrict__ item_end) {
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x) {
         const int64_t lo = part ? g_new[g] - off[g] : 0, hi = part ? off[g + 1] - off[g] : g_new[g] - off[g];
-        const int64_t c = (hi - lo + ENUM_NW - 1) / ENUM_NW;
+        const int64_t c = (hi - lo + chunk - 1) / chunk;
         for (int64_t t = 0; t < c; t++) {
             item_group[start[g] + t] = (int32_t)g;
-            item_first[start[g] + t] = (int32_t)(lo + t * ENUM_NW);
+            item_first[start[g] + t] = (int32_t)(lo + t * chunk);
             item_end[start[g] + t] = (int32_t)hi;
         }
     }

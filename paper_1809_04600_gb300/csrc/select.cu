@@ -17,6 +17,7 @@
 
 #include "context.cuh"
 #include "enumerate.cuh"
+#include "move_tables.cuh"
 
 namespace shci {
 
@@ -275,36 +276,7 @@ struct SelArgs {
     const int32_t *ia, *ib;
 };
 
-// Single moves p -> r of a determinant (A, B): the element is
-//   [h_pr + sum_{k in A} ((pr|kk) - (pk|kr))] + sum_{k in B} (pr|kk)
-// (k = p contributes an exact zero to the first sum), a term of the moving
-// string and one of the other.  Both are tabulated for every string of V and
-// every orbital pair, M[u][0][pr] and M[u][1][pr], so that a move costs one
-// FP64 addition instead of one per electron: those additions held the FP64
-// pipe (74 % busy in the count pass).
-template <int W>
-__global__ void k_move_tables(const uint64_t *__restrict__ str, int64_t U, DevInts I, double *__restrict__ M) {
-    const int n = I.n, np = n * (n + 1) / 2;
-    const int64_t total = U * np;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t u = t / np;
-        const int pr = (int)(t - u * np);
-        int p = (int)((sqrtf(8.0f * (float)pr + 1.0f) - 1.0f) * 0.5f);
-        while (p * (p + 1) / 2 > pr) p--;
-        while ((p + 1) * (p + 2) / 2 <= pr) p++;
-        const int r = pr - p * (p + 1) / 2;
-        const double *jk = I.jk1 + (int64_t)(p * n + r) * n, *j1 = I.j1 + (int64_t)(p * n + r) * n;
-        double same = __ldg(&I.h[p * n + r]), opp = 0.0;
-        for_bits_above<W>(load_str<W>(str, u), -1, [&](int k) {
-            same += __ldg(&jk[k]);
-            opp += __ldg(&j1[k]);
-        });
-        M[2 * u * np + pr] = same;
-        M[(2 * u + 1) * np + pr] = opp;
-    }
-}
-
-// The tables of both spins' strings, owned by one call.
+// The tables of both spins' strings, owned by one call (move_tables.cuh).
 struct MoveTables {
     DevBuf<double> a, b;
 };
@@ -316,6 +288,13 @@ struct MoveTables {
 template <int W>
 static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double rows, MoveTables &T) {
     const int n = c->n_orb;
+    if (c->have_moves) {                    // the connectivity's own
+        S.ma = c->move_a.p;
+        S.mb = c->move_b.p;
+        S.ia = c->ia.p;
+        S.ib = c->ib.p;
+        return;
+    }
     const int64_t np = (int64_t)n * (n + 1) / 2;
     const double entries = (double)(c->Ua + c->Ub) * np;
     const double moves = rows * ((double)S.na * (n - S.na) + (double)S.nb * (n - S.nb));
@@ -323,13 +302,7 @@ static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double row
     size_t fr = 0, tot = 0;
     CUDA_TRY(cudaMemGetInfo(&fr, &tot));
     if (entries * 16.0 > (double)fr / 16.0) return;
-    T.a.alloc((size_t)(2 * c->Ua * np));
-    T.b.alloc((size_t)(2 * c->Ub * np));
-    auto grid = [&](int64_t m) { return (unsigned)std::min<int64_t>(ceil_div(m, SEL_THREADS), (int64_t)c->n_sm * 32); };
-    k_move_tables<W><<<grid(c->Ua * np), SEL_THREADS, 0, c->st>>>(c->astr.p, c->Ua, I, T.a.p);
-    k_move_tables<W><<<grid(c->Ub * np), SEL_THREADS, 0, c->st>>>(c->bstr.p, c->Ub, I, T.b.p);
-    KERNEL_CHECK();
-    g_kernel_launches += 2;
+    make_move_tables<W>(c, I, T.a, T.b);
     S.ma = T.a.p;
     S.mb = T.b.p;
     S.ia = c->ia.p;

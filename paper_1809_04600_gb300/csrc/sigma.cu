@@ -230,7 +230,7 @@ void sigma(shci_ctx *c, int k, const double *x, double *y, bool inter) {
 // Sec. VIII): every product re-enumerates the connected pairs with the helper
 // lists and recomputes H_ij, so H is never stored.  Pass 1 (rows grouped by
 // alpha string) writes y = diag * x + same-spin-beta terms, pass 2 adds the
-// opposite-spin terms (opposite.cuh; without its bitmaps pass 1 does), pass 3
+// opposite-spin terms (opposite.cuh; without its bitmap pass 1 does), pass 3
 // (rows grouped by beta string) the same-spin-alpha terms.
 template <int W, int K>
 static void otf_k(shci_ctx *c, const double *x, double *y) {
@@ -241,7 +241,10 @@ static void otf_k(shci_ctx *c, const double *x, double *y) {
     DevInts I = dev_ints(c);
     A.accumulate = 0;
     launch_enum<W, ENUM_SIGMA, K>(c, A, I, true);
-    if (c->opp_words) launch_opposite<W, ENUM_SIGMA, K>(c, A, I);
+    if (c->opp_pass) {
+        group_vectors(c, A, K);
+        launch_opposite<W, ENUM_SIGMA, K>(c, A, I);
+    }
     A.accumulate = 1;
     launch_enum<W, ENUM_SIGMA, K>(c, A, I, false);
 }
