@@ -143,15 +143,13 @@ __global__ void k_head_flags(const uint64_t *__restrict__ keys, int64_t n, int64
 template <int W>
 __global__ void k_unique_write(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ vals,
                                const int64_t *__restrict__ flags, const int64_t *__restrict__ excl, int64_t n,
-                               uint64_t *__restrict__ ustr, int32_t *__restrict__ sidx, int32_t *__restrict__ first) {
+                               uint64_t *__restrict__ ustr, int32_t *__restrict__ sidx) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t id = excl[i] + flags[i] - 1;
         if (flags[i]) {
 #pragma unroll
             for (int k = 0; k < W; k++) ustr[id * W + k] = keys[i * W + k];
-            first[id] = (int32_t)i;
         }
-        if (i == n - 1) first[id + 1] = (int32_t)n;
         sidx[vals[i]] = (int32_t)id;
     }
 }
@@ -447,58 +445,10 @@ static void unique_strings(shci_ctx *c, int spin, DevBuf<uint64_t> &ustr, DevBuf
     CUDA_TRY(cudaStreamSynchronize(st));
     ustr.alloc((size_t)U * W);
     sidx.alloc((size_t)n);
-    c->i32a.alloc((size_t)U + 1);
     k_unique_write<W><<<grid_for(n), 256, 0, st>>>(c->sort_keys.p, c->sort_vals.p, c->i64a.p, c->i64b.p, n, ustr.p,
-                                                   sidx.p, c->i32a.p);
+                                                   sidx.p);
     KERNEL_CHECK();
     LAUNCHED(3);
-}
-
-// keys that ascend as the strings' determinant counts descend; first: where
-// each string's run begins among the sorted determinants
-__global__ void k_count_keys(const int32_t *__restrict__ first, int64_t U, uint32_t top, uint64_t *__restrict__ keys) {
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < U; u += (int64_t)gridDim.x * blockDim.x)
-        keys[u] = top - (uint32_t)(first[u + 1] - first[u]);
-}
-
-// string order[r] gets number r
-template <int W>
-__global__ void k_renumber(const uint32_t *__restrict__ order, int64_t U, const uint64_t *__restrict__ old,
-                           uint64_t *__restrict__ str, uint32_t *__restrict__ number) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < U; r += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t u = order[r];
-#pragma unroll
-        for (int w = 0; w < W; w++) str[r * W + w] = old[(int64_t)u * W + w];
-        number[u] = (uint32_t)r;
-    }
-}
-
-__global__ void k_apply_number(const uint32_t *__restrict__ number, int64_t n, int32_t *__restrict__ sidx) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        sidx[i] = (int32_t)number[sidx[i]];
-}
-
-// Number the unique strings by decreasing number of determinants (ties as
-// before, ascending): a group's members then fill few words of the bitmaps
-// over the other spin's numbers, and the enumeration's largest work items come
-// first.
-template <int W>
-static void number_by_size(shci_ctx *c, int64_t U, DevBuf<uint64_t> &ustr, DevBuf<int32_t> &sidx) {
-    // right after unique_strings: c->i32a holds the runs' beginnings, the sort buffers are free
-    const int64_t n = c->n_det;
-    cudaStream_t st = c->st;
-    if (U <= 1) return;
-    c->u32a.alloc((size_t)U);
-    c->str_tmp.alloc((size_t)U * W);
-    const uint64_t top = composite_mask(0, n + 1) & 0xFFFFFFFFull;       // at least n, all ones
-    k_count_keys<<<grid_for(U), 256, 0, st>>>(c->i32a.p, U, (uint32_t)top, c->sort_keys.p);
-    KERNEL_CHECK();
-    radix_sort<1>(c->sort_keys.p, c->sort_vals.p, U, c->sw, st, &top, RS_POSITION);
-    k_renumber<W><<<grid_for(U), 256, 0, st>>>(c->sort_vals.p, U, ustr.p, c->str_tmp.p, c->u32a.p);
-    k_apply_number<<<grid_for(n), 256, 0, st>>>(c->u32a.p, n, sidx.p);
-    KERNEL_CHECK();
-    LAUNCHED(3);
-    ustr.swap(c->str_tmp);
 }
 
 template <int W>
@@ -658,6 +608,7 @@ static void opposite_pass_setup(shci_ctx *c) {
     cudaStream_t st = c->st;
     c->bs_pair.alloc((size_t)std::max<int64_t>(c->n_beta_singles, 1));
     c->ga_ib.alloc((size_t)c->n_det);
+    c->x_grouped.alloc((size_t)c->n_det);   // a first product of one vector allocates nothing
     k_singles_info<W><<<grid_for(c->Ub * 32), 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->bstr.p, c->bs_pair.p);
     k_member_index<<<grid_for(c->n_det), 256, 0, st>>>(c->ga_det.p, c->n_det, c->ib.p, c->ga_ib.p);
     KERNEL_CHECK();
@@ -737,9 +688,7 @@ static void lists_w(shci_ctx *c) {
     if (flags & 4) throw ShciError{SHCI_ERR_INVALID, "a determinant occupies an orbital >= n_orb"};
 
     unique_strings<W>(c, 0, c->astr, c->ia, c->Ua);
-    number_by_size<W>(c, c->Ua, c->astr, c->ia);
     unique_strings<W>(c, 1, c->bstr, c->ib, c->Ub);
-    number_by_size<W>(c, c->Ub, c->bstr, c->ib);
     group_by<W>(c, c->ia.p, c->ib.p, c->Ua, c->Ub, 1, c->ga_off, c->ga_det, c->ga_str);
     group_by<W>(c, c->ib.p, c->ia.p, c->Ub, c->Ua, 0, c->gb_off, c->gb_det, c->gb_str);
     CUDA_TRY(cudaMemcpyAsync(&flags, c->counter.p, sizeof(int), cudaMemcpyDeviceToHost, st));

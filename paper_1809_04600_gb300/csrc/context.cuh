@@ -107,10 +107,8 @@ struct shci_ctx {
     DevBuf<uint64_t> sort_keys;
     DevBuf<uint32_t> sort_vals;
     DevBuf<int64_t> i64a, i64b, i64c;
-    DevBuf<int32_t> i32a, seg_len;
+    DevBuf<int32_t> seg_len;
     DevBuf<int64_t> seg_start;
-    DevBuf<uint32_t> u32a;
-    DevBuf<uint64_t> str_tmp;
     DevBuf<unsigned long long> cand;       // candidates screened by a count pass
     DevBuf<int> counter;                   // dynamic work counters / flags
     DevBuf<double> vec_a, vec_b;           // layout conversion for the ABI sigma

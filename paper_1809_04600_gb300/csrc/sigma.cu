@@ -36,12 +36,17 @@ constexpr int SIGMA_THREADS = 256;
 // Rows per warp group: a warp takes R consecutive rows one after another,
 // keeps each row's per-lane partial sums in registers, and reduces the R rows
 // together at the end (below); fewer rows for more vectors (registers).
-template <int K, bool INTER>
+// FEW: a row per warp, for spaces whose groups of R would not fill the GPU's
+// warps.  There a warp's chain of dependent loads (row offset, column,
+// coefficient), row after row, is the time, not the FP64 pipe (24 orbitals, one
+// vector: 2,053 determinants 28.8 to 20.0 us, 5,003 36.7 to 24.8; four vectors,
+// 5,003: 88 to 50).
+template <int K, bool INTER, bool FEW = false>
 struct SigmaRows {
     // the shapes the Davidson iteration launches (one vector, or two interleaved)
     static constexpr bool TUNED = K == 1 || (K == 2 && INTER);
-    static constexpr int R = TUNED ? SHCI_SIGMA_R2 : (K <= 4 ? 4 : 2);
-    static constexpr int SR = TUNED ? SHCI_SIGMA_SR2 : 2;
+    static constexpr int R = FEW ? 1 : (TUNED ? SHCI_SIGMA_R2 : (K <= 4 ? 4 : 2));
+    static constexpr int SR = TUNED ? SHCI_SIGMA_SR2 : (FEW && K <= 4 ? 4 : 2);
     static constexpr int MINB = TUNED ? SHCI_SIGMA_MINB2 : 1;
 };
 
@@ -55,15 +60,13 @@ struct SigmaRows {
 // by a butterfly that halves the rows a lane holds at each of the first
 // log2(R) levels ((R - 1) + (5 - log2 R) adds per vector for R rows), and one
 // lane per row writes y = H_ii x + sum.
-template <int K, bool INTER>
-__global__ void __launch_bounds__(SIGMA_THREADS, SigmaRows<K, INTER>::MINB) k_sigma_stored(int64_t n,
-                                                                                   const int64_t *__restrict__ rowptr,
-                                                                const int32_t *__restrict__ col,
-                                                                const double *__restrict__ val,
-                                                                const double *__restrict__ diag,
-                                                                const double *__restrict__ x, double *__restrict__ y) {
-    constexpr int SR = SigmaRows<K, INTER>::SR;
-    constexpr int R = SigmaRows<K, INTER>::R;
+template <int K, bool INTER, bool FEW>
+__global__ void __launch_bounds__(SIGMA_THREADS, SigmaRows<K, INTER, FEW>::MINB)
+    k_sigma_stored(int64_t n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                   const double *__restrict__ val, const double *__restrict__ diag, const double *__restrict__ x,
+                   double *__restrict__ y) {
+    constexpr int SR = SigmaRows<K, INTER, FEW>::SR;
+    constexpr int R = SigmaRows<K, INTER, FEW>::R;
     constexpr int LOG_R = R == 8 ? 3 : (R == 4 ? 2 : (R == 2 ? 1 : 0));
     const int lane = threadIdx.x & 31;
     const int64_t n_groups = (n + R - 1) / R;
@@ -155,11 +158,22 @@ __global__ void __launch_bounds__(SIGMA_THREADS, SigmaRows<K, INTER>::MINB) k_si
     }
 }
 
+// A row per warp up to as many rows as the grid has warps for groups of R
+// (SIGMA_FEW per SM; the sums are the same ones in the same order).
+constexpr int SIGMA_FEW = 32;
+
 template <int K, bool INTER>
 static void launch_stored(shci_ctx *c, const double *x, double *y) {
-    int blocks = c->n_sm * (2048 / SIGMA_THREADS);
-    k_sigma_stored<K, INTER><<<blocks, SIGMA_THREADS, 0, c->st>>>(c->n_det, c->rowptr.p, c->col.p, c->val.p,
-                                                                 c->diag.p, x, y);
+    const int64_t n = c->n_det;
+    if (n <= (int64_t)c->n_sm * SIGMA_FEW * SigmaRows<K, INTER>::R) {
+        const int blocks = (int)std::max<int64_t>(1, ceil_div(n, SIGMA_THREADS / 32));
+        k_sigma_stored<K, INTER, true><<<blocks, SIGMA_THREADS, 0, c->st>>>(n, c->rowptr.p, c->col.p, c->val.p,
+                                                                           c->diag.p, x, y);
+    } else {
+        const int blocks = c->n_sm * (2048 / SIGMA_THREADS);
+        k_sigma_stored<K, INTER, false><<<blocks, SIGMA_THREADS, 0, c->st>>>(n, c->rowptr.p, c->col.p, c->val.p,
+                                                                            c->diag.p, x, y);
+    }
     KERNEL_CHECK();
 }
 
@@ -184,17 +198,12 @@ void sigma_upper(shci_ctx *c, int k, const double *x, double *y, bool inter);   
 // loads every stored-sigma kernel onto the current device (with lazy module
 // loading a kernel's module is otherwise loaded, and device memory taken, at
 // its first launch)
-template <bool INTER>
+template <bool INTER, int K = 1>
 static void preload_stored() {
     cudaFuncAttributes fa;
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<1, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<2, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<3, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<4, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<5, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<6, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<7, INTER>));
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<8, INTER>));
+    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<K, INTER, false>));
+    CUDA_TRY(cudaFuncGetAttributes(&fa, k_sigma_stored<K, INTER, true>));
+    if constexpr (K < SHCI_MAX_K) preload_stored<INTER, K + 1>();
 }
 
 void sigma_stored_preload() {
