@@ -93,7 +93,10 @@ void launch_opposite(shci_ctx *c, EnumArgs A, const DevInts &I) {
     }
     if (A.n_items == 0) return;
     const size_t smem = sizeof(uint32_t) * opp_table(c->Ub);
-    CUDA_TRY(cudaFuncSetAttribute(k_opposite<W, MODE, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit belongs to the kernel, not to the launch: always the largest table's,
+    // so that contexts of other sizes in other host threads cannot lower it in between
+    CUDA_TRY(cudaFuncSetAttribute(k_opposite<W, MODE, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(sizeof(uint32_t) * OPP_RANGE)));
     int per_sm = 0;
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_opposite<W, MODE, K>, ENUM_THREADS, smem));
     const int blocks = (int)std::min<int64_t>(A.n_items, (int64_t)c->n_sm * std::max(per_sm, 1));
