@@ -319,18 +319,29 @@ __global__ void k_row_parts(const int64_t *__restrict__ cnt_b, int64_t *__restri
     }
 }
 
+// work items of up to `chunk` members of each group; with `choice`, those of the
+// opposite-spin pass, whose costs with and without lookups come back with the count
 static void make_items(shci_ctx *c, const int64_t *off, int64_t n_groups, int chunk, DevBuf<int32_t> &item_group,
-                       DevBuf<int32_t> &item_first, int64_t &n_items) {
+                       DevBuf<int32_t> &item_first, int64_t &n_items, bool *choice = nullptr) {
     cudaStream_t st = c->st;
     DevBuf<int64_t> &cnt = c->i64a, &start = c->i64b, &tmp = c->i64c;
     cnt.alloc((size_t)n_groups + 1);
-    start.alloc((size_t)n_groups + 1);
+    start.alloc((size_t)n_groups + 3);
     tmp.alloc((size_t)scan_tmp_len(n_groups + 1));
     unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n_groups, 256), 4096));
-    k_items_count<<<g, 256, 0, st>>>(off, n_groups, chunk, cnt.p);
+    unsigned long long *costs = reinterpret_cast<unsigned long long *>(start.p + n_groups + 1);
+    k_items_count<<<g, 256, 0, st>>>(off, n_groups, chunk, cnt.p, costs);
     exclusive_scan<int64_t>(cnt.p, start.p, n_groups, tmp.p, st);
-    CUDA_TRY(cudaMemcpyAsync(&n_items, start.p + n_groups, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    if (choice) {
+        k_opp_costs<<<std::min(4096u, (unsigned)ceil_div(n_groups, 8)), 256, 0, st>>>(
+            off, n_groups, chunk, c->as_off.p, c->as_idx.p, ceil_div(c->n_beta_singles, c->Ub), c->Ub, costs);
+        g_kernel_launches += 1;
+    }
+    int64_t got[3];                          // items; costs with tables alone, and with the choice
+    CUDA_TRY(cudaMemcpyAsync(got, start.p + n_groups, sizeof(int64_t) * (choice ? 3 : 1), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
+    n_items = got[0];
+    if (choice) *choice = 1.25 * (double)got[2] < (double)got[1];
     if (n_items > 0x7FFFFFFFll) throw ShciError{SHCI_ERR_INVALID, "too many work items"};
     item_group.alloc((size_t)std::max<int64_t>(n_items, 1));
     item_first.alloc((size_t)std::max<int64_t>(n_items, 1));
@@ -708,7 +719,7 @@ static void lists_w(shci_ctx *c) {
     make_items(c, c->gb_off.p, c->Ub, ENUM_NW, c->item_b_group, c->item_b_first, c->n_items_b);
     if (c->opp_pass) {
         const int rows = opp_item_rows(n, c->n_sm);
-        make_items(c, c->ga_off.p, c->Ua, rows, c->item_o_group, c->item_o_first, c->n_items_o);
+        make_items(c, c->ga_off.p, c->Ua, rows, c->item_o_group, c->item_o_first, c->n_items_o, &c->opp_choice);
     }
 }
 

@@ -81,6 +81,7 @@ struct shci_ctx {
     float opp_factor = 0.5f;               // scan a group of up to this many x the beta singles
     // opposite-spin doubles in a pass of their own (opposite.cuh)
     bool opp_pass = false;
+    bool opp_choice = false;               // tables or lookups for each 32 alpha singles
     DevBuf<int32_t> ga_ib;                 // beta index of each alpha group's members
     DevBuf<int2> bs_pair;                  // beta singles: index, pair index << 1 | sign
     DevBuf<double> x_grouped;              // vectors of a product in the order of the alpha groups' members

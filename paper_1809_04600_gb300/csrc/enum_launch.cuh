@@ -36,6 +36,7 @@ inline EnumArgs enum_args(const shci_ctx *c) {
     A.ow_det = c->ga_det.p;
     A.n_beta_str = c->Ub;
     A.opp_rows = opp_item_rows(c->n_det, c->n_sm);
+    A.opp_beta_singles = (int)ceil_div(c->n_beta_singles, std::max<int64_t>(c->Ub, 1));
     A.bs_pair = c->bs_pair.p;
     A.ma = c->have_moves ? c->move_a.p : nullptr;
     A.mb = c->have_moves ? c->move_b.p : nullptr;
@@ -80,6 +81,22 @@ inline void group_vectors(shci_ctx *c, EnumArgs &A, int k) {
     A.x_grouped = c->x_grouped.p;
 }
 
+template <int W, int MODE, int K, bool CHOICE>
+void launch_opposite_as(shci_ctx *c, const EnumArgs &A, const DevInts &I) {
+    const size_t smem = opp_smem(A.opp_rows, c->Ub);
+    // the limit belongs to the kernel, not to the launch: always the largest table's,
+    // so that contexts of other sizes in other host threads cannot lower it in between
+    CUDA_TRY(cudaFuncSetAttribute(k_opposite<W, MODE, K, CHOICE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)OPP_SMEM_MAX));
+    int per_sm = 0;
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_opposite<W, MODE, K, CHOICE>, ENUM_THREADS,
+                                                           smem));
+    const int blocks = (int)std::min<int64_t>(A.n_items, (int64_t)c->n_sm * std::max(per_sm, 1));
+    k_opposite<W, MODE, K, CHOICE><<<blocks, ENUM_THREADS, smem, c->st>>>(A, I);
+    KERNEL_CHECK();
+    g_kernel_launches += 1;
+}
+
 // The opposite-spin pass (opposite.cuh) over the context's items, or the
 // caller's (rows from A.row_det, ends in A.item_end).
 template <int W, int MODE, int K>
@@ -92,17 +109,9 @@ void launch_opposite(shci_ctx *c, EnumArgs A, const DevInts &I) {
         A.row_det = c->ga_det.p;
     }
     if (A.n_items == 0) return;
-    const size_t smem = sizeof(uint32_t) * opp_table(c->Ub);
-    // the limit belongs to the kernel, not to the launch: always the largest table's,
-    // so that contexts of other sizes in other host threads cannot lower it in between
-    CUDA_TRY(cudaFuncSetAttribute(k_opposite<W, MODE, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(sizeof(uint32_t) * OPP_RANGE)));
-    int per_sm = 0;
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_opposite<W, MODE, K>, ENUM_THREADS, smem));
-    const int blocks = (int)std::min<int64_t>(A.n_items, (int64_t)c->n_sm * std::max(per_sm, 1));
-    k_opposite<W, MODE, K><<<blocks, ENUM_THREADS, smem, c->st>>>(A, I);
-    KERNEL_CHECK();
-    g_kernel_launches += 1;
+    // growth has groups without new members; the other passes choose where k_opp_costs says so
+    if (ModeOf<MODE>::inc || c->opp_choice) launch_opposite_as<W, MODE, K, true>(c, A, I);
+    else if constexpr (!ModeOf<MODE>::inc) launch_opposite_as<W, MODE, K, false>(c, A, I);
 }
 
 }  // namespace shci

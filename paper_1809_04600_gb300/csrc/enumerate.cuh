@@ -108,6 +108,7 @@ struct EnumArgs {
     const int32_t *ow_ib, *ow_det;
     int64_t n_beta_str;
     int opp_rows;                           // rows of an item
+    int opp_beta_singles;                   // beta singles of a string, on average
     const int2 *bs_pair;
     const double *x_grouped;
     // single moves tabulated per string (k_move_tables), or null
@@ -893,9 +894,11 @@ __global__ void __launch_bounds__(ENUM_THREADS, EnumMinBlocks<MODE>::value) k_en
     if (ModeOf<MODE>::count && (threadIdx.x & 31) == 0 && cand_local) atomicAdd(A.cand, cand_local);
 }
 
-// work items: one per chunk of `chunk` members of each group
+// work items: one per chunk of `chunk` members of each group (and two sums set to
+// zero for the kernel that follows)
 static __global__ void k_items_count(const int64_t *__restrict__ off, int64_t n_groups, int chunk,
-                                     int64_t *__restrict__ cnt) {
+                                     int64_t *__restrict__ cnt, unsigned long long *__restrict__ sums) {
+    if (blockIdx.x == 0 && threadIdx.x < 2) sums[threadIdx.x] = 0ull;
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x)
         cnt[g] = (off[g + 1] - off[g] + chunk - 1) / chunk;
 }

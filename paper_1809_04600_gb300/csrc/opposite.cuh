@@ -17,32 +17,63 @@
 // group) and of the beta single (tabulated).
 //
 // Larger beta spaces take several tables, each over a range of OPP_RANGE
-// strings.
+// strings.  A table pays where many rows share it and its singles are many:
+// clearing it and reading the singles' members is one cost for all rows of the
+// item.  Where that costs more than it saves (few alpha singles, or few rows,
+// beside many members and several tables) the rows look their pairs of singles
+// up in the occupancy bitmap one by one.  300,007 determinants over 3 alpha and
+// 134,596 beta strings: product 78.9 ms by tables, 23.8 by lookups, 45.0 by the
+// choice per alpha single in enumerate.cuh; count 66.4, 12.7 and 25.6.
 #pragma once
 #include "enumerate.cuh"
 
 namespace shci {
 
-constexpr int OPP_ROWS = 128;               // rows of an item, at most
+constexpr int OPP_ROWS = 1024;              // rows of an item, at most
 constexpr int OPP_RANGE = 24576;            // beta strings per table: 96 KB, two CTAs per SM
 
 // Rows of an item for n determinants: filling the tables takes about as long as
 // scanning some 30 rows, but a small space has too few groups to spread over
-// the GPU in large items.  About 16 items per SM, of 8 to 128 rows.
+// the GPU in large items.  About 16 items per SM, of 8 to 128 rows; spaces that
+// have 64 items per SM of those take larger ones, because the groups, and with
+// them the members read for a table, grow with V (76 orbitals, 31,500 strings a
+// spin, 5e7 determinants: count pass with the same-spin ones 2.35 s at 128 rows,
+// 1.06 at 1024; product 4.92 and 3.87; 1e7: 110 and 89 ms, 426 and 380).
 inline int opp_item_rows(int64_t n, int n_sm) {
     int rows = 8;
-    while (rows < OPP_ROWS && (int64_t)rows * 32 * n_sm <= n) rows *= 2;
+    while (rows < OPP_ROWS && (int64_t)rows * (rows < 128 ? 32 : 128) * n_sm <= n) rows *= 2;
     return rows;
 }
 
 // the words of the table for U beta strings
-inline int opp_table(int64_t U) { return (int)(U < OPP_RANGE ? U : OPP_RANGE); }
+__host__ __device__ inline int opp_table(int64_t U) { return (int)(U < OPP_RANGE ? U : OPP_RANGE); }
+
+// dynamic shared memory: the table, then the rows' places
+__host__ __device__ inline int opp_places(int64_t U) { return (opp_table(U) + 1) & ~1; }      // their word offset
+inline size_t opp_smem(int rows, int64_t U) { return sizeof(uint32_t) * opp_places(U) + sizeof(int64_t) * rows; }
+constexpr size_t OPP_SMEM_MAX = sizeof(int64_t) * OPP_ROWS + sizeof(uint32_t) * OPP_RANGE;
+
+// Look the pairs of ns alpha singles up one by one instead of filling tables?
+// rows x beta singles x ns lookups against, for each table, the singles' members
+// and a word per row and beta single, and clearing all U words.  A cleared word
+// takes 0.3 ps, the others 3 to 5 ps (the bitmap in L2 or not): the lookups are
+// counted double, the cleared words as a sixteenth.  A row's lookups are one
+// warp's, so fewer rows than warps take as long as that many.
+__host__ __device__ inline int64_t opp_table_cost(int64_t rows, int64_t beta_singles, int64_t members, int64_t U) {
+    return U / 16 + (U + OPP_RANGE - 1) / OPP_RANGE * (members + rows * beta_singles);
+}
+__host__ __device__ inline int64_t opp_lookup_cost(int64_t rows, int64_t beta_singles, int ns) {
+    return 2 * (rows > ENUM_NW ? rows : ENUM_NW) * beta_singles * ns;
+}
+__host__ __device__ inline bool opp_direct(int64_t rows, int64_t beta_singles, int ns, int64_t members, int64_t U) {
+    return opp_lookup_cost(rows, beta_singles, ns) < opp_table_cost(rows, beta_singles, members, U);
+}
 
 struct OppSmem {
-    int64_t pos[OPP_ROWS];                  // fill: each row's next slot; count: pairs so far
     uint32_t queue[ENUM_NW][64];            // beta single << 5 | alpha single
     int64_t occ[32];                        // the singles' rows of the bitmap
     int pq[32];                             // alpha part: pair index << 1 | sign
+    int members;                            // of the singles' groups
 };
 
 template <int MODE, int K>
@@ -114,10 +145,11 @@ __device__ __forceinline__ void opp_flush(OppRow<MODE, K> &R, const EnumArgs &A,
     }
 }
 
-// one row's beta singles against the table of strings [k0, k0 + range)
-template <int MODE, int K>
+// one row's beta singles against the table of strings [k0, k0 + range), or (only
+// with CHOICE: range 0) against the ns singles' rows of the bitmap
+template <int MODE, int K, bool CHOICE>
 __device__ __forceinline__ void opp_scan(OppRow<MODE, K> &R, const EnumArgs &A, const DevInts &I, const OppSmem &S,
-                                         const uint32_t *M, uint32_t *queue, int n, int k0, int range) {
+                                         const uint32_t *M, uint32_t *queue, int n, int ns, int k0, int range) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     for (int t0 = 0; t0 < n; t0 += 32) {
@@ -125,7 +157,13 @@ __device__ __forceinline__ void opp_scan(OppRow<MODE, K> &R, const EnumArgs &A, 
         unsigned m = 0u;
         if (t < n) {
             const unsigned kb = (unsigned)(__ldg(&A.bs_pair[R.sb + t].x) - k0);
-            if (kb < (unsigned)range) m = M[kb];
+            if (kb < (unsigned)range) {
+                m = M[kb];
+            } else if (CHOICE && range == 0) {
+#pragma unroll 4
+                for (int s = 0; s < ns; s++)
+                    m |= (unsigned)((__ldg(&A.occ[S.occ[s] + (kb >> 6)].bits) >> (kb & 63)) & 1ull) << s;
+            }
         }
         if (ModeOf<MODE>::count && !upper_only<MODE>(A)) {
             R.found += __popc(m);
@@ -157,16 +195,25 @@ __device__ __forceinline__ void opp_scan(OppRow<MODE, K> &R, const EnumArgs &A, 
     }
 }
 
-template <int MODE, int K>
+// with the choice, as many CTAs per SM as the kernels without it reach by themselves
+template <int MODE, int K, bool CHOICE>
 struct OppMinBlocks {
-    static constexpr int value = MODE == ENUM_SIGMA && K > 4 ? 2 : 3;
+    static constexpr int value = !CHOICE ? (MODE == ENUM_SIGMA && K > 4 ? 2 : 3)
+                                         : (ModeOf<MODE>::count ? 6 : (MODE != ENUM_SIGMA || K <= 2 ? 5 : (K <= 5 ? 4 : 3)));
 };
 
-template <int W, int MODE, int K>
-__global__ void __launch_bounds__(ENUM_THREADS, OppMinBlocks<MODE, K>::value) k_opposite(EnumArgs A, DevInts I) {
-    extern __shared__ uint32_t M[];         // [opp_table(Ub)]
+// CHOICE: tables or lookups for each 32 alpha singles (opp_direct), and nothing
+// where they have no members.  Without it tables always: the choice costs 5 % of
+// a product where it is never taken (24 orbitals, 60,017 determinants: 0.72 to
+// 0.77 ms), so it is taken only where it saves a fifth of the whole pass
+// (k_opp_costs).
+template <int W, int MODE, int K, bool CHOICE>
+__global__ void __launch_bounds__(ENUM_THREADS, OppMinBlocks<MODE, K, CHOICE>::value) k_opposite(EnumArgs A, DevInts I) {
+    extern __shared__ uint32_t M[];         // [opp_table(Ub)], then [opp_rows] places
     __shared__ OppSmem S;
     __shared__ int item_sh;
+    // fill: each row's next slot; count: pairs so far
+    int64_t *const pos = reinterpret_cast<int64_t *>(M + opp_places(A.n_beta_str));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *queue = S.queue[warp];
     unsigned long long cand = 0;
@@ -182,9 +229,11 @@ __global__ void __launch_bounds__(ENUM_THREADS, OppMinBlocks<MODE, K>::value) k_
         const int last = A.item_end ? A.item_end[item] : (int)(A.ga_off[a + 1] - g_beg);
         const int rows = min(last - first, A.opp_rows);
         const Str<W> Aa = load_str<W>(A.astr, a);
-        for (int r = threadIdx.x; r < rows; r += ENUM_THREADS) {
-            const int64_t i = A.row_det[g_beg + first + r];
-            S.pos[r] = ModeOf<MODE>::fill ? A.rowptr[i] + A.part_off[i] : 0;
+        if (ModeOf<MODE>::fill || ModeOf<MODE>::count) {
+            for (int r = threadIdx.x; r < rows; r += ENUM_THREADS) {
+                const int64_t i = A.row_det[g_beg + first + r];
+                pos[r] = ModeOf<MODE>::fill ? A.rowptr[i] + A.part_off[i] : 0;
+            }
         }
         for (int64_t s0 = s_beg; s0 < s_end; s0 += 32) {
             const int ns = (int)min((int64_t)32, s_end - s0);
@@ -196,12 +245,25 @@ __global__ void __launch_bounds__(ENUM_THREADS, OppMinBlocks<MODE, K>::value) k_
                 if (!ModeOf<MODE>::count) move_info<W>(Aa, load_str<W>(A.astr, k), pq, neg);
                 S.pq[threadIdx.x] = (pq << 1) | (neg & 1);
             }
-            for (int64_t k0 = 0; k0 < A.n_beta_str; k0 += OPP_RANGE) {
-                const int range = (int)min((int64_t)OPP_RANGE, A.n_beta_str - k0);
+            bool direct = false;
+            if constexpr (CHOICE) {
+                if (warp == 0) {
+                    const int k = lane < ns ? A.as_idx[s0 + lane] : -1;
+                    const int len = __reduce_add_sync(0xffffffffu, k < 0 ? 0 : (int)(A.ow_off[k + 1] - A.ow_off[k]));
+                    if (lane == 0) S.members = len;
+                }
+                __syncthreads();
+                const int members = S.members;
+                if (members == 0) continue;               // the same for all threads
+                direct = opp_direct(rows, A.opp_beta_singles, ns, members, A.n_beta_str);
+            }
+            // looked up: one round without a table
+            for (int64_t k0 = 0; k0 < (CHOICE && direct ? 1 : A.n_beta_str); k0 += OPP_RANGE) {
+                const int range = CHOICE && direct ? 0 : (int)min((int64_t)OPP_RANGE, A.n_beta_str - k0);
                 for (int e = threadIdx.x; e < range; e += ENUM_THREADS) M[e] = 0u;
                 __syncthreads();
                 // a warp per single: its members' bits
-                for (int s = warp; s < ns; s += ENUM_NW) {
+                for (int s = warp; s < (CHOICE && direct ? 0 : ns); s += ENUM_NW) {
                     const int k = A.as_idx[s0 + s];
                     const int64_t end = A.ow_off[k + 1];
                     for (int64_t p = A.ow_off[k] + lane; p < end; p += 32) {
@@ -217,19 +279,19 @@ __global__ void __launch_bounds__(ENUM_THREADS, OppMinBlocks<MODE, K>::value) k_
                     const int b = A.ib[R.i];
                     R.sb = A.bs_off[b];
                     const int n = (int)(A.bs_off[b + 1] - R.sb);
-                    R.pos = S.pos[r];
+                    R.pos = ModeOf<MODE>::fill ? pos[r] : 0;
                     R.found = 0;
                     R.qn = 0;
 #pragma unroll
                     for (int q = 0; q < (K > 0 ? K : 1); q++) R.acc[q] = 0.0;
                     if (MODE == ENUM_GRAD) R.ci = A.x_grouped[R.place];
-                    opp_scan<MODE, K>(R, A, I, S, M, queue, n, (int)k0, range);
+                    opp_scan<MODE, K, CHOICE>(R, A, I, S, M, queue, n, ns, (int)k0, range);
                     if (ModeOf<MODE>::count) {
                         const int f = __reduce_add_sync(0xffffffffu, R.found);
-                        if (lane == 0) S.pos[r] += f;
+                        if (lane == 0) pos[r] += f;
                         if (k0 == 0) cand += lane == 0 ? (unsigned long long)n * ns : 0ull;
                     } else if (ModeOf<MODE>::fill) {
-                        if (lane == 0) S.pos[r] = R.pos;
+                        if (lane == 0) pos[r] = R.pos;
                     } else if (MODE == ENUM_SIGMA) {
                         double s;
                         const int q = warp_sum_many<(K > 0 ? K : 1)>(R.acc, s);
@@ -243,10 +305,36 @@ __global__ void __launch_bounds__(ENUM_THREADS, OppMinBlocks<MODE, K>::value) k_
         if (ModeOf<MODE>::count) {
             __syncthreads();
             for (int r = threadIdx.x; r < rows; r += ENUM_THREADS)
-                A.cnt[A.row_det[g_beg + first + r]] = S.pos[r];
+                A.cnt[A.row_det[g_beg + first + r]] = pos[r];
         }
     }
     if (ModeOf<MODE>::count && lane == 0 && cand) atomicAdd(A.cand, cand);
+}
+
+// Costs of the pass over all items, in opp_direct's units: sums[0] with tables
+// only, sums[1] with the choice.  A warp per group.
+static __global__ void k_opp_costs(const int64_t *__restrict__ off, int64_t n_groups, int rows_max,
+                                   const int64_t *__restrict__ as_off, const int32_t *__restrict__ as_idx,
+                                   int64_t beta_singles, int64_t U, unsigned long long *__restrict__ sums) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long table = 0, least = 0;
+    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < n_groups;
+         a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int64_t g = off[a + 1] - off[a], items = (g + rows_max - 1) / rows_max;
+        const int64_t rows = (g + items - 1) / items, s_end = as_off[a + 1];
+        for (int64_t s0 = as_off[a]; s0 < s_end; s0 += 32) {
+            const int ns = (int)min((int64_t)32, s_end - s0);
+            const int k = lane < ns ? as_idx[s0 + lane] : -1;
+            const int members = __reduce_add_sync(0xffffffffu, k < 0 ? 0 : (int)(off[k + 1] - off[k]));
+            const int64_t t = opp_table_cost(rows, beta_singles, members, U), d = opp_lookup_cost(rows, beta_singles, ns);
+            table += (unsigned long long)(items * t);
+            least += (unsigned long long)(items * (d < t ? d : t));
+        }
+    }
+    if (lane == 0 && table) {
+        atomicAdd(&sums[0], table);
+        atomicAdd(&sums[1], least);
+    }
 }
 
 }  // namespace shci
