@@ -26,6 +26,7 @@
 // choice per alpha single in enumerate.cuh; count 66.4, 12.7 and 25.6.
 #pragma once
 #include "enumerate.cuh"
+#include "prims.cuh"
 
 namespace shci {
 
@@ -145,6 +146,19 @@ __device__ __forceinline__ void opp_flush(OppRow<MODE, K> &R, const EnumArgs &A,
     }
 }
 
+// the first 32 queued pairs, and the rest moved up
+template <int MODE, int K>
+__device__ __forceinline__ void opp_flush_full(OppRow<MODE, K> &R, const EnumArgs &A, const DevInts &I, const OppSmem &S,
+                                               uint32_t *queue) {
+    const int lane = threadIdx.x & 31;
+    opp_flush<MODE, K>(R, A, I, S, queue, 32);
+    R.qn -= 32;
+    const uint32_t keep = lane < R.qn ? queue[32 + lane] : 0u;
+    __syncwarp();
+    if (lane < R.qn) queue[lane] = keep;
+    __syncwarp();
+}
+
 // one row's beta singles against the table of strings [k0, k0 + range), or (only
 // with CHOICE: range 0) against the ns singles' rows of the bitmap
 template <int MODE, int K, bool CHOICE>
@@ -169,6 +183,41 @@ __device__ __forceinline__ void opp_scan(OppRow<MODE, K> &R, const EnumArgs &A, 
             R.found += __popc(m);
             continue;
         }
+        // Rows of the upper triangle: the set bits lane by lane, 32 at a time, so that a
+        // row's pairs of one beta string stand together.  Such determinants are near
+        // one another in V as a selection orders it, and the product scatters into
+        // them (24 orbitals, 1.2e5 determinants, one vector: 351 us by scans of the
+        // groups, 328 in this order; 60,017: a bit at a time of every lane is as slow
+        // as a random order, 236 us, this 217, ascending determinants 216).
+        if (upper_only<MODE>(A) && !ModeOf<MODE>::count) {
+            const int own = __popc(m), incl = warp_incl_scan(own), total = __shfl_sync(0xffffffffu, incl, 31);
+            for (int q0 = 0; q0 < total; q0 += 32) {
+                const int slot = q0 + lane;
+                int q = 0;                                // the lane that holds bit `slot`: the first with incl > slot
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1) {
+                    const int v = __shfl_sync(0xffffffffu, incl, q + step - 1);
+                    if (v <= slot) q += step;
+                }
+                q = min(q, 31);
+                unsigned w = __shfl_sync(0xffffffffu, m, q);
+                int nth = slot - __shfl_sync(0xffffffffu, incl - own, q), bit = 0;
+#pragma unroll
+                for (int half = 16; half >= 1; half >>= 1) {          // its nth set bit
+                    const int c = __popc(w & ((1u << half) - 1u));
+                    if (nth >= c) {
+                        nth -= c;
+                        w >>= half;
+                        bit += half;
+                    }
+                }
+                if (slot < total) queue[R.qn + lane] = ((uint32_t)(t0 + q) << 5) | (uint32_t)bit;
+                R.qn += min(32, total - q0);
+                __syncwarp();
+                if (R.qn >= 32) opp_flush_full<MODE, K>(R, A, I, S, queue);
+            }
+            continue;
+        }
         // a round takes one bit of every lane that has some left
         for (unsigned some = __ballot_sync(0xffffffffu, m != 0u); some; some = __ballot_sync(0xffffffffu, m != 0u)) {
             if (m) {
@@ -177,14 +226,7 @@ __device__ __forceinline__ void opp_scan(OppRow<MODE, K> &R, const EnumArgs &A, 
             }
             R.qn += __popc(some);
             __syncwarp();
-            if (R.qn >= 32) {
-                opp_flush<MODE, K>(R, A, I, S, queue, 32);
-                R.qn -= 32;
-                const uint32_t keep = lane < R.qn ? queue[32 + lane] : 0u;
-                __syncwarp();
-                if (lane < R.qn) queue[lane] = keep;
-                __syncwarp();
-            }
+            if (R.qn >= 32) opp_flush_full<MODE, K>(R, A, I, S, queue);
         }
     }
     // the queue names this table's singles: empty it before they are replaced

@@ -1,6 +1,8 @@
 // sigma = H c from the upper triangle of H alone (SHCI_STORED_UPPER), the form
 // the paper stores (Sec. V, "Hamiltonian Matrix"): each stored pair i < j is
 // applied in both directions, the transposed half by FP64 atomic adds into L2.
+#include <algorithm>
+
 #include "enum_launch.cuh"
 
 namespace shci {
@@ -15,6 +17,10 @@ constexpr int UPPER_THREADS = 256;
 // bound it (four vectors on the 1e6 heat-bath space: 0.81 of the measured
 // atomic rate); the shapes tried (rows per group / nonzeros per lane per step
 // / CTAs per SM: 4/4/3, 4/2/4, 2/4/4, 4/4/2) were within 3 % of one another.
+// FEW: a row per warp and four nonzeros per lane and step, for spaces whose
+// groups of R rows would not fill the GPU's warps: there the chain of loads of a
+// warp's rows is the time (24 orbitals, one vector: 5,003 determinants 65 to
+// 47 us, 60,017 210 to 157; eight vectors, 5,003: 142 to 126).
 #ifndef SHCI_UPPER_R
 #define SHCI_UPPER_R 4
 #endif
@@ -24,10 +30,10 @@ constexpr int UPPER_THREADS = 256;
 #ifndef SHCI_UPPER_MINB
 #define SHCI_UPPER_MINB 3
 #endif
-template <int K, bool INTER>
+template <int K, bool INTER, bool FEW = false>
 struct UpperRows {
-    static constexpr int R = K <= 2 ? SHCI_UPPER_R : (K <= 4 ? 2 : 1);
-    static constexpr int SR = K <= 2 ? SHCI_UPPER_SR : 2;
+    static constexpr int R = FEW ? 1 : (K <= 2 ? SHCI_UPPER_R : (K <= 4 ? 2 : 1));
+    static constexpr int SR = FEW ? 4 : (K <= 2 ? SHCI_UPPER_SR : 2);
     static constexpr int MINB = K <= 2 ? SHCI_UPPER_MINB : 1;
 };
 
@@ -39,12 +45,12 @@ __global__ void k_sigma_diag(int64_t n, const double *__restrict__ diag, const d
         y[e] = diag[INTER ? e / K : e % n] * x[e];
 }
 
-template <int K, bool INTER>
-__global__ void __launch_bounds__(UPPER_THREADS, UpperRows<K, INTER>::MINB) k_sigma_upper(
+template <int K, bool INTER, bool FEW>
+__global__ void __launch_bounds__(UPPER_THREADS, UpperRows<K, INTER, FEW>::MINB) k_sigma_upper(
     int64_t n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col, const double *__restrict__ val,
     const double *__restrict__ x, double *y) {
-    constexpr int SR = UpperRows<K, INTER>::SR;
-    constexpr int R = UpperRows<K, INTER>::R;
+    constexpr int SR = UpperRows<K, INTER, FEW>::SR;
+    constexpr int R = UpperRows<K, INTER, FEW>::R;
     constexpr int LOG_R = R == 8 ? 3 : (R == 4 ? 2 : (R == 2 ? 1 : 0));
     const int lane = threadIdx.x & 31;
     const int64_t n_groups = (n + R - 1) / R;
@@ -125,11 +131,24 @@ __global__ void __launch_bounds__(UPPER_THREADS, UpperRows<K, INTER>::MINB) k_si
     }
 }
 
+// A row per warp up to as many rows as the grid has warps for groups of R (64 per
+// SM), twice as many for one vector: always, it takes 5 to 20 % longer from four
+// vectors on and 36,007 determinants, or eight and 20,011, whose atomics bound it.
+template <int K>
+constexpr int UPPER_FEW = K == 1 ? 128 : 64;
+
 template <int K, bool INTER>
 static void launch_upper(shci_ctx *c, const double *x, double *y) {
+    constexpr int R = UpperRows<K, INTER>::R;
     const int blocks = c->n_sm * (2048 / UPPER_THREADS);
     k_sigma_diag<K, INTER><<<blocks, UPPER_THREADS, 0, c->st>>>(c->n_det, c->diag.p, x, y);
-    k_sigma_upper<K, INTER><<<blocks, UPPER_THREADS, 0, c->st>>>(c->n_det, c->rowptr.p, c->col.p, c->val.p, x, y);
+    if (c->n_det <= (int64_t)c->n_sm * UPPER_FEW<K> * R) {
+        const int rows = (int)std::max<int64_t>(1, ceil_div(c->n_det, UPPER_THREADS / 32));
+        k_sigma_upper<K, INTER, true><<<rows, UPPER_THREADS, 0, c->st>>>(c->n_det, c->rowptr.p, c->col.p, c->val.p, x, y);
+    } else {
+        k_sigma_upper<K, INTER, false><<<blocks, UPPER_THREADS, 0, c->st>>>(c->n_det, c->rowptr.p, c->col.p, c->val.p, x,
+                                                                           y);
+    }
     KERNEL_CHECK();
 }
 
