@@ -383,7 +383,7 @@ static void make_items_part(shci_ctx *c, const int64_t *off, const int64_t *g_ne
 // taken from the determinant-ordered member lists rdet / rstr
 template <int W, int MODE>
 static void extend_pass(shci_ctx *c, EnumArgs E, const DevInts &I, bool alpha_part, const PartItems &items,
-                        const int32_t *rdet, const uint64_t *rstr) {
+                        const int32_t *rdet, const uint64_t *rstr, bool opp = false) {
     if (items.n == 0) return;
     E.item_group = items.group.p;
     E.item_first = items.first.p;
@@ -391,7 +391,7 @@ static void extend_pass(shci_ctx *c, EnumArgs E, const DevInts &I, bool alpha_pa
     E.n_items = items.n;
     E.row_det = rdet;
     E.row_str = rstr;
-    launch_enum<W, MODE, 0>(c, E, I, alpha_part);
+    launch_enum<W, MODE, 0>(c, E, I, alpha_part, opp);
 }
 
 template <int W, int MODE>
@@ -578,11 +578,10 @@ __global__ void k_occ_place(const int64_t *__restrict__ off, int64_t Ua, int64_t
     }
 }
 
-// the bitmap of determinants [from, n), whose members begin at off
+// the bitmap of determinants [from, n), whose members begin at off, in the cells of occ
 static void occupancy(shci_ctx *c, int64_t from, const int64_t *off, DevBuf<OccCell> &occ) {
     cudaStream_t st = c->st;
     const size_t cells = (size_t)(c->Ua * c->occ_words);
-    occ.alloc(cells);
     CUDA_TRY(cudaMemsetAsync(occ.p, 0, sizeof(OccCell) * cells, st));
     k_occ_set<<<grid_for(c->n_det - from), 256, 0, st>>>(c->ia.p, c->ib.p, from, c->n_det, c->occ_words, occ.p);
     k_occ_place<<<grid_for(c->Ua * 32), 256, 0, st>>>(off, c->Ua, c->occ_words, occ.p);
@@ -629,22 +628,24 @@ static void opposite_pass_setup(shci_ctx *c) {
 
 // Beta-single lists and the occupancy bitmap for the opposite-spin doubles.
 // SHCI_OPP_SPIN=scan: no bitmap, every alpha single's group is scanned;
-// lookup: every (alpha single, beta single) pair is looked up; auto (default):
-// the enumeration chooses per alpha single (scan the group when it is short
-// compared with the CTA's beta-single lists, SHCI_OPP_FACTOR times at most).
-// The bitmap is skipped when it would take more than 4 GB.
+// lookup: every (alpha single, beta single) pair is looked up; auto (default): a
+// pass of their own (opposite.cuh), and in a batch's products the choice per alpha
+// single (scan the group when it is short compared with the CTA's beta-single
+// lists, SHCI_OPP_FACTOR times at most).  The bitmap is skipped above 3.3e8 cells
+// (16 bytes each, 5.3 GB) and where the memory for it is not free.
+constexpr double OCC_CELLS = 4.0e9 / 12.0;
+
 template <int W>
 static void opposite_spin_setup(shci_ctx *c) {
-    cudaStream_t st = c->st;
     c->n_beta_singles = string_singles<W>(c, c->bstr.p, c->Ub, c->n_beta, c->bs_off, c->bs_idx);
     c->occ_words = (c->Ub + 63) / 64;
-    const double bytes = (double)c->Ua * c->occ_words * 12.0;
     const char *env = getenv("SHCI_OPP_SPIN");
     std::string pref = env ? env : "auto";
     c->opp_lookup = false;
     c->opp_hybrid = false;
     c->opp_pass = false;
-    if (pref == "scan" || bytes > 4.0e9) {
+    if (pref == "scan" || (double)c->Ua * c->occ_words > OCC_CELLS ||
+        !try_alloc(c->occ, (size_t)(c->Ua * c->occ_words))) {
         c->occ.reset();
         c->bs_pair.reset();
         c->ga_ib.reset();
@@ -663,13 +664,14 @@ static void opposite_spin_setup(shci_ctx *c) {
 
 // SHCI_AUTO: store both triangles of H when their nnz_full elements (12 bytes
 // each) fit 80 % of the free device memory and the context's budget, else the
-// upper triangle alone when its nnz_full / 2 elements fit, else apply H on the fly
-static int decide_mode(shci_ctx *c, int mode, int64_t nnz_full) {
+// upper triangle alone when its nnz_full / 2 elements fit, else apply H on the fly.
+// held: bytes taken now that are given back before the call returns
+static int decide_mode(shci_ctx *c, int mode, int64_t nnz_full, double held = 0.0) {
     if (mode != SHCI_AUTO) return mode;
     size_t free_b = 0, total_b = 0;
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     double need = (double)nnz_full * 12.0;
-    double cap = 0.8 * (double)free_b;
+    double cap = std::min(0.8 * ((double)free_b + held), (double)free_b);
     if (c->stored_budget >= 0.0) cap = std::min(cap, c->stored_budget);
     if (need < cap) return SHCI_STORED;
     return 0.5 * need < cap ? SHCI_STORED_UPPER : SHCI_ON_THE_FLY;
@@ -890,9 +892,10 @@ static void new_members(shci_ctx *c, int64_t n_old, DevBuf<int64_t> &off, DevBuf
 // Algorithms 1 and 2).  The lists are rebuilt for all of V; a second copy of
 // the per-string groups with members in determinant order puts each group's
 // new members in a suffix.  New rows take every candidate from the usual
-// lists (group scans or bitmap lookups, as in a full build); old rows take
-// only the new candidates, the suffixes of the determinant-ordered groups
-// (j >= s), each warp reading its row's suffixes directly.  The old rows are
+// lists, as in a full build; old rows take only the new candidates (j >= s): the
+// same-spin ones in the suffixes of the determinant-ordered groups, each warp
+// reading its row's suffix directly, the opposite-spin ones by the pass over a
+// bitmap of the new members alone, or in the suffixes too.  The old rows are
 // copied into the grown matrix ahead of their new elements.
 // events on the context's stream marking the parts of an incremental update
 struct PhaseMarks {
@@ -956,10 +959,18 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     Ao.n_old = n_old;
     Ao.ga_new = ga_new.p;
     Ao.gb_new = gb_new.p;
-    // and the opposite-spin pass's view of the new members alone
+    // and the opposite-spin pass's view of the new members alone: its bitmap is as
+    // large as V's however few they are, and the old and the grown matrix are held
+    // beside it.  So only where it is small, or at most 4 KB per new determinant (which
+    // bring some 14 KB of elements each), and free; otherwise the old rows read the
+    // new members of their alpha singles' groups in the alpha-grouped part.
     DevBuf<int32_t> new_det, new_ib;
     DevBuf<OccCell> new_occ;
-    if (c->opp_pass) {
+    const int64_t cells = c->Ua * c->occ_words;
+    const bool opp_old = c->opp_pass && sizeof(OccCell) * (double)cells <= 6.4e7 + 4096.0 * (double)(n - n_old) &&
+                         try_alloc(new_occ, (size_t)cells);
+    const double new_occ_bytes = sizeof(OccCell) * (double)new_occ.n;
+    if (opp_old) {
         new_members(c, n_old, off_tmp, new_det);
         new_ib.alloc((size_t)(n - n_old));
         k_member_index<<<grid_for(n - n_old), 256, 0, st>>>(new_det.p, n - n_old, c->ib.p, new_ib.p);
@@ -995,13 +1006,11 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     extend_pass<W, ENUM_COUNT_INC>(c, Ao, I, false, ib_old, gbd.p, gbs.p);
     An.cnt = Ao.cnt = cnt_a.p;
     extend_pass<W, ENUM_COUNT_INC>(c, An, I, true, ia_new, gad.p, gas.p);
-    extend_pass<W, ENUM_COUNT_INC>(c, Ao, I, true, ia_old, gad.p, gas.p);
+    extend_pass<W, ENUM_COUNT_INC>(c, Ao, I, true, ia_old, gad.p, gas.p, !opp_old);
     An.cnt = Ao.cnt = cnt_o.p;
     CUDA_TRY(cudaMemsetAsync(cnt_o.p, 0, sizeof(int64_t) * n, st));
-    if (c->opp_pass) {
-        extend_opposite<W, ENUM_COUNT_INC>(c, An, I, io_new, gad.p);
-        extend_opposite<W, ENUM_COUNT_INC>(c, Ao, I, io_old, gad.p);
-    }
+    if (c->opp_pass) extend_opposite<W, ENUM_COUNT_INC>(c, An, I, io_new, gad.p);
+    if (opp_old) extend_opposite<W, ENUM_COUNT_INC>(c, Ao, I, io_old, gad.p);
     k_extend_rows<<<grid_for(n), 256, 0, st>>>(c->rowptr.p, n_old, c->cnt_b.p, cnt_a.p, cnt_o.p, n, len.p, off_b.p,
                                                off_a.p, off_o.p);
     KERNEL_CHECK();
@@ -1020,7 +1029,7 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     // one (both triangles may then fall back to the upper one, by a rebuild)
     int mode = c->mode;
     if (mode != SHCI_ON_THE_FLY && c->mode_req == SHCI_AUTO) {
-        const int fit = decide_mode(c, SHCI_AUTO, nnz_full);
+        const int fit = decide_mode(c, SHCI_AUTO, nnz_full, new_occ_bytes);
         if (fit == SHCI_ON_THE_FLY) mode = SHCI_ON_THE_FLY;
         else if (mode == SHCI_STORED && fit == SHCI_STORED_UPPER) return false;
     }
@@ -1044,12 +1053,10 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
         extend_pass<W, ENUM_FILL_INC>(c, Ao, I, false, ib_old, gbd.p, gbs.p);
         An.part_off = Ao.part_off = off_a.p;
         extend_pass<W, ENUM_FILL_INC>(c, An, I, true, ia_new, gad.p, gas.p);
-        extend_pass<W, ENUM_FILL_INC>(c, Ao, I, true, ia_old, gad.p, gas.p);
-        if (c->opp_pass) {
-            An.part_off = Ao.part_off = off_o.p;
-            extend_opposite<W, ENUM_FILL_INC>(c, An, I, io_new, gad.p);
-            extend_opposite<W, ENUM_FILL_INC>(c, Ao, I, io_old, gad.p);
-        }
+        extend_pass<W, ENUM_FILL_INC>(c, Ao, I, true, ia_old, gad.p, gas.p, !opp_old);
+        An.part_off = Ao.part_off = off_o.p;
+        if (c->opp_pass) extend_opposite<W, ENUM_FILL_INC>(c, An, I, io_new, gad.p);
+        if (opp_old) extend_opposite<W, ENUM_FILL_INC>(c, Ao, I, io_old, gad.p);
         c->col.swap(col);
         c->val.swap(val);
     } else {

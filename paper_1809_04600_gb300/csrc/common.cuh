@@ -69,6 +69,20 @@ struct DevBuf {
     }
 };
 
+// alloc for a buffer the caller can do without: false, and the buffer empty, when
+// the memory is not there
+template <typename T>
+inline bool try_alloc(DevBuf<T> &b, size_t count) {
+    try {
+        b.alloc(count);
+    } catch (const ShciError &e) {
+        if (e.code != SHCI_ERR_OOM) throw;
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
 // ---------------------------------------------------------------- device helpers
 
 // *p += v as a global-memory reduction (no result returned).  For a pointer

@@ -46,8 +46,10 @@ inline EnumArgs enum_args(const shci_ctx *c) {
 
 // One pass of the alpha-grouped (alpha_part) or beta-grouped enumeration:
 // a persistent grid whose CTAs take work items from an atomic counter.
+// opp: the opposite-spin doubles in the alpha-grouped part although the context
+// has a pass for them.
 template <int W, int MODE, int K>
-void launch_enum(shci_ctx *c, EnumArgs A, const DevInts &I, bool alpha_part) {
+void launch_enum(shci_ctx *c, EnumArgs A, const DevInts &I, bool alpha_part, bool opp = false) {
     CUDA_TRY(cudaMemsetAsync(c->counter.p + 1, 0, sizeof(int), c->st));
     if (!A.item_group) {                    // the context's items unless the caller gave its own
         A.item_group = alpha_part ? c->item_a_group.p : c->item_b_group.p;
@@ -55,7 +57,7 @@ void launch_enum(shci_ctx *c, EnumArgs A, const DevInts &I, bool alpha_part) {
         A.n_items = alpha_part ? c->n_items_a : c->n_items_b;
     }
     const int blocks = c->n_sm * (2048 / ENUM_THREADS);
-    if (alpha_part && c->opp_pass) k_enum_alpha<W, MODE, K, false><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
+    if (alpha_part && c->opp_pass && !opp) k_enum_alpha<W, MODE, K, false><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
     else if (alpha_part) k_enum_alpha<W, MODE, K, true><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
     else k_enum_beta<W, MODE, K><<<blocks, ENUM_THREADS, 0, c->st>>>(A, I);
     KERNEL_CHECK();

@@ -1,0 +1,81 @@
+"""Calls at the limit of the device's memory: growth beside a large occupancy
+bitmap (the bitmap of the new members alone would not fit), and a build without
+room for a bitmap.  Results as with room to spare, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import shci_synth as S
+from tests import gpu_common as G
+from tests.test_gpu_extend import _extend
+from tests.test_gpu_opposite import _dets, _strings
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+def _free():
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _leave(nbytes):
+    """Take all free memory but nbytes."""
+    return torch.empty(max(_free() - int(nbytes), 0), dtype=torch.uint8, device="cuda")
+
+
+def _sparse():
+    """26 orbitals, 5 electrons a spin, random strings: a bitmap of some 65,000 x 900 cells, 0.9 GB."""
+    rng = np.random.default_rng(3)
+    s = _strings(range(26), 5)
+    pick = rng.choice(s.size * s.size, 150_011, replace=False)
+    h, eri, ec = S.integrals(26, 5, 41)
+    return h, eri, ec, _dets(s[pick // s.size], s[pick % s.size], 1)
+
+
+@pytest.mark.parametrize("upper", [False, True])
+def test_growth_beside_a_large_bitmap(upper):
+    P = G.lib()
+    h, eri, ec, dets = _sparse()
+    head = dets.shape[0] - 29
+    mode = P.SHCI_STORED_UPPER if upper else P.SHCI_STORED
+    B = G.Built(P, h, eri, ec, dets[:head], 5, 5, mode=mode)
+    taken = _leave(600 * MB)
+    try:
+        _extend(P, B, dets[head:])
+    finally:
+        del taken
+        _free()
+    assert B.stats()["extend_incremental"] == 1
+    F = G.Built(P, h, eri, ec, dets, 5, 5, mode=mode)
+    assert F.nnz == B.nnz
+    for x, y in zip(F.pairs(), B.pairs()):
+        assert np.array_equal(x, y)
+    x = S.random_vectors(dets.shape[0], 2, 4)
+    # the same terms in another order: below 1e-12 of the largest sum of magnitudes for m < 4500 terms
+    ii, jj, vv = F.pairs()
+    rows = np.abs(F.diag())
+    np.add.at(rows, ii, np.abs(vv))
+    np.add.at(rows, jj, np.abs(vv))
+    assert np.all(np.abs(F.sigma(x) - B.sigma(x)) <= 1e-12 * rows * np.max(np.abs(x)))
+    F.close()
+    B.close()
+
+
+def test_build_without_room_for_a_bitmap():
+    P = G.lib()
+    h, eri, ec, dets = _sparse()
+    F = G.Built(P, h, eri, ec, dets, 5, 5)
+    want = F.pairs()
+    F.close()
+    taken = _leave(600 * MB)
+    try:
+        B = G.Built(P, h, eri, ec, dets, 5, 5)
+    finally:
+        del taken
+        _free()
+    for x, y in zip(want, B.pairs()):
+        assert np.array_equal(x, y)
+    B.close()

@@ -1,8 +1,8 @@
 """Products over the upper triangle with a row per warp (small spaces) and with
 groups of rows, on both sides of the sizes where the form changes, against the
 product over both triangles: the same m terms per row in another order differ by
-less than 2 m 2^-53 of the sum of their magnitudes, below 1e-12 of it for the
-m < 4500 terms of a row here."""
+less than 2 m 2^-53 of the sum of their magnitudes, below 2e-12 of it for the
+at most 7,875 excitations of a determinant here."""
 import numpy as np
 import pytest
 import torch
@@ -33,4 +33,4 @@ def test_both_sides_of_the_change_of_form(k, side):
     for q in range(k):
         scale[q] += np.bincount(ii, np.abs(vv) * a[q, jj], edge + side)
         scale[q] += np.bincount(jj, np.abs(vv) * a[q, ii], edge + side)
-    assert np.all(np.abs(got - want) <= 1e-12 * scale)
+    assert np.all(np.abs(got - want) <= 2e-12 * scale)
