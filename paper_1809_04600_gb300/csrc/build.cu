@@ -729,7 +729,8 @@ static void lists_w(shci_ctx *c) {
 // elements, when that is little work beside them: a table entry costs about
 // what a single in full does, a row of V has some ten to thirty, evaluated
 // once to store H and in every product on the fly (but a batch's systems share
-// the memory).  At most a 32nd of the free memory (64 MB in any case).  1e6
+// the memory).  At most a 32nd of the free memory (64 MB in any case), taken
+// after the matrix: where the two do not fit together there are no tables.  1e6
 // determinants of 24 orbitals: the same-spin kernels of a product on the fly
 // 4.5 to 1.7 ms each, those that write H 7.9 and 6.3 to 3.6 and 3.9.
 template <int W>
@@ -743,7 +744,8 @@ static void connectivity_moves(shci_ctx *c, int mode) {
         CUDA_TRY(cudaMemGetInfo(&fr, &tot));
         fits = entries * 16.0 <= (double)fr / 32.0;
     }
-    if (!fits) {
+    if (!fits || !try_alloc(c->move_a, (size_t)(c->Ua * c->n_orb * (c->n_orb + 1))) ||
+        !try_alloc(c->move_b, (size_t)(c->Ub * c->n_orb * (c->n_orb + 1)))) {
         c->move_a.reset();
         c->move_b.reset();
         return;
@@ -795,6 +797,18 @@ static void count_w(shci_ctx *c, bool upper) {
     c->rows_upper = upper;
 }
 
+// The arrays of a stored H.  Without room for them the single-move tables of an
+// earlier form or space go first.
+static void alloc_matrix(shci_ctx *c, int64_t nnz, DevBuf<int32_t> &col, DevBuf<double> &val) {
+    const size_t m = (size_t)std::max<int64_t>(nnz, 1);
+    if (try_alloc(col, m) && try_alloc(val, m)) return;
+    c->have_moves = false;
+    c->move_a.reset();
+    c->move_b.reset();
+    col.alloc(m);
+    val.alloc(m);
+}
+
 // Store H in mode SHCI_STORED or SHCI_STORED_UPPER after the lists and a
 // count pass (recounted when the row lengths held are of the other form).
 template <int W>
@@ -802,10 +816,8 @@ static void store_w(shci_ctx *c, int mode) {
     const bool upper = mode == SHCI_STORED_UPPER;
     if (c->rows_upper != upper) count_w<W>(c, upper);
     c->mode = mode;
+    alloc_matrix(c, stored_entries(c), c->col, c->val);
     if (!c->have_moves) connectivity_moves<W>(c, mode);
-    const int64_t nnz = stored_entries(c);
-    c->col.alloc((size_t)std::max<int64_t>(nnz, 1));
-    c->val.alloc((size_t)std::max<int64_t>(nnz, 1));
     DevInts I = dev_ints(c);
     EnumArgs A = enum_args(c);
     A.rowptr = c->rowptr.p;
@@ -945,7 +957,6 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
         make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 0, rows, io_old);
         make_items_part(c, c->ga_off.p, ga_new.p, c->Ua, 1, rows, io_new);
     }
-    connectivity_moves<W>(c, c->mode);
     // new rows: every candidate, the context's lists
     EnumArgs An = enum_args(c);
     // old rows: new candidates only, determinant-ordered lists
@@ -1036,14 +1047,16 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
     if (mode == SHCI_STORED || mode == SHCI_STORED_UPPER) {
         DevBuf<int32_t> col;
         DevBuf<double> val;
-        col.alloc((size_t)std::max<int64_t>(nnz, 1));
-        val.alloc((size_t)std::max<int64_t>(nnz, 1));
+        alloc_matrix(c, nnz, col, val);
+        connectivity_moves<W>(c, mode);
         const unsigned gw = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n_old, 8), (int64_t)c->n_sm * 8));
         k_copy_rows<<<gw, 256, 0, st>>>(c->rowptr.p, c->col.p, c->val.p, n_old, rowptr.p, col.p, val.p);
         KERNEL_CHECK();
         LAUNCHED(1);
         pm.mark(3);
         for (EnumArgs *E : {&An, &Ao}) {
+            E->ma = c->have_moves ? c->move_a.p : nullptr;
+            E->mb = c->have_moves ? c->move_b.p : nullptr;
             E->rowptr = rowptr.p;
             E->col = col.p;
             E->val = val.p;
@@ -1063,6 +1076,7 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
         pm.mark(3);
         c->col.reset();
         c->val.reset();
+        connectivity_moves<W>(c, mode);
     }
     pm.mark(4);
     c->mode = mode;

@@ -286,7 +286,7 @@ struct MoveTables {
 // a quarter, since the tables are written and read back) and takes at most a
 // sixteenth of the free memory; otherwise S keeps evaluating each move.
 template <int W>
-static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double rows, MoveTables &T) {
+static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double rows, MoveTables &T, bool own) {
     const int n = c->n_orb;
     if (c->have_moves) {                    // the connectivity's own
         S.ma = c->move_a.p;
@@ -295,6 +295,7 @@ static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double row
         S.ib = c->ib.p;
         return;
     }
+    if (!own) return;
     const int64_t np = (int64_t)n * (n + 1) / 2;
     const double entries = (double)(c->Ua + c->Ub) * np;
     const double moves = rows * ((double)S.na * (n - S.na) + (double)S.nb * (n - S.nb));
@@ -307,6 +308,18 @@ static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double row
     S.mb = T.b.p;
     S.ia = c->ia.p;
     S.ib = c->ib.p;
+}
+
+// f(true), and where the memory runs out f(false): without tables of the call's own
+template <typename F>
+static void with_tables(F f) {
+    try {
+        f(true);
+    } catch (const ShciError &e) {
+        if (e.code != SHCI_ERR_OOM) throw;
+        cudaGetLastError();
+        f(false);
+    }
 }
 
 // The test |v| cmax >= eps without FP64 arithmetic where the answer is not
@@ -729,7 +742,8 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_compact(const uint64_t *__r
 }
 
 template <int W, int KW>
-static void select_w(shci_ctx *c, int k, const double *cd, double eps1, DevBuf<uint64_t> &result, int64_t &n_new) {
+static void select_w(shci_ctx *c, int k, const double *cd, double eps1, DevBuf<uint64_t> &result, int64_t &n_new,
+                     bool tables) {
     cudaStream_t st = c->st;
     const int64_t n = c->n_det;
     SelArgs S = sel_args(c, eps1);
@@ -737,7 +751,7 @@ static void select_w(shci_ctx *c, int k, const double *cd, double eps1, DevBuf<u
     S.c = cd;
     const DevInts I = dev_ints(c);
     MoveTables moves;
-    tabulate_moves<W>(c, S, I, (double)n, moves);
+    tabulate_moves<W>(c, S, I, (double)n, moves, tables);
     DevBuf<unsigned long long> cnt;
     DevBuf<int64_t> off, tmp;
     const int64_t total = count_candidates<W, KW, false>(c, S, I, cnt, off, tmp);
@@ -1108,12 +1122,12 @@ static void reduce_terms(shci_ctx *c, SelArgs &S, const DevInts &I, int64_t tota
 
 template <int W, int KW>
 static double pt2_w(shci_ctx *c, const double *cd, double e_var, double eps2, int nbatch, int64_t &n_pert,
-                    int &nbatch_used, int64_t &candidates) {
+                    int &nbatch_used, int64_t &candidates, bool tables) {
     SelArgs S = sel_args(c, eps2);
     S.c = cd;
     const DevInts I = dev_ints(c);
     MoveTables moves;
-    tabulate_moves<W>(c, S, I, (double)c->n_det, moves);
+    tabulate_moves<W>(c, S, I, (double)c->n_det, moves, tables);
     TermWork T;
     // batches: enough that one batch's candidates and their sort fit a quarter of free memory
     constexpr double BYTES_PER_CAND = 2.0 * 8 * KW + 8 + 2 * 4;
@@ -1282,7 +1296,8 @@ __global__ void k_check_draws(const int64_t *__restrict__ draws, int64_t m, cons
 
 template <int W, int KW>
 static void pt2_samples_w(shci_ctx *c, const double *cd, double e_var, double eps2, double eps2_d, int64_t n_d,
-                          int n_samples, const int64_t *draws, double *out, int nbatch, const int *batch_of_sample) {
+                          int n_samples, const int64_t *draws, double *out, int nbatch, const int *batch_of_sample,
+                          bool tables) {
     cudaStream_t st = c->st;
     const int64_t n = c->n_det;
     const double csum = abs_sum(c, cd, n);
@@ -1306,7 +1321,7 @@ static void pt2_samples_w(shci_ctx *c, const double *cd, double e_var, double ep
     sib.alloc((size_t)n_d);
     MoveTables moves;
     SelArgs S0 = sel_args(c, eps2);
-    tabulate_moves<W>(c, S0, I, (double)std::min(n_d, n) * n_samples, moves);
+    tabulate_moves<W>(c, S0, I, (double)std::min(n_d, n) * n_samples, moves, tables);
     uint64_t vary = 1;                      // bits of an index of V
     while ((int64_t)vary < n - 1) vary = 2 * vary + 1;
     const int gb = (int)std::min<int64_t>(ceil_div(n_d, SEL_THREADS), (int64_t)c->n_sm * 16);
@@ -1401,8 +1416,8 @@ void pt2_samples(shci_ctx *c, const double *coef, double e_var, double eps2, dou
     }
     std::vector<double> res((size_t)2 * n_samples);
 #define CALL(W, KW) \
-    pt2_samples_w<W, KW>(c, cd, e_var, eps2, eps2_d, n_d, n_samples, dd, res.data(), nbatch, batch_of_sample)
-    DISPATCH_KEYS(c, CALL);
+    pt2_samples_w<W, KW>(c, cd, e_var, eps2, eps2_d, n_d, n_samples, dd, res.data(), nbatch, batch_of_sample, tables)
+    with_tables([&](bool tables) { DISPATCH_KEYS(c, CALL); });
 #undef CALL
     for (size_t e = 0; e < res.size(); e++) out[e] = res[e];
 }
@@ -1481,8 +1496,8 @@ void pt2(shci_ctx *c, const double *coef, double e_var, double eps2, int nbatch,
     int64_t np = 0, cands = 0;
     int used = 0;
     double v = 0.0;
-#define CALL(W, KW) v = pt2_w<W, KW>(c, cd, e_var, eps2, nbatch, np, used, cands)
-    DISPATCH_KEYS(c, CALL);
+#define CALL(W, KW) v = pt2_w<W, KW>(c, cd, e_var, eps2, nbatch, np, used, cands, tables)
+    with_tables([&](bool tables) { DISPATCH_KEYS(c, CALL); });
 #undef CALL
     *e2 = v;
     if (n_pert) *n_pert = np;
@@ -1505,13 +1520,13 @@ void pt2(shci_ctx *c, const double *coef, double e_var, double eps2, int nbatch,
 // unevaluated ones is below 0.4 target (all batches: exact, zero deviation).
 template <int W, int KW>
 static void psto_w(shci_ctx *c, const double *cd, double e_var, double eps_psto, double eps_dtm, int nbatch,
-                   double target, double &est, double &err, int &done) {
+                   double target, double &est, double &err, int &done, bool tables) {
     SelArgs S = sel_args(c, eps_psto);
     S.c = cd;
     S.nbatch = nbatch;
     const DevInts I = dev_ints(c);
     MoveTables moves;
-    tabulate_moves<W>(c, S, I, (double)c->n_det * nbatch, moves);
+    tabulate_moves<W>(c, S, I, (double)c->n_det * nbatch, moves, tables);
     TermWork T;
     sorted_space<W, KW>(c, T.vs);
     double sum = 0.0, sum2 = 0.0;
@@ -1571,8 +1586,9 @@ void pt2_3step(shci_ctx *c, const double *coef, double e_var, double eps2, doubl
     ensure_lists(c);
     if (eps2_psto < eps2_dtm) {
 #define CALL(W, KW)                                                                                            \
-    psto_w<W, KW>(c, cd, e_var, eps2_psto, eps2_dtm, nbatch_psto, target, out->psto, out->psto_err, out->psto_batches)
-        DISPATCH_KEYS(c, CALL);
+    psto_w<W, KW>(c, cd, e_var, eps2_psto, eps2_dtm, nbatch_psto, target, out->psto, out->psto_err, out->psto_batches, \
+                  tables)
+        with_tables([&](bool tables) { DISPATCH_KEYS(c, CALL); });
 #undef CALL
     }
     // 3: stochastic at eps2, minus its eps2_psto part; one batch per sample, drawn
@@ -1666,8 +1682,8 @@ void select_dets(shci_ctx *c, int k, const double *coef, double eps1, int mem, i
     }
     DevBuf<uint64_t> result;
     int64_t n_new = 0;
-#define CALL(W, KW) select_w<W, KW>(c, k, cd, eps1, result, n_new)
-    DISPATCH_KEYS(c, CALL);
+#define CALL(W, KW) select_w<W, KW>(c, k, cd, eps1, result, n_new, tables)
+    with_tables([&](bool tables) { DISPATCH_KEYS(c, CALL); });
 #undef CALL
     *n_out = n_new;
     const int KW = 2 * c->W;

@@ -79,3 +79,43 @@ def test_build_without_room_for_a_bitmap():
     for x, y in zip(want, B.pairs()):
         assert np.array_equal(x, y)
     B.close()
+
+
+@pytest.mark.parametrize("upper", [False, True])
+def test_matrix_without_room_for_the_move_tables(upper):
+    """A matrix asked for is stored where it fits beside the lists, with the tables
+    of single moves or without."""
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 120_000)
+    mode = P.SHCI_STORED_UPPER if upper else P.SHCI_STORED
+    dh, de, dd = G.dev(h), G.dev(eri), G.dev(dets)
+    x = G.dev(S.random_vectors(dets.shape[0], 1, 4))
+    y = [torch.empty_like(x), torch.empty_like(x)]
+
+    def build():
+        ctx = P.Context(0, torch.cuda.current_stream())
+        P.shci_load_integrals(ctx.handle, cfg.n_orb, ec, dh, de)
+        return ctx, P.shci_build_connectivity(ctx.handle, cfg.n_alpha, cfg.n_beta, dd, mode)
+
+    build()[0].close()                            # the library's modules are loaded
+    before = _free()
+    ctx, pairs = build()
+    used = before - _free()
+    stats = P.shci_get_stats(ctx.handle)
+    tables = 16 * (stats["n_alpha_strings"] + stats["n_beta_strings"]) * 300
+    assert tables > 16 * MB
+    P.shci_sigma(ctx.handle, x, y[0])
+    ctx.close()
+    taken = _leave(used - tables // 2)
+    try:
+        ctx, again = build()
+    finally:
+        del taken
+        _free()
+    assert again == pairs
+    P.shci_sigma(ctx.handle, x, y[1])
+    ctx.close()
+    if upper:                                     # atomic sums: 2 m 2^-53 of magnitudes below 1e3, m < 4500
+        assert (y[0] - y[1]).abs().max() < 1e-9
+    else:
+        assert torch.equal(y[0], y[1])
