@@ -1352,6 +1352,7 @@ int shci_batch_create(shci_ctx *ctx, int n_sys, const shci_system_desc *systems,
         for (int s = 0; s < n_sys; s++) {
             shci_ctx *c = b->subs[s];
             if (b->modes[s] != SHCI_ON_THE_FLY) shci::store(c, b->modes[s]);
+            shci::drop_opposite_pass(c);    // the batch's kernel does without
             if (c->mode == SHCI_STORED) b->stats.n_stored++;
             else if (c->mode == SHCI_STORED_UPPER) b->stats.n_stored_upper++;
             else b->stats.n_on_the_fly++;

@@ -618,7 +618,6 @@ static void opposite_pass_setup(shci_ctx *c) {
     cudaStream_t st = c->st;
     c->bs_pair.alloc((size_t)std::max<int64_t>(c->n_beta_singles, 1));
     c->ga_ib.alloc((size_t)c->n_det);
-    c->x_grouped.alloc((size_t)c->n_det);   // a first product of one vector allocates nothing
     k_singles_info<W><<<grid_for(c->Ub * 32), 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->bstr.p, c->bs_pair.p);
     k_member_index<<<grid_for(c->n_det), 256, 0, st>>>(c->ga_det.p, c->n_det, c->ib.p, c->ga_ib.p);
     KERNEL_CHECK();
@@ -754,6 +753,15 @@ static void connectivity_moves(shci_ctx *c, int mode) {
     c->have_moves = true;
 }
 
+// what products on the fly keep: the tables, and room for one vector in the order
+// of the groups, so that a first product allocates nothing (a batch's members
+// take part in its own kernel, which needs neither)
+template <int W>
+static void products_on_the_fly(shci_ctx *c) {
+    connectivity_moves<W>(c, SHCI_ON_THE_FLY);
+    if (c->opp_pass && !c->batch_member) c->x_grouped.alloc((size_t)c->n_det);
+}
+
 // count pass: entries of the beta-grouped part and of the alpha-grouped part
 // of each row, their offsets (rowptr) and the pair counts; with upper set,
 // only the pairs j > i
@@ -814,6 +822,7 @@ static void alloc_matrix(shci_ctx *c, int64_t nnz, DevBuf<int32_t> &col, DevBuf<
 template <int W>
 static void store_w(shci_ctx *c, int mode) {
     const bool upper = mode == SHCI_STORED_UPPER;
+    c->x_grouped.reset();                   // of products on the fly; a gradient takes it again
     if (c->rows_upper != upper) count_w<W>(c, upper);
     c->mode = mode;
     alloc_matrix(c, stored_entries(c), c->col, c->val);
@@ -848,7 +857,7 @@ static void build_w(shci_ctx *c, int mode) {
         c->mode = mode;
         c->col.reset();
         c->val.reset();
-        connectivity_moves<W>(c, mode);
+        products_on_the_fly<W>(c);
     }
     CUDA_TRY(cudaStreamSynchronize(c->st));
 }
@@ -863,6 +872,15 @@ void store(shci_ctx *c, int mode) {
     if (c->W == 1) store_w<1>(c, mode);
     else store_w<2>(c, mode);
     c->built = true;
+}
+
+void drop_opposite_pass(shci_ctx *c) {
+    c->opp_pass = false;
+    c->bs_pair.reset();
+    c->ga_ib.reset();
+    c->item_o_group.reset();
+    c->item_o_first.reset();
+    c->x_grouped.reset();
 }
 
 // the new members of the alpha groups, in the groups' order: flags, then places
@@ -1076,7 +1094,7 @@ static bool extend_w(shci_ctx *c, int64_t n_old) {
         pm.mark(3);
         c->col.reset();
         c->val.reset();
-        connectivity_moves<W>(c, mode);
+        products_on_the_fly<W>(c);
     }
     pm.mark(4);
     c->mode = mode;

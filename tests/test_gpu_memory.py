@@ -119,3 +119,23 @@ def test_matrix_without_room_for_the_move_tables(upper):
         assert (y[0] - y[1]).abs().max() < 1e-9
     else:
         assert torch.equal(y[0], y[1])
+
+
+def test_a_batch_holds_nothing_of_the_opposite_spin_pass(monkeypatch):
+    """Beyond what it holds when every pair of singles is looked up: the lists
+    of the pass (8 bytes per beta single, 12 per determinant) are released."""
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 800_000)
+    dh, de, dd = G.dev(h), G.dev(eri), G.dev(dets)
+    system = {"n_orb": cfg.n_orb, "n_alpha": cfg.n_alpha, "n_beta": cfg.n_beta, "h": dh, "eri": de, "dets": dd}
+    ctx = P.Context(0, torch.cuda.current_stream())
+    used = {}
+    for opp in ("auto", "lookup", "auto"):        # the first loads the library's modules
+        monkeypatch.setenv("SHCI_OPP_SPIN", opp)
+        before = _free()
+        b = P.shci_batch_create(ctx.handle, [system], 0.0)
+        used[opp] = before - _free()
+        P.shci_batch_destroy(b)
+    ctx.close()
+    # allocations below 1 MB share blocks of 2 MB: at most a few blocks more
+    assert used["auto"] <= used["lookup"] + 6 * MB, used
