@@ -225,10 +225,15 @@ __global__ void k_det_keys(const uint64_t *__restrict__ dets, int64_t n, int n_o
         store_key<KW>(keys, i, make_key<W, KW>(load_str<W>(dets, 2 * i), load_str<W>(dets, 2 * i + 1), n_orb));
 }
 
-// the key bits that n_orb orbitals can set
+// The key bits that n_orb orbitals can set.  One-word keys are sorted by them;
+// longer ones have digits that are the same in every key where few orbitals are
+// in use, and a reduction that finds them costs less than a pass (the rule of
+// OrbMask in build.cu; 76 orbitals, selection from 9,001 determinants 3.70 to
+// 3.45 ms, from 100,003 at a tighter threshold 15.55 to 15.37).
 template <int W, int KW>
 struct KeyMask {
     uint64_t w[KW];
+    const uint64_t *known() const { return KW == 1 ? w : nullptr; }
     explicit KeyMask(int n_orb) {
         auto low = [](int bits) { return bits >= 64 ? ~0ull : (bits <= 0 ? 0ull : (1ull << bits) - 1); };
         for (int k = 0; k < KW; k++) w[k] = KW == 1 ? low(2 * n_orb) : low(n_orb - 64 * (k % W));
@@ -244,7 +249,7 @@ static void sorted_space(shci_ctx *c, DevBuf<uint64_t> &vs) {
     k_det_keys<W, KW><<<blocks, SEL_THREADS, 0, c->st>>>(c->dets.p, n, c->n_orb, vs.p);
     KERNEL_CHECK();
     g_kernel_launches += 1;
-    radix_sort<KW>(vs.p, nullptr, n, c->sw, c->st, KeyMask<W, KW>(c->n_orb).w, RS_KEYS);
+    radix_sort<KW>(vs.p, nullptr, n, c->sw, c->st, KeyMask<W, KW>(c->n_orb).known(), RS_KEYS);
 }
 
 // ---------------------------------------------------------------- selection kernels
@@ -763,7 +768,7 @@ static void select_w(shci_ctx *c, int k, const double *cd, double eps1, DevBuf<u
     cand.alloc((size_t)total * KW);
     S.out = cand.p;
     fill_candidates<W, KW, SEL_DETS>(c, S, I);
-    radix_sort<KW>(cand.p, nullptr, total, c->sw, st, KeyMask<W, KW>(c->n_orb).w, RS_KEYS);
+    radix_sort<KW>(cand.p, nullptr, total, c->sw, st, KeyMask<W, KW>(c->n_orb).known(), RS_KEYS);
     DevBuf<uint64_t> vs;
     sorted_space<W, KW>(c, vs);
     const int64_t windows = ceil_div(total, 32);
@@ -1086,7 +1091,7 @@ static void reduce_terms(shci_ctx *c, SelArgs &S, const DevInts &I, int64_t tota
     S.mags = T.mag.p;
     constexpr int FOR = MODE == RUN_PT ? SEL_TERMS : (MODE == RUN_SAMPLE ? SEL_SAMPLE : SEL_MAGS);
     fill_candidates<W, KW, FOR>(c, S, I);
-    radix_sort<KW>(T.cand.p, T.idx.p, total, c->sw, st, KeyMask<W, KW>(c->n_orb).w, RS_POSITION);
+    radix_sort<KW>(T.cand.p, T.idx.p, total, c->sw, st, KeyMask<W, KW>(c->n_orb).known(), RS_POSITION);
     const int blocks = c->n_sm * 8;
     T.part.alloc((size_t)2 * blocks);
     T.npart.alloc((size_t)blocks);
