@@ -101,6 +101,7 @@ __device__ __forceinline__ void red_add(double *p, double v) {
 // instead of 5 NV: FP64 additions are what such a reduction costs.
 template <int NV>
 __device__ __forceinline__ int warp_sum_many(const double (&in)[NV], double &sum) {
+    static_assert(NV <= 32, "a value per lane at most");
     constexpr int P = NV <= 1 ? 1 : (NV <= 2 ? 2 : (NV <= 4 ? 4 : (NV <= 8 ? 8 : (NV <= 16 ? 16 : 32))));
     const int lane = threadIdx.x & 31;
     double v[P];

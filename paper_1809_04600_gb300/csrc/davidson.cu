@@ -472,7 +472,7 @@ static void subspace_guess(shci_ctx *c, int k, double *T) {
     else
         k_guess_block<2><<<16, 256, 0, st>>>(c->dets.p, c->diag.p, c->sort_vals.p, m, SHCI_MAX_SUB, I, w.guess_G.p);
     KERNEL_CHECK();
-    k_jacobi<<<1, 256, JACOBI_SMEM, st>>>(w.guess_G.p, SHCI_MAX_SUB, m, 0, w.guess_val.p, w.guess_vec.p);
+    k_jacobi<<<1, 256, JACOBI_SMEM_SIGNS, st>>>(w.guess_G.p, SHCI_MAX_SUB, m, 0, w.guess_val.p, w.guess_vec.p);
     KERNEL_CHECK();
     CUDA_TRY(cudaMemsetAsync(T, 0, sizeof(double) * k * n, st));
     k_guess_scatter<<<4, 256, 0, st>>>(w.guess_vec.p, SHCI_MAX_SUB, c->sort_vals.p, m, k, n, T);
@@ -682,7 +682,7 @@ int davidson(shci_ctx *c, int k, double tol, int max_iter, const double *guess, 
     const auto t_entry = std::chrono::steady_clock::now();
     static bool jacobi_attr = false;
     if (!jacobi_attr) {
-        CUDA_TRY(cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM));
+        CUDA_TRY(cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM_SIGNS));
         jacobi_attr = true;
     }
     Dav d;
@@ -758,7 +758,7 @@ int davidson(shci_ctx *c, int k, double tol, int max_iter, const double *guess, 
     bool conv = false;
     std::vector<double> theta(k), rnorm(k);
     for (it = 1; it <= max_iter; it++) {
-        k_jacobi<<<1, 256, JACOBI_SMEM, st>>>(w.G.p, d.m_max, m, m_eig, w.eval.p, w.evec.p);
+        k_jacobi<<<1, 256, JACOBI_SMEM_SIGNS, st>>>(w.G.p, d.m_max, m, m_eig, w.eval.p, w.evec.p);
         KERNEL_CHECK();
         g_kernel_launches += 1;
         timer.mark(DP_EIG);

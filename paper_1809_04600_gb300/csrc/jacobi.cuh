@@ -559,6 +559,10 @@ __device__ __forceinline__ bool append_eig(const double *G, int ld, int n, doubl
 // carried out, on the bordered matrix in the old eigenvectors' basis, in FP32
 // and without the rotations too small to matter for a sign (angles below
 // 1e-4): X holds the eigenvectors they lead to, ~1e-5 accurate, by columns.
+// That decides the sign where FP32 tells the eigenvalues apart, which append_eig
+// needs of the poles too (closer ones it refuses), and where no rotation's two
+// diagonal elements are closer than that (it may turn by +45 degrees here and by
+// -45 in FP64).
 // FP32 runs at 75 times the FP64 rate, so this takes a third of the FP64
 // iteration's time.  A, Qf: 64 x 65 floats each in shared memory; X overwrites A.
 __device__ __forceinline__ void jacobi_signs(const double *G, int ld, int m, int mp, const double *eval,
@@ -718,11 +722,14 @@ __device__ __forceinline__ void apply_signs(int ld, int m, double *__restrict__ 
 // Eigen-decomposition of the m x m matrix G whose leading m_prev x m_prev
 // block's is in eval / evec (m_prev = 0: nothing is known): vector by vector
 // when the block only grew, by Jacobi otherwise (the first solve after a
-// restart).  SIGNS: with the signs of the Jacobi iteration (jsm: JACOBI_SMEM
-// bytes); a batch returns energies only and does without.  Per Davidson step
-// of a whole solve: 176 us with Jacobi alone and 88 with this, 52 of it for the
-// signs, for one root (up to 24 vectors), 1.2 ms and 0.30 for the slowest of
-// eight batched systems of four roots (up to 48 vectors, no signs).
+// restart).  SIGNS: with the signs of the Jacobi iteration (jsm: JACOBI_SMEM_SIGNS
+// bytes); where an append is refused, that iteration from the old eigenvectors
+// itself, which are kept until then when several vectors are appended (a first one
+// refused leaves them as they were).  A batch returns energies only and does
+// without.  Per Davidson step of a whole solve: 176 us with Jacobi alone and 88
+// with this, 52 of it for the signs, for one root (up to 24 vectors), 1.2 ms and
+// 0.30 for the slowest of eight batched systems of four roots (up to 48 vectors,
+// no signs).
 template <bool QSHARED, bool SIGNS>
 __device__ __forceinline__ void subspace_eig(const double *G, int ld, int m, int m_prev, double *__restrict__ eval,
                                              double *__restrict__ evec, double *jsm, double *qg = nullptr) {
@@ -734,14 +741,35 @@ __device__ __forceinline__ void subspace_eig(const double *G, int ld, int m, int
     }
     typedef float (*Rows)[SHCI_MAX_SUB + 1];
     Rows X = reinterpret_cast<Rows>(jsm + SHCI_MAX_SUB * (SHCI_MAX_SUB + 1));     // behind append_eig's matrix
+    const bool keep = SIGNS && m - old > 1;
+    double *kept = jsm + 2 * SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);       // behind jacobi_solve's two matrices
+    if (keep) {
+        for (int e = threadIdx.x; e < old * (old + 1); e += blockDim.x) {
+            const int l = e / (old + 1), r = e - l * (old + 1);
+            kept[e] = r < old ? __ldcg(&evec[l * ld + r]) : __ldcg(&eval[l]);
+        }
+    }
     if (SIGNS) jacobi_signs(G, ld, m, old, eval, evec, X, reinterpret_cast<Rows>(jsm));
     while (have < m && append_eig(G, ld, have, eval, evec, jsm)) have++;
-    if (have < m) jacobi_solve<QSHARED>(G, ld, m, have, eval, evec, jsm, qg);
-    else if (SIGNS) apply_signs(ld, m, evec, X);
+    if (have == m) {
+        if (SIGNS) apply_signs(ld, m, evec, X);
+        return;
+    }
+    if (keep && have > old) {
+        for (int e = threadIdx.x; e < old * (old + 1); e += blockDim.x) {
+            const int l = e / (old + 1), r = e - l * (old + 1);
+            if (r < old) evec[l * ld + r] = kept[e];
+            else eval[l] = kept[e];
+        }
+        have = old;
+        __syncthreads();
+    }
+    jacobi_solve<QSHARED>(G, ld, m, have, eval, evec, jsm, qg);
 }
 
 constexpr size_t JACOBI_SMEM_A = sizeof(double) * SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);
 constexpr size_t JACOBI_SMEM = 2 * JACOBI_SMEM_A;
+constexpr size_t JACOBI_SMEM_SIGNS = JACOBI_SMEM + sizeof(double) * SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);
 constexpr int JACOBI_Q_DOUBLES = SHCI_MAX_SUB * (SHCI_MAX_SUB + 1);
 
 }  // namespace shci
