@@ -57,6 +57,14 @@ void load_integrals(shci_ctx *c, int n_orb, double e_core, const double *h, cons
         for (int q = 0; q < p; q++)
             if (!(std::abs(hh[p * n_orb + q] - hh[q * n_orb + p]) <= 1e-12))
                 throw ShciError{SHCI_ERR_INVALID, "h is not symmetric"};
+    // what the single-move tables, one entry per pair of orbitals, leave out of it
+    std::vector<double> skew(hh.size(), 0.0);
+    bool any_skew = false;
+    for (int p = 0; p < n_orb; p++)
+        for (int q = p + 1; q < n_orb; q++) {
+            skew[p * n_orb + q] = hh[p * n_orb + q] - hh[q * n_orb + p];
+            any_skew = any_skew || skew[p * n_orb + q] != 0.0;
+        }
     c->built = false;
     c->h.alloc(hh.size());
     c->eri.alloc((size_t)neri);
@@ -64,6 +72,11 @@ void load_integrals(shci_ctx *c, int n_orb, double e_core, const double *h, cons
     c->j1.alloc((size_t)n_orb * n_orb * n_orb);
     c->jdiag.alloc((size_t)n_orb * n_orb);
     c->jkdiag.alloc((size_t)n_orb * n_orb);
+    if (any_skew) {
+        c->hskew.alloc(skew.size());
+        CUDA_TRY(cudaMemcpyAsync(c->hskew.p, skew.data(), sizeof(double) * skew.size(), cudaMemcpyHostToDevice, c->st));
+    }
+    c->have_skew = any_skew;
     CUDA_TRY(cudaMemcpyAsync(c->h.p, hh.data(), sizeof(double) * hh.size(), cudaMemcpyHostToDevice, c->st));
     CUDA_TRY(cudaMemcpyAsync(c->eri.p, eri, sizeof(double) * neri, kind, c->st));
     int64_t total = (int64_t)n_orb * n_orb * n_orb;
@@ -87,6 +100,7 @@ DevInts dev_ints(const shci_ctx *c) {
     I.j1 = c->j1.p;
     I.jdiag = c->jdiag.p;
     I.jkdiag = c->jkdiag.p;
+    I.hskew = c->have_skew ? c->hskew.p : nullptr;
     I.e_core = c->e_core;
     I.n = c->n_orb;
     return I;

@@ -569,7 +569,9 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
                         set_bit(m, r + (spin ? beta : 0));
                         if (own) {
                             const int pr = pair_idx(p, r);
-                            v = flip_sign(__ldg(&own[pr]) + __ldg(&other[pr]), p < r);
+                            v = __ldg(&own[pr]) + __ldg(&other[pr]);
+                            if (I.hskew) v += __ldg(&I.hskew[p * n + r]);
+                            v = flip_sign(v, p < r);
                         } else {
                             const Str<W> &si = spin ? B : A;
                             Str<W> sj = si;
