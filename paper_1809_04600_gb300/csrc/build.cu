@@ -57,14 +57,15 @@ void load_integrals(shci_ctx *c, int n_orb, double e_core, const double *h, cons
         for (int q = 0; q < p; q++)
             if (!(std::abs(hh[p * n_orb + q] - hh[q * n_orb + p]) <= 1e-12))
                 throw ShciError{SHCI_ERR_INVALID, "h is not symmetric"};
-    // what the single-move tables, one entry per pair of orbitals, leave out of it
-    std::vector<double> skew(hh.size(), 0.0);
-    bool any_skew = false;
+    // The single-move tables hold one entry per pair of orbitals.  Where h_pq and h_qp
+    // differ by more than the rounding of a term they are not used.
+    double top = 0.0, skew = 0.0;
     for (int p = 0; p < n_orb; p++)
-        for (int q = p + 1; q < n_orb; q++) {
-            skew[p * n_orb + q] = hh[p * n_orb + q] - hh[q * n_orb + p];
-            any_skew = any_skew || skew[p * n_orb + q] != 0.0;
+        for (int q = 0; q <= p; q++) {
+            top = std::max(top, std::abs(hh[p * n_orb + q]));
+            skew = std::max(skew, std::abs(hh[p * n_orb + q] - hh[q * n_orb + p]));
         }
+    c->h_even = skew <= 0x1p-51 * top;
     c->built = false;
     c->h.alloc(hh.size());
     c->eri.alloc((size_t)neri);
@@ -72,11 +73,6 @@ void load_integrals(shci_ctx *c, int n_orb, double e_core, const double *h, cons
     c->j1.alloc((size_t)n_orb * n_orb * n_orb);
     c->jdiag.alloc((size_t)n_orb * n_orb);
     c->jkdiag.alloc((size_t)n_orb * n_orb);
-    if (any_skew) {
-        c->hskew.alloc(skew.size());
-        CUDA_TRY(cudaMemcpyAsync(c->hskew.p, skew.data(), sizeof(double) * skew.size(), cudaMemcpyHostToDevice, c->st));
-    }
-    c->have_skew = any_skew;
     CUDA_TRY(cudaMemcpyAsync(c->h.p, hh.data(), sizeof(double) * hh.size(), cudaMemcpyHostToDevice, c->st));
     CUDA_TRY(cudaMemcpyAsync(c->eri.p, eri, sizeof(double) * neri, kind, c->st));
     int64_t total = (int64_t)n_orb * n_orb * n_orb;
@@ -100,7 +96,6 @@ DevInts dev_ints(const shci_ctx *c) {
     I.j1 = c->j1.p;
     I.jdiag = c->jdiag.p;
     I.jkdiag = c->jkdiag.p;
-    I.hskew = c->have_skew ? c->hskew.p : nullptr;
     I.e_core = c->e_core;
     I.n = c->n_orb;
     return I;
@@ -751,7 +746,7 @@ static void connectivity_moves(shci_ctx *c, int mode) {
     c->have_moves = false;
     const double entries = (double)(c->Ua + c->Ub) * c->n_orb * (c->n_orb + 1) / 2;
     const double per_row = mode == SHCI_ON_THE_FLY && !c->batch_member ? 128.0 : 24.0;
-    bool fits = entries <= per_row * (double)c->n_det;
+    bool fits = c->h_even && entries <= per_row * (double)c->n_det;
     if (fits && entries * 16.0 > 6.4e7) {
         size_t fr = 0, tot = 0;
         CUDA_TRY(cudaMemGetInfo(&fr, &tot));

@@ -200,7 +200,6 @@ struct DevInts {
     const double *j1;       // [n*n][n]: (pq|kk)             (opposite-spin mean field)
     const double *jdiag;    // [n][n]:   (kk|ll)
     const double *jkdiag;   // [n][n]:   (kk|ll) - (kl|lk)
-    const double *hskew;    // [n][n]:   h_pq - h_qp above the diagonal, 0 elsewhere; null when h is exactly symmetric
     double e_core;
     int n;
 };

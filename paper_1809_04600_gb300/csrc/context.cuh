@@ -50,8 +50,7 @@ struct shci_ctx {
     int n_orb = 0;
     double e_core = 0.0;
     DevBuf<double> h, eri, jk1, j1, jdiag, jkdiag;
-    DevBuf<double> hskew;                  // empty when h is exactly symmetric
-    bool have_skew = false;
+    bool h_even = true;                    // h_pq and h_qp differ by rounding at most
     // heat-bath lists for the selection (built on first use per set of integrals)
     bool hb_valid = false;
     HBList hb_same, hb_opp;

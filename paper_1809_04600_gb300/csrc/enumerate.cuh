@@ -224,20 +224,6 @@ __device__ __forceinline__ void move_info(const Str<W> &si, const Str<W> &sj, in
     neg = bits_between<W>(sj, p < q ? p : q, p < q ? q : p);
 }
 
-// what h adds to a tabulated move (particle in si, hole in sj) when it is symmetric
-// to rounding only: the table holds h_pq of p > q
-template <int W>
-__device__ __forceinline__ double skew_of(const DevInts &I, const Str<W> &si, const Str<W> &sj) {
-    Str<W> pi, qj;
-#pragma unroll
-    for (int k = 0; k < W; k++) {
-        const uint64_t d = si.w[k] ^ sj.w[k];
-        pi.w[k] = si.w[k] & d;
-        qj.w[k] = sj.w[k] & d;
-    }
-    return __ldg(&I.hskew[lowest_bit<W>(pi) * I.n + lowest_bit<W>(qj)]);
-}
-
 __device__ __forceinline__ double eri_pairs(const DevInts &I, int pq, int rs) {
     int hi = pq > rs ? pq : rs, lo = pq > rs ? rs : pq;
     return __ldg(&I.eri[(int64_t)hi * (hi + 1) / 2 + lo]);
@@ -256,9 +242,7 @@ __device__ __forceinline__ double eval_pair(const DevInts &I, const Str<W> &si, 
     if (!(ctx & 1) && own && xor_popc<W>(si, sj) == 2) {
         int pq, neg;
         move_info<W>(si, sj, pq, neg);
-        double v = __ldg(&own[pq]) + __ldg(&oth[pq]);
-        if (I.hskew) v += skew_of<W>(I, si, sj);
-        return flip_sign(v, neg);
+        return flip_sign(__ldg(&own[pq]) + __ldg(&oth[pq]), neg);
     }
     if (ctx & 1) {
         int pq_b, neg_b;

@@ -300,7 +300,7 @@ static void tabulate_moves(shci_ctx *c, SelArgs &S, const DevInts &I, double row
         S.ib = c->ib.p;
         return;
     }
-    if (!own) return;
+    if (!own || !c->h_even) return;
     const int64_t np = (int64_t)n * (n + 1) / 2;
     const double entries = (double)(c->Ua + c->Ub) * np;
     const double moves = rows * ((double)S.na * (n - S.na) + (double)S.nb * (n - S.nb));
@@ -569,9 +569,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(SelArgs S, DevInts I) {
                         set_bit(m, r + (spin ? beta : 0));
                         if (own) {
                             const int pr = pair_idx(p, r);
-                            v = __ldg(&own[pr]) + __ldg(&other[pr]);
-                            if (I.hskew) v += __ldg(&I.hskew[p * n + r]);
-                            v = flip_sign(v, p < r);
+                            v = flip_sign(__ldg(&own[pr]) + __ldg(&other[pr]), p < r);
                         } else {
                             const Str<W> &si = spin ? B : A;
                             Str<W> sj = si;

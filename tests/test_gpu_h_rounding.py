@@ -1,6 +1,6 @@
 """h symmetric to rounding only (the library takes up to 1e-12): an element H_ij
-carries h_pq of the particle p in D_i and the hole q in D_j, whether its single
-moves are tabulated or not.
+carries h_pq of the particle p in D_i and the hole q in D_j, whether V is large
+enough to tabulate its single moves or not.
 
 An element is a sum of at most 12 terms below 8: within 12 x 2^-53 x 96 = 1.3e-13
 of its value; h_pq and h_qp differ by 9e-13 here."""
@@ -22,7 +22,7 @@ def _integrals(n):
 
 
 @pytest.mark.parametrize("mode", ["SHCI_STORED", "SHCI_STORED_UPPER"])
-@pytest.mark.parametrize("step", [1, 40])                 # tables for 3,136 determinants, none for 79
+@pytest.mark.parametrize("step", [1, 40])                 # 3,136 determinants, enough for tables, and 79
 def test_stored_elements(mode, step):
     P = G.lib()
     h, eri, ec = _integrals(8)
