@@ -124,7 +124,6 @@ __device__ __forceinline__ int warp_sum_many(const double (&in)[NV], double &sum
     return own;
 }
 
-__device__ __forceinline__ int popc2(uint64_t a, uint64_t b) { return __popcll(a ^ b); }
 
 template <int W>
 struct Str {

@@ -30,7 +30,6 @@ struct HBList {
     DevBuf<uint32_t> rs;
     DevBuf<double> val;
     DevBuf<float> kf;
-    int64_t entries = 0;
 };
 
 namespace shci {

@@ -14,7 +14,8 @@
 //     and screened by each warp with XOR + popcount + ballot.
 //   k_enum_beta: rows grouped by beta string b; candidates share b
 //     (same-spin alpha excitations), staged the same way.
-// Row i's entries are laid out [beta-grouped part | alpha-grouped part].
+// Row i's entries are laid out [beta-grouped part | alpha-grouped part |
+// opposite-spin part]; the last is empty where k_enum_alpha takes those pairs too.
 //
 // Only a few percent of the screened candidates are connected, so matches are
 // not evaluated where they are found: each warp appends them to a queue in

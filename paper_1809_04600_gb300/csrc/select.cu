@@ -116,7 +116,6 @@ static void build_hb_list(shci_ctx *c, int same, HBList &L) {
         KERNEL_CHECK();
         g_kernel_launches += 1;
     }
-    L.entries = n_valid;
     CUDA_TRY(cudaStreamSynchronize(st));
 }
 
@@ -1204,7 +1203,7 @@ __global__ void k_sum_in_order(const double *__restrict__ part, int m, double *_
 // energy of that space went from 61.5 ms with the last form to 50.7 with this.
 static void alias_table(const double *c, int64_t n, double sum, double *prob, uint32_t *alias) {
     const double scale = (double)n / sum;
-    std::vector<uint32_t> stack((size_t)n);              // small columns from the front, large ones from the back
+    std::vector<uint32_t> stack((size_t)n);              // the small columns
     int64_t ns = 0, nl = 0;
     for (int64_t i = 0; i < n; i++) {
         prob[i] = std::fabs(c[i]) * scale;
