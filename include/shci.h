@@ -386,7 +386,8 @@ typedef struct {
 
 /* Build every system's connectivity (Sec. III) and decide how each H is held
  * within stored_budget_bytes of device memory (< 0: no budget beyond 80 % of
- * the free memory), 12 bytes per stored nonzero: when the upper triangles of
+ * the free memory, which includes what the build held and the batch does not
+ * read), 12 bytes per stored nonzero: when the upper triangles of
  * all systems fit, every system is stored, as both triangles for the systems
  * taken in ascending order of pair count while the budget allows and as its
  * upper triangle for the rest; otherwise upper triangles are stored in that

@@ -1340,19 +1340,26 @@ int shci_batch_create(shci_ctx *ctx, int n_sys, const shci_system_desc *systems,
             b->stats.total_det += c->n_det;
             b->stats.total_nnz_upper += c->nnz_upper;
         }
-        // the storage plan (plan.h) within the budget and 80 % of the free memory
+        // the storage plan (plan.h) within the budget and 80 % of the memory that is
+        // free, or will be once the members drop what the batch does not read (on-the-fly
+        // members keep their bitmap and tables: those count where all are stored)
         size_t free_b = 0, total_b = 0;
         CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-        double left = 0.8 * (double)free_b;
-        if (stored_budget_bytes >= 0.0) left = std::min(left, stored_budget_bytes);
         std::vector<int64_t> pairs;
         for (auto *c : b->subs) pairs.push_back(c->nnz_upper);
-        b->modes = shci::storage_plan(pairs, left);
+        for (bool stored : {true, false}) {
+            double back = 0.0;
+            for (auto *c : b->subs) back += shci::batch_unread(c, stored);
+            double left = std::min(0.8 * ((double)free_b + back), (double)free_b);
+            if (stored_budget_bytes >= 0.0) left = std::min(left, stored_budget_bytes);
+            b->modes = shci::storage_plan(pairs, left);
+            if (std::find(b->modes.begin(), b->modes.end(), (int)SHCI_ON_THE_FLY) == b->modes.end()) break;
+        }
         // pass 2: store, and describe each system to the kernel
         for (int s = 0; s < n_sys; s++) {
             shci_ctx *c = b->subs[s];
             if (b->modes[s] != SHCI_ON_THE_FLY) shci::store(c, b->modes[s]);
-            shci::drop_opposite_pass(c);    // the batch's kernel does without
+            shci::drop_batch_unread(c);
             if (c->mode == SHCI_STORED) b->stats.n_stored++;
             else if (c->mode == SHCI_STORED_UPPER) b->stats.n_stored_upper++;
             else b->stats.n_on_the_fly++;

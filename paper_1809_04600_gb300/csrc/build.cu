@@ -883,13 +883,26 @@ void store(shci_ctx *c, int mode) {
     c->built = true;
 }
 
-void drop_opposite_pass(shci_ctx *c) {
+double batch_unread(const shci_ctx *c, bool stored) {
+    double bytes = 8.0 * (c->bs_pair.n + c->x_grouped.n) + 4.0 * (c->ga_ib.n + c->item_o_group.n + c->item_o_first.n);
+    if (stored) bytes += 16.0 * c->occ.n + 8.0 * (c->move_a.n + c->move_b.n);
+    return bytes;
+}
+
+void drop_batch_unread(shci_ctx *c) {
     c->opp_pass = false;
     c->bs_pair.reset();
     c->ga_ib.reset();
     c->item_o_group.reset();
     c->item_o_first.reset();
     c->x_grouped.reset();
+    if (c->mode == SHCI_ON_THE_FLY) return;
+    c->opp_lookup = false;
+    c->opp_hybrid = false;
+    c->occ.reset();
+    c->have_moves = false;
+    c->move_a.reset();
+    c->move_b.reset();
 }
 
 // the new members of the alpha groups, in the groups' order: flags, then places

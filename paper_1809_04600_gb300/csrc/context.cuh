@@ -140,9 +140,11 @@ void extend(shci_ctx *c, int64_t n_new, const uint64_t *new_dets, int mem, doubl
 // store a context built in any mode as SHCI_STORED or SHCI_STORED_UPPER
 // (the lists are kept; the rows are recounted when their form differs)
 void store(shci_ctx *c, int mode);
-// release what only the opposite-spin pass reads; products, gradients and growth
-// then take the general path
-void drop_opposite_pass(shci_ctx *c);
+// Release what a batch's kernel does not read of a member: the lists of the
+// opposite-spin pass and, of a stored one, the occupancy bitmap and the tables of
+// single moves.  batch_unread: their bytes (stored: the member is or will be).
+void drop_batch_unread(shci_ctx *c);
+double batch_unread(const shci_ctx *c, bool stored);
 void export_pairs(shci_ctx *c, int64_t cap, int64_t *i_out, int64_t *j_out, double *v_out, int64_t *n_out);
 
 // sigma.cu: y = H x for k vectors; `inter` selects the interleaved [n][k]

@@ -139,3 +139,44 @@ def test_a_batch_holds_nothing_of_the_opposite_spin_pass(monkeypatch):
     ctx.close()
     # allocations below 1 MB share blocks of 2 MB: at most a few blocks more
     assert used["auto"] <= used["lookup"] + 6 * MB, used
+
+
+def test_a_stored_batch_neither_holds_nor_counts_what_it_does_not_read():
+    """The bitmap and the tables of single moves serve a member's build: a batch that
+    stores H releases them, and plans its storage with their memory."""
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 400_000)
+    n = dets.shape[0]
+    dh, de, dd = G.dev(h), G.dev(eri), G.dev(dets)
+    system = {"n_orb": cfg.n_orb, "n_alpha": cfg.n_alpha, "n_beta": cfg.n_beta, "h": dh, "eri": de, "dets": dd}
+    ctx = P.Context(0, torch.cuda.current_stream())
+    P.shci_load_integrals(ctx.handle, cfg.n_orb, ec, dh, de)
+    pairs = P.shci_build_connectivity(ctx.handle, cfg.n_alpha, cfg.n_beta, dd, P.SHCI_ON_THE_FLY)
+    stats = P.shci_get_stats(ctx.handle)
+    ctx.close()
+    ua, ub = stats["n_alpha_strings"], stats["n_beta_strings"]
+    tables, matrix = 16 * (ua + ub) * 300, 24 * pairs
+    assert 300 * (ua + ub) <= 24 * n and tables > 32 * MB      # a batch's member takes them
+    ctx = P.Context(0, torch.cuda.current_stream())
+    used, modes = {}, {}
+    for budget in (0.0, -1.0, 0.0, -1.0):                       # the first two load the library's modules
+        before = _free()
+        b = P.shci_batch_create(ctx.handle, [system], budget)
+        used[budget] = before - _free()
+        modes[budget] = int(P.shci_batch_get_modes(b, 1)[0])
+        P.shci_batch_destroy(b)
+    assert modes == {0.0: P.SHCI_ON_THE_FLY, -1.0: P.SHCI_STORED}
+    # blocks of 2 MB: at most a few more
+    assert used[-1.0] <= used[0.0] + matrix - tables + 8 * MB, (used, matrix, tables)
+    # 80 % of the free memory is short of both triangles by 0.4 of the tables, and
+    # beyond them by as much with the tables released
+    taken = _leave(used[0.0] + matrix / 0.8 - tables // 2)
+    try:
+        b = P.shci_batch_create(ctx.handle, [system])
+        mode = int(P.shci_batch_get_modes(b, 1)[0])
+        P.shci_batch_destroy(b)
+    finally:
+        del taken
+        _free()
+    ctx.close()
+    assert mode == P.SHCI_STORED
