@@ -673,11 +673,13 @@ static void opposite_spin_setup(shci_ctx *c) {
 // SHCI_AUTO: store both triangles of H when their nnz_full elements (12 bytes
 // each) fit 80 % of the free device memory and the context's budget, else the
 // upper triangle alone when its nnz_full / 2 elements fit, else apply H on the fly.
-// held: bytes taken now that are given back before the call returns
+// held: bytes taken now that are given back before the call returns.  So are the
+// single-move tables of an earlier form or space (alloc_matrix).
 static int decide_mode(shci_ctx *c, int mode, int64_t nnz_full, double held = 0.0) {
     if (mode != SHCI_AUTO) return mode;
     size_t free_b = 0, total_b = 0;
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+    held += 8.0 * (c->move_a.n + c->move_b.n);
     double need = (double)nnz_full * 12.0;
     double cap = std::min(0.8 * ((double)free_b + held), (double)free_b);
     if (c->stored_budget >= 0.0) cap = std::min(cap, c->stored_budget);

@@ -180,3 +180,33 @@ def test_a_stored_batch_neither_holds_nor_counts_what_it_does_not_read():
         _free()
     ctx.close()
     assert mode == P.SHCI_STORED
+
+
+def test_the_choice_of_form_does_not_count_tables_of_an_earlier_build():
+    """SHCI_AUTO after a build on the fly: its tables of single moves make way for H."""
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 400_000)
+    dh, de, dd = G.dev(h), G.dev(eri), G.dev(dets)
+
+    def build(ctx, mode):
+        return P.shci_build_connectivity(ctx.handle, cfg.n_alpha, cfg.n_beta, dd, mode)
+
+    modes = []
+    for short in (0.0, 1.0):                                    # the first loads the library's modules
+        ctx = P.Context(0, torch.cuda.current_stream())
+        P.shci_load_integrals(ctx.handle, cfg.n_orb, ec, dh, de)
+        pairs = build(ctx, P.SHCI_ON_THE_FLY)
+        stats = P.shci_get_stats(ctx.handle)
+        tables = 16 * (stats["n_alpha_strings"] + stats["n_beta_strings"]) * 300
+        assert tables > 32 * MB
+        # 80 % of the free memory is short of the upper triangle by 0.4 of the tables,
+        # and beyond it by as much without them
+        taken = _leave(12 * pairs / 0.8 - short * tables // 2) if short else None
+        try:
+            build(ctx, P.SHCI_AUTO)
+            modes.append(P.shci_get_stats(ctx.handle)["mode"])
+        finally:
+            del taken
+            _free()
+        ctx.close()
+    assert modes == [P.SHCI_STORED, P.SHCI_STORED_UPPER]
