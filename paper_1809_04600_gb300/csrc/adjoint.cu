@@ -80,8 +80,9 @@ static void backward_w(shci_ctx *c, const double *cv, double *gdh, double *geri,
     A.geri = geri;
     A.geri_len = eri_len;
     DevInts I = dev_ints(c);
-    launch_enum<W, ENUM_GRAD, 1>(c, A, I, true);
-    if (c->opp_pass) {
+    const bool pass = takes_opposite_pass(c, 1);
+    launch_enum<W, ENUM_GRAD, 1>(c, A, I, true, !pass);
+    if (pass) {
         group_vectors(c, A, 1);
         launch_opposite<W, ENUM_GRAD, 1>(c, A, I);
     }

@@ -71,6 +71,13 @@ static __global__ void k_group_vectors(const int32_t *__restrict__ mdet, int64_t
         out[e] = __ldg(&x[(int64_t)mdet[e / k] * k + e % k]);
 }
 
+// Does a product or gradient of k vectors take the opposite-spin pass?  Where the
+// memory for its grouped vectors is not there, the alpha-grouped kernel finds those
+// pairs instead, by the choice per alpha single.
+inline bool takes_opposite_pass(shci_ctx *c, int k) {
+    return c->opp_pass && try_alloc(c->x_grouped, (size_t)c->n_det * k);
+}
+
 // A.x in the order of the alpha groups' members, for the opposite-spin pass on
 // the fly: a pair's place is then where its coefficient is.
 inline void group_vectors(shci_ctx *c, EnumArgs &A, int k) {

@@ -249,8 +249,9 @@ static void otf_k(shci_ctx *c, const double *x, double *y) {
     A.diag = c->diag.p;
     DevInts I = dev_ints(c);
     A.accumulate = 0;
-    launch_enum<W, ENUM_SIGMA, K>(c, A, I, true);
-    if (c->opp_pass) {
+    const bool pass = takes_opposite_pass(c, K);
+    launch_enum<W, ENUM_SIGMA, K>(c, A, I, true, !pass);
+    if (pass) {
         group_vectors(c, A, K);
         launch_opposite<W, ENUM_SIGMA, K>(c, A, I);
     }

@@ -210,3 +210,45 @@ def test_the_choice_of_form_does_not_count_tables_of_an_earlier_build():
             _free()
         ctx.close()
     assert modes == [P.SHCI_STORED, P.SHCI_STORED_UPPER]
+
+
+def test_products_without_room_for_their_grouped_vectors():
+    """Eight vectors on the fly with room for the two layouts of the vectors and no third."""
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 400_000)
+    n, k = dets.shape[0], 8
+    x = G.dev(S.random_vectors(n, k, 4))
+    want, got = torch.empty_like(x), torch.empty_like(x)
+    F = G.Built(P, h, eri, ec, dets, cfg.n_alpha, cfg.n_beta, mode=P.SHCI_ON_THE_FLY)
+    P.shci_sigma(F.ctx.handle, x, want)
+    B = G.Built(P, h, eri, ec, dets, cfg.n_alpha, cfg.n_beta, mode=P.SHCI_ON_THE_FLY)
+    taken = _leave(2.5 * 8 * k * n)
+    try:
+        P.shci_sigma(B.ctx.handle, x, got)
+    finally:
+        del taken
+        _free()
+    # the same m <= 16470 terms in another order: 2 m 2^-53 of sums of magnitudes below 1e3
+    assert (want - got).abs().max() < 4e-9
+    F.close()
+    B.close()
+
+
+def test_gradient_without_room_for_its_grouped_vector():
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 1_000_000)
+    c = G.dev(S.random_vectors(dets.shape[0], 1, 4))[0]
+    B = G.Built(P, h, eri, ec, dets, cfg.n_alpha, cfg.n_beta, mode=P.SHCI_STORED_UPPER)
+    out = [[torch.empty((24, 24), dtype=torch.float64, device="cuda"),
+            torch.empty(eri.size, dtype=torch.float64, device="cuda")] for _ in range(2)]
+    # 32 copies of the gradient, 12 and 2 MB, and not 8 MB more
+    taken = _leave(19 * MB)
+    try:
+        P.shci_energy_backward(B.ctx.handle, c, 1.0, *out[0])
+    finally:
+        del taken
+        _free()
+    P.shci_energy_backward(B.ctx.handle, c, 1.0, *out[1])
+    for a, b in zip(*out):
+        assert (a - b).abs().max() <= 1e-7 * b.abs().max()
+    B.close()
