@@ -621,12 +621,17 @@ __global__ void k_singles_info(const int64_t *__restrict__ off, const int32_t *_
     }
 }
 
-// what the opposite-spin pass needs beside the bitmap
+// what the opposite-spin pass needs beside the bitmap; there is no pass without
+// the memory for it (the choice per alpha single needs the bitmap alone)
 template <int W>
 static void opposite_pass_setup(shci_ctx *c) {
     cudaStream_t st = c->st;
-    c->bs_pair.alloc((size_t)std::max<int64_t>(c->n_beta_singles, 1));
-    c->ga_ib.alloc((size_t)c->n_det);
+    if (!try_alloc(c->bs_pair, (size_t)std::max<int64_t>(c->n_beta_singles, 1)) ||
+        !try_alloc(c->ga_ib, (size_t)c->n_det)) {
+        c->bs_pair.reset();
+        c->ga_ib.reset();
+        return;
+    }
     k_singles_info<W><<<grid_for(c->Ub * 32), 256, 0, st>>>(c->bs_off.p, c->bs_idx.p, c->Ub, c->bstr.p, c->bs_pair.p);
     k_member_index<<<grid_for(c->n_det), 256, 0, st>>>(c->ga_det.p, c->n_det, c->ib.p, c->ga_ib.p);
     KERNEL_CHECK();
@@ -770,7 +775,7 @@ static void connectivity_moves(shci_ctx *c, int mode) {
 template <int W>
 static void products_on_the_fly(shci_ctx *c) {
     connectivity_moves<W>(c, SHCI_ON_THE_FLY);
-    if (c->opp_pass && !c->batch_member) c->x_grouped.alloc((size_t)c->n_det);
+    if (c->opp_pass && !c->batch_member) try_alloc(c->x_grouped, (size_t)c->n_det);
 }
 
 // count pass: entries of the beta-grouped part and of the alpha-grouped part

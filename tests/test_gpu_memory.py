@@ -252,3 +252,29 @@ def test_gradient_without_room_for_its_grouped_vector():
     for a, b in zip(*out):
         assert (a - b).abs().max() <= 1e-7 * b.abs().max()
     B.close()
+
+
+def test_build_without_room_for_the_lists_of_the_pass(monkeypatch):
+    P = G.lib()
+    cfg, h, eri, ec, dets = G.system("sel_24o_6a6b_1m", 1_000_000)
+    x = G.dev(S.random_vectors(dets.shape[0], 1, 4))
+    dd = G.dev(dets)
+    y = [torch.empty_like(x), torch.empty_like(x)]
+    F = G.Built(P, h, eri, ec, dets, cfg.n_alpha, cfg.n_beta, mode=P.SHCI_ON_THE_FLY)
+    P.shci_sigma(F.ctx.handle, x, y[0])
+    monkeypatch.setenv("SHCI_OPP_SPIN", "lookup")               # everything but the pass's lists
+    B = G.Built(P, h, eri, ec, dets, cfg.n_alpha, cfg.n_beta, mode=P.SHCI_ON_THE_FLY)
+    P.shci_sigma(B.ctx.handle, x, y[1])
+    monkeypatch.delenv("SHCI_OPP_SPIN")
+    taken = _leave(5 * MB)                                      # 4 MB for the members' indices, more for the singles
+    try:
+        pairs = P.shci_build_connectivity(B.ctx.handle, cfg.n_alpha, cfg.n_beta, dd, P.SHCI_ON_THE_FLY)
+        P.shci_sigma(B.ctx.handle, x, y[1])
+    finally:
+        del taken
+        _free()
+    assert pairs == F.nnz
+    # the same m <= 16470 terms in another order: 2 m 2^-53 of sums of magnitudes below 1e3
+    assert (y[0] - y[1]).abs().max() < 4e-9
+    F.close()
+    B.close()
