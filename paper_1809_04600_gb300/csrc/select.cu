@@ -845,8 +845,8 @@ __device__ __forceinline__ void run_terms(const RunArgs &A, int64_t e, double *v
 // and finished 32 at a time (is a in V, H_aa, the contribution).  A thread per
 // run, adding up its terms one by one, took 27 ms for 1.8e8 terms and 18 ms
 // for a sample of 5e7, nearly all of it the longest runs' chains of dependent
-// loads; this form 4.8 and 5.5, with the FP64 pipe 78 % busy (the tree's
-// additions, H_aa, the division).  The order of every sum is fixed.
+// loads; this form 4.8 and 5.5, with the FP64 pipe 66 and 81 % busy (the tree's
+// additions, H_aa, the division) and HBM 52 and 33 %.  The order of every sum is fixed.
 constexpr int RUN_CHUNK = 16;
 
 template <int W, int KW, int MODE>

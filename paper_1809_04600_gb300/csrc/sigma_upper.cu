@@ -14,7 +14,7 @@ constexpr int UPPER_THREADS = 256;
 // H_ij x_j to its row sum and scatters H_ij x_i into y_j with an atomic add,
 // and the row sums are added to y_i atomically too (other rows scatter into
 // it concurrently).  Summation order varies from run to run.  The FP64 atomics
-// bound it (four vectors on the 1e6 heat-bath space: 0.81 of the measured
+// bound it (four vectors on the 1e6 heat-bath space: 0.83 of the measured
 // atomic rate); the shapes tried (rows per group / nonzeros per lane per step
 // / CTAs per SM: 4/4/3, 4/2/4, 2/4/4, 4/4/2) were within 3 % of one another.
 // FEW: a row per warp and four nonzeros per lane and step, for spaces whose
